@@ -81,13 +81,13 @@ typedef struct pndf_query {
 /* Optional per-query counters (40 bytes), written when stats_dev != NULL. */
 typedef struct pndf_query_stats {
     uint32_t nodes;        /* hierarchy nodes tested                                 */
-    uint32_t leaf_blocks;  /* leaf blocks whose triangles were tested                */
-    uint32_t tri_tests;    /* triangles tested against m                             */
+    uint32_t leaf_blocks;  /* leaf blocks reached                                     */
+    uint32_t tri_tests;    /* triangles decided one by one (past the group filter)    */
     uint32_t hits;         /* contributing hits (m inside, q <= 16)                  */
     uint32_t hit_hash;     /* sum mod 2^32 of MurmurHash3-fmix32(triangle id) over hits */
     uint32_t fp64_tris;    /* triangles evaluated in FP64 (normal area < 1e-10)      */
     uint32_t degenerate;   /* zero-area normal triangles met inside their bbox       */
-    uint32_t quads;        /* per-quad (level 0) boxes tested                        */
+    uint32_t quads;        /* quads whose edge functions were tested, in 2 x 2 groups */
     uint32_t cluster_checks; /* nodes whose cluster residual was compared with the cut */
     uint32_t clusters;     /* cluster nodes whose two triangles were tested          */
 } pndf_query_stats;
@@ -155,12 +155,11 @@ typedef struct pndf_eval_config {
  * A node at level l covers 2^l x 2^l quads; it stores the bounding box of the
  * normals of all texels of its quads, so the normal triangles of every quad
  * below it lie inside.  Levels leaf_level..L are stored (2^L >= N-1), each
- * in Morton order so the four children of a node are contiguous, plus level
- * 0 (one box per quad, Morton order, so a leaf block's 16 quads are
- * contiguous) and beside it one capsule per quad (8 bytes: the segment
- * between the quad's two farthest normals and a radius holding all four, a
- * tighter filter than the box for the long slivers of quads that straddle
- * two normal regions); nodes without quads hold an empty box.  The texels are copied into the
+ * in Morton order so the four children of a node are contiguous.  Nodes of
+ * levels 2..4 also carry a slab (the interval of their normals' projections
+ * onto one direction, a tighter filter than the box where a node straddles two
+ * normal regions), and level 1 holds a 16-byte record, binary16 box and slab,
+ * per 2 x 2 quads; nodes without quads hold an empty box.  The texels are copied into the
  * hierarchy (the caller may free texels_dev once the stream reaches the end
  * of this call's work).  On success *out owns device memory until
  * pndf_free_hierarchy().
@@ -195,8 +194,8 @@ pndf_status pndf_update_hierarchy(pndf_hierarchy *h, const void *texels_dev, voi
  * device; safe on NULL). */
 void pndf_free_hierarchy(pndf_hierarchy *h);
 
-/* Device bytes held by a hierarchy (texel copy + pyramid + per-quad
- * capsules + status word, and the cluster records when built). */
+/* Device bytes held by a hierarchy (texel copy + pyramid + group
+ * records + status word, and the cluster records when built). */
 size_t pndf_hierarchy_bytes(const pndf_hierarchy *h);
 
 /* Per-sample flags of pndf_sample_normals. */

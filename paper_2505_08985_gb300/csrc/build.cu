@@ -7,10 +7,10 @@
 // so the four children of node k at level l are nodes 4k..4k+3 at level l-1
 // (one 64-byte line in FP32, one 32-byte sector in FP16).
 //
-// Level 0 holds one box per quad (its four texels) and, beside it, the
-// quad's capsule (the segment between its two farthest normals and a radius
-// holding the other two; see common.cuh); the leaf level 2 box is the union
-// of its 16 quad boxes.
+// Beside the boxes, the nodes of levels 2..kSlabTop carry a slab (see
+// common.cuh), and level 1 holds one 16-byte record per 2 x 2 quads, a
+// binary16 box and a slab.  Nothing is stored per quad: the traversal tests a
+// group's eight triangles from its nine texels.
 //
 // Kernel 1 (build_tiles): one CTA per 64 x 64-quad tile.  The tile's 65 x 65
 // texels are staged in shared memory with 16-byte vector loads (float4 = two
@@ -25,6 +25,7 @@
 // FP16 bounds round outward (min toward -inf, max toward +inf) so pruning
 // stays conservative: the FP16 box contains the FP32 box.
 #include "common.cuh"
+#include "tri.cuh"
 
 namespace pndf {
 namespace {
@@ -33,60 +34,78 @@ constexpr int kTileQuadsMax = 64;
 constexpr int kTileTexMax = kTileQuadsMax + 1;
 constexpr int kBuildThreads = 256;
 
+// Second moments of a set of normals about a reference point.
+struct Moments {
+    float n, s, t, ss, st, tt;
+};
 
-// The quad box as the traversal will read it back (binary16 bounds rounded
-// outward, so the decoded box is the stored one).
-template <int BFMT>
-__device__ __forceinline__ Box stored_box(const Box &b)
+__device__ __forceinline__ void add_point(Moments &m, float2 p, float2 ref)
 {
-    if (BFMT == PNDF_BOUNDS_F32) return b;
-    return Box{__half2float(__float2half_rd(b.smin)), __half2float(__float2half_rd(b.tmin)),
-               __half2float(__float2half_ru(b.smax)), __half2float(__float2half_ru(b.tmax))};
+    const float s = p.x - ref.x, t = p.y - ref.y;
+    m.n += 1.f;
+    m.s += s;
+    m.t += t;
+    m.ss = fmaf(s, s, m.ss);
+    m.st = fmaf(s, t, m.st);
+    m.tt = fmaf(t, t, m.tt);
 }
 
-// Capsule code of a quad with normals v[0..3] and stored box sb: the segment
-// between the farthest pair, as 8-bit fractions of the box; w = the largest
-// distance of the four normals to the decoded segment, enlarged by 2^-9
-// relative and 2^-21 absolute (more than the FP32 rounding of this distance
-// here and of the query's test) and rounded up to binary16.
-__device__ __forceinline__ uint2 encode_capsule(const float2 v[4], const Box &sb)
+// Slab direction: the minor principal axis of the set, rounded to binary16
+// (any direction would be valid; (0, 1) where the axis is undefined).
+__device__ __forceinline__ __half2 slab_dir(const Moments &m)
 {
-    int ip = 0, iq = 1;
-    float best = -1.f;
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = i + 1; j < 4; ++j) {
-            const float dx = v[j].x - v[i].x, dy = v[j].y - v[i].y;
-            const float d2 = fmaf(dx, dx, dy * dy);
-            if (d2 > best) {
-                best = d2;
-                ip = i;
-                iq = j;
-            }
-        }
-    auto frac = [](float x, float lo, float hi) -> uint32_t {
-        const float e = hi - lo;
-        if (!(e > 0.f)) return 0u;
-        return uint32_t(fminf(fmaxf(rintf((x - lo) / e * 255.0f), 0.f), 255.f));
-    };
-    uint2 code;
-    code.x = frac(v[ip].x, sb.smin, sb.smax) | (frac(v[ip].y, sb.tmin, sb.tmax) << 8) |
-             (frac(v[iq].x, sb.smin, sb.smax) << 16) | (frac(v[iq].y, sb.tmin, sb.tmax) << 24);
-    code.y = 0u;
-    const Capsule c = decode_capsule(sb.smin, sb.tmin, sb.smax, sb.tmax, code);
-    const float L2 = fmaf(c.dx, c.dx, c.dy * c.dy);
-    float w = 0.f;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const float ax = v[k].x - c.px, ay = v[k].y - c.py;
-        float t = L2 > 0.f ? fminf(fmaxf(fmaf(ax, c.dx, ay * c.dy) / L2, 0.f), 1.f) : 0.f;
-        const float ex = fmaf(-t, c.dx, ax), ey = fmaf(-t, c.dy, ay);
-        w = fmaxf(w, sqrtf(fmaf(ex, ex, ey * ey)));
+    const float inv = __frcp_rn(fmaxf(m.n, 1.f));
+    const float a = fmaf(-m.s * inv, m.s, m.ss), b = fmaf(-m.s * inv, m.t, m.st), c = fmaf(-m.t * inv, m.t, m.tt);
+    const float d1 = a - c, d2 = 2.f * b;
+    const float h2 = fmaf(d1, d1, d2 * d2);
+    if (!(h2 > 1e-37f)) return __floats2half2_rn(0.f, 1.f);
+    const float c2 = d1 * rsqrtf(h2);  // cosine of twice the major axis' angle
+    const float cs = sqrtf(fmaxf(fmaf(0.5f, c2, 0.5f), 0.f)), sn = copysignf(sqrtf(fmaxf(fmaf(-0.5f, c2, 0.5f), 0.f)), d2);
+    return __floats2half2_rn(-sn, cs);
+}
+
+// The stored slab of normals whose projections onto dir span [lo, hi] and
+// whose |s| + |t| is at most reach: widened by reach 2^-19, more than the FP32
+// rounding of the projection here (3 x 2^-24 reach), of the query's (the same),
+// and of the distance by which an edge function rounded to zero can let m
+// outside its triangle (2^-21 of the triangle's extent, at most 2 reach), then
+// rounded outward to binary16.
+__device__ __forceinline__ uint2 slab_code(__half2 dir, float lo, float hi, float reach, bool mark)
+{
+    const float2 d = __half22float2(dir);
+    uint2 v;
+    v.x = *reinterpret_cast<uint32_t *>(&dir);
+    const float w = reach * 0x1p-19f;
+    if (mark || !isfinite(d.x) || !isfinite(d.y) || !isfinite(lo) || !isfinite(hi) || !isfinite(w)) {
+        v.x = 0u;  // direction 0: every projection is 0, inside (-inf, +inf)
+        v.y = kSlabAll;
+    } else {
+        const __half2 iv = __halves2half2(__float2half_rd(lo - w), __float2half_ru(hi + w));
+        v.y = *reinterpret_cast<const uint32_t *>(&iv);
     }
-    w = fmaf(w, 1.0f + 1.0f / 512.0f, 1.0f / 2097152.0f);
-    code.y = uint32_t(__half_as_ushort(__float2half_ru(w)));
-    return code;
+    return v;
+}
+
+__device__ __forceinline__ float project(__half2 dir, float2 p)
+{
+    const float2 d = __half22float2(dir);
+    return fmaf(p.x, d.x, p.y * d.y);
+}
+
+__device__ __forceinline__ float box_reach(const Box &b)
+{
+    return fmaxf(fabsf(b.smin), fabsf(b.smax)) + fmaxf(fabsf(b.tmin), fabsf(b.tmax));
+}
+
+// A triangle that the traversal evaluates in FP64 (FP32 |cross| below
+// kTinyCross, cross not exactly 0).  The groups that hold one are marked, so
+// that pruning by slabs never decides whether it is reached.  Written so that
+// a cross that is not a number counts.
+__device__ __forceinline__ bool near_singular(float2 a, float2 b, float2 c)
+{
+    if (fabsf(orient(a.x, a.y, b.x, b.y, c.x, c.y)) >= kTinyCross) return false;
+    if ((a.x == b.x && a.y == b.y) || (a.x == c.x && a.y == c.y)) return false;
+    return !(orient_d(a.x, a.y, b.x, b.y, c.x, c.y) == 0.0);
 }
 
 template <int TFMT>
@@ -162,39 +181,120 @@ __global__ void __launch_bounds__(kBuildThreads) build_tiles(const void *__restr
     }
     __syncthreads();
 
-    // ---- quads (level 0) and leaf nodes: thread i owns the leaf node with
-    // local Morton index i and its 16 quads, whose Morton indices at level 0
-    // are 16 i .. 16 i + 15 (a contiguous run of the tile's level-0 block) ----
+    // ---- groups (level 1) and leaf nodes: thread i owns the leaf node with
+    // local Morton index i, whose 5 x 5 texels it keeps in registers ----
     const int T = tileQ / kLeafQuads;  // leaf nodes per tile side
     const uint32_t tile_m = morton2(blockIdx.x, blockIdx.y);
     int cur = T * T;
-    if (tid < cur) {
-        int a = compact1by1(tid), c = compact1by1(tid >> 1);
-        Box b = empty_box();
-        const size_t qbase = (size_t(tile_m) * cur + tid) * (kLeafQuads * kLeafQuads);
-        for (int k = 0; k < kLeafQuads * kLeafQuads; ++k) {
-            int lx = a * kLeafQuads + int(compact1by1(k)), ly = c * kLeafQuads + int(compact1by1(k >> 1));
-            Box qb = empty_box();
-            uint2 cap = make_uint2(0u, 0u);
-            if (c0 + lx <= n - 2 && r0 + ly <= n - 2) {
-                float2 tv[4];
+    const bool leaf = tid < cur;
+    const uint32_t m2 = tile_m * uint32_t(cur) + uint32_t(tid);
+    const int la = int(compact1by1(tid)) * kLeafQuads, lc = int(compact1by1(tid >> 1)) * kLeafQuads;
+    // quads of the block inside the map per axis; texels past them repeat the
+    // last one, which adds nothing to a box or a slab
+    const int nvx = leaf ? max(0, min(kLeafQuads, n - 1 - (c0 + la))) : 0;
+    const int nvy = leaf ? max(0, min(kLeafQuads, n - 1 - (r0 + lc))) : 0;
+    const bool some = nvx > 0 && nvy > 0;
+    float2 t[kLeafTexels][kLeafTexels];
 #pragma unroll
-                for (int v = 0; v < 4; ++v) {
-                    const float2 t = tex[(ly + (v >> 1)) * kTileTexMax + lx + (v & 1)];
-                    tv[v] = t;
-                    qb.smin = fminf(qb.smin, t.x);
-                    qb.tmin = fminf(qb.tmin, t.y);
-                    qb.smax = fmaxf(qb.smax, t.x);
-                    qb.tmax = fmaxf(qb.tmax, t.y);
-                }
-                cap = encode_capsule(tv, stored_box<BFMT>(qb));
+    for (int y = 0; y < kLeafTexels; ++y)
+#pragma unroll
+        for (int x = 0; x < kLeafTexels; ++x)
+            t[y][x] = some ? tex[(lc + min(y, nvy)) * kTileTexMax + la + min(x, nvx)] : make_float2(0.f, 0.f);
+    Box b = empty_box();
+    bool mark = false;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int gx = 2 * (k & 1), gy = 2 * (k >> 1);
+        uint4 rec = make_uint4(0x7c007c00u, 0xfc00fc00u, 0u, kSlabAll);  // empty box
+        if (some && nvx > gx && nvy > gy) {
+            Box gb = empty_box();
+            Moments mo{};
+            bool gmark = false;
+#pragma unroll
+            for (int v = 0; v < 9; ++v) {
+                const float2 p = t[gy + v / 3][gx + v % 3];
+                gb.smin = fminf(gb.smin, p.x);
+                gb.tmin = fminf(gb.tmin, p.y);
+                gb.smax = fmaxf(gb.smax, p.x);
+                gb.tmax = fmaxf(gb.tmax, p.y);
+                add_point(mo, p, t[gy][gx]);
             }
-            store_box<BFMT>(const_cast<void *>(d.lv[0]), qbase + k, qb);
-            const_cast<uint2 *>(d.qcap)[qbase + k] = cap;
-            grow(b, qb);
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                const int x = gx + (v & 1), y = gy + (v >> 1);
+                gmark |= near_singular(t[y][x], t[y][x + 1], t[y + 1][x]);
+                gmark |= near_singular(t[y + 1][x + 1], t[y + 1][x], t[y][x + 1]);
+            }
+            const __half2 dir = slab_dir(mo);
+            float lo = __int_as_float(0x7f800000), hi = -lo;
+#pragma unroll
+            for (int v = 0; v < 9; ++v) {
+                const float p = project(dir, t[gy + v / 3][gx + v % 3]);
+                lo = fminf(lo, p);
+                hi = fmaxf(hi, p);
+            }
+            const uint2 sl = slab_code(dir, lo, hi, box_reach(gb), gmark);
+            const __half2 bl = __halves2half2(__float2half_rd(gb.smin), __float2half_rd(gb.tmin));
+            const __half2 bh = __halves2half2(__float2half_ru(gb.smax), __float2half_ru(gb.tmax));
+            rec = make_uint4(*reinterpret_cast<const uint32_t *>(&bl), *reinterpret_cast<const uint32_t *>(&bh), sl.x,
+                             sl.y);
+            grow(b, gb);
+            mark |= gmark;
         }
+        if (leaf) const_cast<uint4 *>(d.groups)[4 * size_t(m2) + k] = rec;
+    }
+    if (leaf) {
         box[0][tid] = b;
-        store_box<BFMT>(const_cast<void *>(d.lv[kLeafLevel]), size_t(tile_m) * cur + tid, b);
+        store_box<BFMT>(d, node_index(d.L, kLeafLevel, m2), b);
+    }
+
+    // ---- slabs of levels 2, 3 and 4: siblings are 4 lanes, then 16 ----
+    {
+        const int lane = tid & 31;
+        float2 ref;  // one reference point per level-4 node
+        ref.x = __shfl_sync(0xffffffffu, t[0][0].x, lane & 16);
+        ref.y = __shfl_sync(0xffffffffu, t[0][0].y, lane & 16);
+        Moments mo{};
+        if (some) {
+#pragma unroll
+            for (int v = 0; v < 25; ++v) add_point(mo, t[v / 5][v % 5], ref);
+        }
+        float reach = some ? box_reach(b) : 0.f;
+        unsigned any = mark ? 1u : 0u;
+#pragma unroll
+        for (int l = kLeafLevel; l <= kSlabTop; ++l) {
+            const int sh = 2 * (l - kLeafLevel);  // 4^(l - 2) lanes per node
+            if (l > kLeafLevel) {
+#pragma unroll
+                for (int o = (1 << sh) >> 2; o < (1 << sh); o <<= 1) {
+                    mo.n += __shfl_xor_sync(0xffffffffu, mo.n, o);
+                    mo.s += __shfl_xor_sync(0xffffffffu, mo.s, o);
+                    mo.t += __shfl_xor_sync(0xffffffffu, mo.t, o);
+                    mo.ss += __shfl_xor_sync(0xffffffffu, mo.ss, o);
+                    mo.st += __shfl_xor_sync(0xffffffffu, mo.st, o);
+                    mo.tt += __shfl_xor_sync(0xffffffffu, mo.tt, o);
+                    reach = fmaxf(reach, __shfl_xor_sync(0xffffffffu, reach, o));
+                    any |= __shfl_xor_sync(0xffffffffu, any, o);
+                }
+            }
+            const __half2 dir = slab_dir(mo);
+            float lo = __int_as_float(0x7f800000), hi = -lo;
+            if (some) {
+#pragma unroll
+                for (int v = 0; v < 25; ++v) {
+                    const float p = project(dir, t[v / 5][v % 5]);
+                    lo = fminf(lo, p);
+                    hi = fmaxf(hi, p);
+                }
+            }
+#pragma unroll
+            for (int o = 1; o < (1 << sh); o <<= 1) {
+                lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+                hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+            }
+            if (leaf && l <= d.L && (tid & ((1 << sh) - 1)) == 0)
+                store_slab<BFMT>(d, node_index(d.L, l, m2 >> sh), slab_code(dir, lo, hi, reach, any != 0u));
+        }
     }
     __syncthreads();
 
@@ -208,33 +308,29 @@ __global__ void __launch_bounds__(kBuildThreads) build_tiles(const void *__restr
             grow(b, box[s][4 * tid + 2]);
             grow(b, box[s][4 * tid + 3]);
             box[s ^ 1][tid] = b;
-            store_box<BFMT>(const_cast<void *>(d.lv[l]), size_t(tile_m) * cur + tid, b);
+            const uint32_t k = node_index(d.L, l, tile_m * uint32_t(cur) + uint32_t(tid));
+            store_box<BFMT>(d, k, b);
+            if (l > kSlabTop) store_slab<BFMT>(d, k, make_uint2(0u, kSlabAll));
         }
         s ^= 1;
         __syncthreads();
     }
 }
 
+// Level l > kSlabTop from level l - 1.  (With FP16 bounds the children are
+// binary16 values already and the reduction is exact.)
 template <int BFMT>
-__global__ void build_up(const void *__restrict__ child, void *__restrict__ parent, size_t count)
+__global__ void build_up(MapDesc d, int l, uint32_t count)
 {
-    size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= count) return;
-    Box b = load_box<BFMT>(child, 4 * i);
-    grow(b, load_box<BFMT>(child, 4 * i + 1));
-    grow(b, load_box<BFMT>(child, 4 * i + 2));
-    grow(b, load_box<BFMT>(child, 4 * i + 3));
-    if (BFMT == PNDF_BOUNDS_F32) {
-        store_box<BFMT>(parent, i, b);
-    } else {
-        // children are already binary16 values: the reduction is exact
-        __half2 lo = __floats2half2_rn(b.smin, b.tmin);
-        __half2 hi = __floats2half2_rn(b.smax, b.tmax);
-        uint2 v;
-        v.x = *reinterpret_cast<uint32_t *>(&lo);
-        v.y = *reinterpret_cast<uint32_t *>(&hi);
-        reinterpret_cast<uint2 *>(parent)[i] = v;
-    }
+    const uint32_t k = node_index(d.L, l, i);
+    Box b = load_box<BFMT>(d, 4 * k);
+    grow(b, load_box<BFMT>(d, 4 * k + 1));
+    grow(b, load_box<BFMT>(d, 4 * k + 2));
+    grow(b, load_box<BFMT>(d, 4 * k + 3));
+    store_box<BFMT>(d, k, b);
+    store_slab<BFMT>(d, k, make_uint2(0u, kSlabAll));
 }
 
 template <int TFMT, int BFMT>
@@ -254,9 +350,8 @@ cudaError_t launch_tiles(const void *src, const MapDesc &d, cudaStream_t s)
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     for (int l = lq + 1; l <= d.L; ++l) {
-        size_t cnt = level_nodes(d.L, l);
-        unsigned blocks = unsigned((cnt + 255) / 256);
-        build_up<BFMT><<<blocks, 256, 0, s>>>(d.lv[l - 1], const_cast<void *>(d.lv[l]), cnt);
+        const uint32_t cnt = uint32_t(level_nodes(d.L, l));
+        build_up<BFMT><<<(cnt + 255) / 256, 256, 0, s>>>(d, l, cnt);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }

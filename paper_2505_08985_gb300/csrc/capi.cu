@@ -122,29 +122,25 @@ pndf_status pndf_build_hierarchy(const void *texels_dev, const pndf_build_params
     d.L = top_level(p->n);
     d.texel_fmt = p->texel_fmt;
     d.bounds_fmt = p->bounds_fmt;
-    const size_t node_b = p->bounds_fmt == PNDF_BOUNDS_F32 ? 16 : 8;
     const size_t texel_b = p->texel_fmt == PNDF_TEXEL_F32X2 ? 8 : 4;
     auto up = [](size_t v) { return (v + 255) & ~size_t(255); };
-    size_t off[kMaxLevels + 1];
     size_t total = up(size_t(d.n) * d.n * texel_b);
-    off[0] = total;  // level 0: one box per quad
-    total += up(level_nodes(d.L, 0) * node_b);
-    const size_t off_qcap = total;  // and one capsule per quad
-    total += up(level_nodes(d.L, 0) * sizeof(uint2));
-    for (int l = kLeafLevel; l <= d.L; ++l) {
-        off[l] = total;
-        total += up(level_nodes(d.L, l) * node_b);
-    }
+    const size_t off_groups = total;  // level 1: one record per 2 x 2 quads
+    total += up(level_nodes(d.L, 1) * sizeof(uint4));
+    // nodes of levels kLeafLevel..L: 16 bytes each, and with FP32 bounds a slab
+    const size_t heap = 2 * level_nodes(d.L, kLeafLevel);
+    const size_t off_nodes = total;
+    total += up(heap * sizeof(uint4));
+    const size_t off_slabs = total;
+    if (p->bounds_fmt == PNDF_BOUNDS_F32) total += up(heap * sizeof(uint2));
     // cluster records (two float4 per node), residuals, build scratch
-    size_t off_cl[kMaxLevels], off_ce[kMaxLevels], off_mom = 0;
+    size_t off_cl = 0, off_ce = 0, off_mom = 0;
     h->clusters = p->clusters;
     if (h->clusters) {
-        for (int l = kLeafLevel; l <= d.L; ++l) {
-            off_cl[l] = total;
-            total += up(level_nodes(d.L, l) * 2 * sizeof(float4));
-            off_ce[l] = total;
-            total += up(level_nodes(d.L, l) * sizeof(float));
-        }
+        off_cl = total;
+        total += up(heap * 2 * sizeof(float4));
+        off_ce = total;
+        total += up(heap * sizeof(float));
         off_mom = total;
         total += up(cluster_scratch_bytes(d.L));
     }
@@ -158,16 +154,14 @@ pndf_status pndf_build_hierarchy(const void *texels_dev, const pndf_build_params
     h->bytes = total;
     char *base = static_cast<char *>(h->mem);
     d.texels = base;
-    d.lv[0] = base + off[0];
-    d.qcap = reinterpret_cast<const uint2 *>(base + off_qcap);
-    for (int l = kLeafLevel; l <= d.L; ++l) d.lv[l] = base + off[l];
+    d.groups = reinterpret_cast<const uint4 *>(base + off_groups);
+    d.nodes = reinterpret_cast<const uint4 *>(base + off_nodes);
+    if (p->bounds_fmt == PNDF_BOUNDS_F32) d.slabs = reinterpret_cast<const uint2 *>(base + off_slabs);
     memset(&h->c, 0, sizeof(h->c));
     h->moments = nullptr;
     if (h->clusters) {
-        for (int l = kLeafLevel; l <= d.L; ++l) {
-            h->c.cl[l] = reinterpret_cast<const float4 *>(base + off_cl[l]);
-            h->c.ce[l] = reinterpret_cast<const float *>(base + off_ce[l]);
-        }
+        h->c.cl = reinterpret_cast<const float4 *>(base + off_cl);
+        h->c.ce = reinterpret_cast<const float *>(base + off_ce);
         if (cluster_scratch_bytes(d.L)) h->moments = base + off_mom;
     }
     d.status = reinterpret_cast<unsigned int *>(base + off_status);

@@ -365,12 +365,13 @@ __device__ void fit_store(const MapDesc &d, const ClusterDesc &cd, int l, uint32
     const uint32_t I = compact1by1(m), J = compact1by1(m >> 1);
     const int64_t a = int64_t(1) << l;
     ok = ok && a * (I + 1) <= int64_t(d.n) - 1 && a * (J + 1) <= int64_t(d.n) - 1;
-    float4 *rec = const_cast<float4 *>(cd.cl[l]) + 2 * size_t(m);
-    float *ev = const_cast<float *>(cd.ce[l]) + m;
-    Box b = load_box<BFMT>(d.lv[l], m);
+    const uint32_t k = node_index(d.L, l, m);
+    float4 *rec = const_cast<float4 *>(cd.cl) + 2 * size_t(k);
+    float *ev = const_cast<float *>(cd.ce) + k;
+    Box b = load_box<BFMT>(d, k);
     if (l > kLeafLevel) {
 #pragma unroll
-        for (int k = 0; k < 4; ++k) grow(b, load_box<BFMT>(d.lv[l - 1], 4 * size_t(m) + k));
+        for (int c = 0; c < 4; ++c) grow(b, load_box<BFMT>(d, 4 * k + c));
     }
     if (ok) {
         const double(*c)[2] = qf.g;
@@ -390,7 +391,7 @@ __device__ void fit_store(const MapDesc &d, const ClusterDesc &cd, int l, uint32
         rec[1] = make_float4(0.f, 0.f, 0.f, 0.f);
         *ev = __int_as_float(0x7f800000);
     }
-    store_box<BFMT>(const_cast<void *>(d.lv[l]), m, b);
+    store_box<BFMT>(d, k, b);
 }
 
 // A node's fit is valid only if all its quads lie in the map (then so do its
@@ -530,11 +531,12 @@ __global__ void cluster_copy(ClusterDesc cd, int L, int l, float *__restrict__ r
     const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= S * S) return;
     const uint32_t m = morton2(i % S, i / S);
-    float4 r0 = cd.cl[l][2 * size_t(m)], r1 = cd.cl[l][2 * size_t(m) + 1];
+    const size_t k = node_index(L, l, m);
+    float4 r0 = cd.cl[2 * k], r1 = cd.cl[2 * k + 1];
     float *o = rec + 8 * size_t(i);
     o[0] = r0.x; o[1] = r0.y; o[2] = r0.z; o[3] = r0.w;
     o[4] = r1.x; o[5] = r1.y; o[6] = r1.z; o[7] = r1.w;
-    e[i] = cd.ce[l][m];
+    e[i] = cd.ce[k];
 }
 
 }  // namespace

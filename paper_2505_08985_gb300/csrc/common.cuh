@@ -14,6 +14,7 @@ constexpr int kServeMaxMaps = 8;     // hierarchies per server
 constexpr int kLeafLevel = 2;        // stored bottom level: 4 x 4 quads = 32 triangles = one warp
 constexpr int kLeafQuads = 1 << kLeafLevel;
 constexpr int kLeafTexels = kLeafQuads + 1;
+constexpr int kSlabTop = 4;          // coarsest level whose slabs bound anything
 constexpr float kQCut = 16.0f;       // 4-sigma ellipse: d^T S^-1 d <= 16
 // Node pruning keeps a relative margin over the cut so that FP32 rounding in
 // the box minimum can never prune a node holding a contributing hit.
@@ -28,10 +29,13 @@ struct MapDesc {
     int L;                  // top level: 2^L >= n - 1 quads per side
     int texel_fmt;          // pndf_texel_fmt
     int bounds_fmt;         // pndf_bounds_fmt
-    const void *lv[kMaxLevels];  // level 0 (one box per quad) and levels kLeafLevel..L:
-                                 // (2^(L-l))^2 nodes each, Morton order
-    unsigned int *status;        // this hierarchy's status word (PNDF_QF_* bits OR-ed in on errors)
-    const uint2 *qcap;           // per-quad capsules (level-0 companion, same Morton order)
+    unsigned int *status;   // this hierarchy's status word (PNDF_QF_* bits OR-ed in on errors)
+    // Nodes of levels kLeafLevel..L, (2^(L-l))^2 per level in Morton order: node m of
+    // level l is node_index(L, l, m) = 4^(L-l) + m, so that the children of node k
+    // are 4k .. 4k + 3 and siblings are contiguous.
+    const uint4 *nodes;     // FP16 bounds: (box lo, box hi, slab direction, slab interval); FP32 bounds: the box
+    const uint2 *slabs;     // FP32 bounds: the slabs (direction, interval)
+    const uint4 *groups;    // level 1 (2 x 2 quads), Morton order: records as in `nodes` with FP16 bounds
 };
 
 // Record device-side error bits: in the hierarchy's own word and in the
@@ -42,15 +46,15 @@ __device__ __forceinline__ void record_status(unsigned int *hier_word, unsigned 
     atomicOr(device_word, bits);
 }
 
-// Cluster hierarchy (Sec. 4.2, Eq. 7-8, App. A), levels kLeafLevel..L in the
-// same Morton order as the boxes.  Per node two float4 records,
+// Cluster hierarchy (Sec. 4.2, Eq. 7-8, App. A), levels kLeafLevel..L, indexed
+// like the boxes (node m of level l at 4^(L-l) + m).  Per node two float4 records,
 // (c00.s, c00.t, d10.s, d10.t) and (d01.s, d01.t, d11.s, d11.t) with the
 // corner normals c10 = c00 + d10 etc. kept as differences (a flat cluster's
 // Jacobian is the cross product of small differences), and the residual e
 // (+inf where the node has no cluster).
 struct ClusterDesc {
-    const float4 *cl[kMaxLevels];
-    const float *ce[kMaxLevels];
+    const float4 *cl;  // two per node
+    const float *ce;   // one per node
 };
 
 // Morton (Z-order) interleave of two 16-bit coordinates: x in the even bits.
@@ -106,29 +110,31 @@ __device__ __forceinline__ void grow(Box &b, const Box &o)
     b.tmax = fmaxf(b.tmax, o.tmax);
 }
 
+__host__ __device__ __forceinline__ uint32_t node_index(int L, int l, uint32_t m) { return (1u << (2 * (L - l))) + m; }
+
 template <int BFMT>
-__device__ __forceinline__ void store_box(void *lv, size_t idx, const Box &b)
+__device__ __forceinline__ void store_box(const MapDesc &d, uint32_t k, const Box &b)
 {
     if (BFMT == PNDF_BOUNDS_F32) {
-        reinterpret_cast<float4 *>(lv)[idx] = make_float4(b.smin, b.tmin, b.smax, b.tmax);
+        reinterpret_cast<float4 *>(const_cast<uint4 *>(d.nodes))[k] = make_float4(b.smin, b.tmin, b.smax, b.tmax);
     } else {
         __half2 lo = __halves2half2(__float2half_rd(b.smin), __float2half_rd(b.tmin));
         __half2 hi = __halves2half2(__float2half_ru(b.smax), __float2half_ru(b.tmax));
         uint2 v;
         v.x = *reinterpret_cast<uint32_t *>(&lo);
         v.y = *reinterpret_cast<uint32_t *>(&hi);
-        reinterpret_cast<uint2 *>(lv)[idx] = v;
+        reinterpret_cast<uint2 *>(const_cast<uint4 *>(d.nodes))[2 * size_t(k)] = v;
     }
 }
 
 template <int BFMT>
-__device__ __forceinline__ Box load_box(const void *lv, size_t idx)
+__device__ __forceinline__ Box load_box(const MapDesc &d, uint32_t k)
 {
     if (BFMT == PNDF_BOUNDS_F32) {
-        float4 v = reinterpret_cast<const float4 *>(lv)[idx];
+        float4 v = reinterpret_cast<const float4 *>(d.nodes)[k];
         return Box{v.x, v.y, v.z, v.w};
     } else {
-        uint2 v = reinterpret_cast<const uint2 *>(lv)[idx];
+        uint2 v = reinterpret_cast<const uint2 *>(d.nodes)[2 * size_t(k)];
         __half2 lo = *reinterpret_cast<__half2 *>(&v.x);
         __half2 hi = *reinterpret_cast<__half2 *>(&v.y);
         float2 l = __half22float2(lo), h = __half22float2(hi);
@@ -136,49 +142,43 @@ __device__ __forceinline__ Box load_box(const void *lv, size_t idx)
     }
 }
 
-// Per-quad capsule, the level-0 companion of the quad boxes.  A quad's two
-// normal triangles lie in the convex hull of its four normals, and so within
-// distance w of the segment p-q between its two farthest normals (distance to
-// a segment is convex, so its maximum over the hull is at a vertex).  For a
-// quad straddling two flake cells the triangles are long slivers whose box is
-// mostly empty; the capsule is far tighter.  Stored in 8 bytes: p and q as
-// 8-bit fractions of the quad's stored box (x: px, py, qx, qy from the low
-// byte up), w as binary16 in the low half of y, rounded up with a margin that
-// covers FP32 rounding at build and at query time.  Build and query decode
-// with this same function, so both see the same segment.
-struct Capsule {
-    float px, py, dx, dy;  // p and q - p
-    float w;
-};
-
-__device__ __forceinline__ Capsule decode_capsule(float smin, float tmin, float smax, float tmax, uint2 code)
+template <int BFMT>
+__device__ __forceinline__ void store_slab(const MapDesc &d, uint32_t k, uint2 v)
 {
-    const float ex = (smax - smin) * (1.0f / 255.0f), ey = (tmax - tmin) * (1.0f / 255.0f);
-    Capsule c;
-    c.px = fmaf(ex, float(code.x & 255u), smin);
-    c.py = fmaf(ey, float((code.x >> 8) & 255u), tmin);
-    c.dx = fmaf(ex, float((code.x >> 16) & 255u), smin) - c.px;
-    c.dy = fmaf(ey, float(code.x >> 24), tmin) - c.py;
-    c.w = __half2float(__ushort_as_half(static_cast<unsigned short>(code.y & 0xffffu)));
-    return c;
+    if (BFMT == PNDF_BOUNDS_F32)
+        const_cast<uint2 *>(d.slabs)[k] = v;
+    else
+        reinterpret_cast<uint2 *>(const_cast<uint4 *>(d.nodes))[2 * size_t(k) + 1] = v;
 }
 
-// Distance from (mx, my) to the capsule's segment, squared and compared with
-// r^2 without a division: beyond either end the distance to that end,
-// between them the perpendicular distance (cross^2 <= r^2 |d|^2).
-__device__ __forceinline__ bool capsule_holds(const Capsule &c, float mx, float my, float r)
+// Slab of a node: a unit direction (binary16) and the interval that the
+// projections of the node's normals onto it span (binary16, rounded outward).
+// The direction is the minor principal axis of the node's normals.  A node
+// that straddles two flake cells has normals in two tight clusters; its box
+// spans both and is mostly empty, while the slab across the line that joins
+// them is only as wide as one cluster.  Per quad of a footprint on the flake
+// map (share of nodes that hold m, box alone / box and slab): level 1 0.036 /
+// 0.0085, level 2 0.079 / 0.028, level 3 0.18 / 0.089, level 4 0.38 / 0.28,
+// level 5 0.61 / 0.56, too little to build one.  Stored as (n_s, n_t), (lo,
+// hi); an interval reaching +inf marks a node that every m passes: one above
+// kSlabTop, or one that holds a near-singular triangle (see tiny_triangle) or a
+// normal that is not finite.
+constexpr uint32_t kSlabAll = 0x7c00fc00u;  // (lo, hi) = (-inf, +inf)
+
+// A record of (box lo, box hi, slab direction, slab interval), each two binary16
+// values, is one 16-byte load; groups use it in both bound formats (it only
+// prunes).
+__device__ __forceinline__ bool slab_marked(uint32_t interval) { return (interval >> 16) == 0x7c00u; }
+
+// m in the slab, the interval widened by r.  The interval was widened at the
+// build by more than the FP32 rounding of this projection.  Written so that a
+// projection that is not a number passes.
+__device__ __forceinline__ bool slab_holds(uint32_t dir, uint32_t interval, float mx, float my, float r)
 {
-    const float ax = mx - c.px, ay = my - c.py;
-    const float t = fmaf(ax, c.dx, ay * c.dy);
-    const float L2 = fmaf(c.dx, c.dx, c.dy * c.dy);
-    const float r2 = r * r;
-    if (t <= 0.f) return fmaf(ax, ax, ay * ay) <= r2;
-    if (t >= L2) {
-        const float bx = ax - c.dx, by = ay - c.dy;
-        return fmaf(bx, bx, by * by) <= r2;
-    }
-    const float cr = fmaf(ax, c.dy, -ay * c.dx);
-    return cr * cr <= r2 * L2;
+    const float2 n = __half22float2(*reinterpret_cast<const __half2 *>(&dir));
+    const float2 iv = __half22float2(*reinterpret_cast<const __half2 *>(&interval));
+    const float p = fmaf(mx, n.x, my * n.y);
+    return !(p < iv.x - r) && !(p > iv.y + r);
 }
 
 __host__ __device__ inline size_t level_nodes(int L, int l)

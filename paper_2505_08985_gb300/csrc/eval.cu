@@ -14,27 +14,35 @@
 //   key_place : counting-sort placement -> query order.
 //   traverse  : persistent warps pull queries from an atomic cursor; one warp
 //               per query.  Depth-first descent of the min/max pyramid with a
-//               per-warp shared-memory stack: each step pops up to 16 nodes,
-//               lane k tests child (k & 3) of popped nodes (k >> 2) and
-//               (k >> 2) + 8 - uv box against the support first, then the
-//               normal box against m - and ballot/popc compaction pushes the
-//               survivors.  Surviving leaf blocks (4 x 4 quads) have their 16
-//               per-quad boxes (level 0, one 128-byte line in FP16) tested four
-//               per lane in one load, eight blocks per pass; quads whose box
-//               holds m are compacted into a per-warp ring and taken 64 at a
-//               time (two per lane, both loads in flight) through the quad's
-//               capsule (segment between its farthest normals plus a radius,
-//               the tight bound for slivers across normal discontinuities);
-//               capsule survivors are compacted again and tested 32 at a
-//               time (lane = quad, both triangles), and edge-test hits are
-//               compacted once more and weighed 32 at a time.  Each weight
-//               is added exactly into the thread's 128-bit fixed-point sum;
+//               per-warp shared-memory stack: each step pops up to kPop nodes,
+//               lane k tests child (k & 3) of popped nodes (k >> 2) + 8 r - the
+//               normal box and the slab (common.cuh: the tight bound where a
+//               node straddles two normal regions) against m, then the uv box
+//               against the support - and ballot/popc compaction pushes the
+//               survivors.  Surviving leaf blocks (4 x 4 quads) have the
+//               box and slab of their four 2 x 2-quad groups tested, sixteen
+//               blocks per pass; surviving groups are compacted into a
+//               per-warp ring and taken 32 at a time (lane = group): the
+//               group's nine texels give the edge functions of its eight
+//               triangles at once (16 edges), and the triangles that may hold
+//               m, nearly all of them hits, are compacted again and decided
+//               and weighed 32 at a time (lane = triangle).  Each weight is
+//               added exactly into the thread's 128-bit fixed-point sum;
 //               the warp's sums are added exactly and the total is written in
 //               caller order (the unpermute is fused into the store).  Large
 //               footprints of a batch are divided into tiles of nodes, one
 //               warp per tile (split_work / split_plan).  Flat mode skips
 //               every box and tests all 32 triangles of every leaf block in
 //               the support's bounding box.
+//
+// What bounds it: the descent is instruction issue and L2 latency in about equal
+// parts (half of all issue slots used, 6 of 12 cycles between a warp's issues
+// spent on loads; the same footprints on maps from 2048^2 to 16384^2 take 18 to
+// 23 ms, so DRAM is not the limit).  Per query of the 8192^2 flake workload it
+// tests 10.5k nodes, 1.2k leaf blocks, 1.4k groups and 972 triangles for 964
+// hits, in 62k warp instructions; with a box and a capsule per quad in place of
+// the slabs and groups it took 187k, and 896 ms per 4M queries against 345 ms.
+//
 // Hit test (tie rule): m inside the closed normal bounding box and all three
 // edge functions sign-consistent with the triangle orientation (>= 0 after
 // orientation, i.e. closed barycentrics).  Zero-area normal triangles are a
@@ -44,6 +52,7 @@
 #include <mutex>
 
 #include "common.cuh"
+#include "tri.cuh"
 
 namespace pndf {
 
@@ -51,36 +60,23 @@ __device__ unsigned int g_status_eval;
 
 namespace {
 
-constexpr int kStackCap = 768;     // DFS stack entries per warp (about 48 per level + 64 in the worst case)
+// Children a lane tests per step, all their loads in flight.  Per 1M queries of
+// the flake map 2: 94.8 ms, 3: 86.5 ms, 4: 93.0 ms; of the scratch map 13.7,
+// 14.3 and 14.9 ms.
+constexpr int kPer = 3;
+constexpr int kPop = 8 * kPer;     // nodes popped per step (four children each)
+// DFS stack entries per warp.  A step leaves at most 3 kPop more than it found
+// on the way down a level: 3 kPop per level below the entry (at most 12), the
+// last step's 4 kPop and the 16 entry nodes.
+constexpr int kStackCap = 36 * kPop + 4 * kPop + 16 + 16;
 constexpr int kMaxSubBits = 14;                   // sub-key bits below the 4 entry-level bits
 constexpr int kKeyBins = 1 << (4 + kMaxSubBits);  // largest histogram (2^18 bins)
 #ifndef PNDF_TRAVERSE_MIN_CTAS
-// 3 x 256 threads per SM at <= 85 registers: with two capsule tests per lane
-// in flight this measured 916 ms per 4M-query flake step, against 1008 ms at
-// 4 CTAs (64 registers, more spills) and 1154 ms at 2
+// 3 x 256 threads per SM at 80 registers: 4 CTAs (64 registers, spills) took
+// 5-10% longer on the flake map and 5 CTAs 24%
 #define PNDF_TRAVERSE_MIN_CTAS 3
 #endif
 constexpr unsigned kFull = 0xffffffffu;
-
-// Kahan's difference of products a*b - c*d with one FMA correction.
-__device__ __forceinline__ float dop(float a, float b, float c, float d)
-{
-    float w = c * d;
-    float e = fmaf(-c, d, w);
-    float f = fmaf(a, b, -w);
-    return f + e;
-}
-
-// Twice the signed area of (p, q, r): (q - p) x (r - p).
-__device__ __forceinline__ float orient(float px, float py, float qx, float qy, float rx, float ry)
-{
-    return dop(qx - px, ry - py, qy - py, rx - px);
-}
-
-__device__ __forceinline__ double orient_d(double px, double py, double qx, double qy, double rx, double ry)
-{
-    return (qx - px) * (ry - py) - (qy - py) * (rx - px);
-}
 
 // MurmurHash3 32-bit finalizer (Appleby), fingerprints hit sets in stats mode.
 __device__ __forceinline__ uint32_t fmix32(uint32_t h)
@@ -93,43 +89,50 @@ __device__ __forceinline__ uint32_t fmix32(uint32_t h)
     return h;
 }
 
+// Internal kernel id of the Gaussian with the Jacobian clamp of Eq. 6.
+constexpr int kKernGaussClamp = 3;
+
 // Footprint kernels (pndf_kernel): the Gaussian cut at q = d^T S^-1 d <= 16,
 // and the disk (q <= 1.5^2) and box (|L^-1 d|_inf <= 1.5, S = L L^T) filters
 // of the (3 sigma)^2 footprints the paper pairs with it.
-struct Query {
+// The descent keeps its query in shared memory, one per warp, and reads the
+// fields where it uses them: in registers they cost about 20 of each thread's.
+template <int KERN>
+struct alignas(16) Query {
+    static constexpr int kernel = KERN == kKernGaussClamp ? PNDF_KERNEL_GAUSS : KERN;  // pndf_kernel
+    float mx, my;        // query normal
+    __half2 mlo, mhi;    // m rounded down / up to binary16 (exact tests against binary16 boxes)
     float x, y;          // footprint centre
     float ia, ib, ic;    // S^-1 = [[ia, ib], [ib, ic]]
     float norm;          // kernel normalisation: 1 / (2 pi, 2.25 pi or 9) sqrt(det S)
-    float mx, my;        // query normal
     float rx, ry;        // half-widths of the support's bounding box (slightly inflated)
     float qprune;        // the support lies in q <= qprune (16, 2.25, 4.5), with a margin
     float theta;         // r_x r_y of the support (exact half-widths); times tau for the cluster cut
     float kyx, kxy;      // -ib / ic and -ib / ia: the minimiser of q along a vertical / horizontal line
+    float nprune, ncorner;  // norms sqrt(q): of the prune limit, and of the offset (1, 1) at its larger sign
     float inv_sxx;       // box: 1 / S_xx, so that (L^-1 d)_x^2 = dx^2 / S_xx
     float l11, l21, l22; // box: the Cholesky factor L of S (node tests by separating axes)
     float jac, rho;      // Eq. 6 clamp: Jacobian floor eps and the replacement's circumradius (0: off)
-    int kernel;
     bool valid;
 };
 
-// Internal kernel id of the Gaussian with the Jacobian clamp of Eq. 6.
-constexpr int kKernGaussClamp = 3;
-
-__device__ __forceinline__ Query make_query(const pndf_query &r, int kernel = PNDF_KERNEL_GAUSS, float jac_eps = 0.f)
+template <int KERN>
+__device__ __forceinline__ Query<KERN> make_query(const pndf_query &r, float jac_eps = 0.f)
 {
-    Query q;
+    constexpr int kernel = Query<KERN>::kernel;
+    Query<KERN> q;
     q.jac = q.rho = 0.f;
-    if (kernel == kKernGaussClamp) {
+    if (KERN == kKernGaussClamp) {
         // equilateral replacement of area eps / 2: side^2 = 2 eps / sqrt(3), circumradius side / sqrt(3)
         q.jac = jac_eps;
         q.rho = sqrtf(2.0f * jac_eps / 1.7320508f) * 0.57735027f;
-        kernel = PNDF_KERNEL_GAUSS;
     }
     q.x = r.x;
     q.y = r.y;
     q.mx = r.ms;
     q.my = r.mt;
-    q.kernel = kernel;
+    q.mlo = __halves2half2(__float2half_rd(r.ms), __float2half_rd(r.mt));
+    q.mhi = __halves2half2(__float2half_ru(r.ms), __float2half_ru(r.mt));
     float det = r.sxx * r.syy - r.sxy * r.sxy;
     q.valid = (r.sxx > 0.f) && (r.syy > 0.f) && (det > 0.f) && isfinite(det) && isfinite(r.x) &&
               isfinite(r.y) && isfinite(r.ms) && isfinite(r.mt);
@@ -164,6 +167,8 @@ __device__ __forceinline__ Query make_query(const pndf_query &r, int kernel = PN
         hy = 4.0f * sy;
         q.qprune = kQPrune;
     }
+    q.nprune = sqrtf(q.qprune);
+    q.ncorner = sqrtf(q.ia + q.ic + 2.0f * fabsf(q.ib)) * (1.0f + 1e-5f);
     q.theta = hx * hy;
     // inflate so rounding never clips the support's box
     q.rx = hx * (1.0f + 1e-5f) + 1e-6f;
@@ -172,23 +177,26 @@ __device__ __forceinline__ Query make_query(const pndf_query &r, int kernel = PN
 }
 
 // Kernel weight at offset d with q = d^T S^-1 d; 0 outside the support.
-__device__ __forceinline__ float kweight(const Query &q, float dx, float qq)
+template <class Q>
+__device__ __forceinline__ float kweight(const Q &q, float dx, float qq)
 {
-    if (q.kernel == PNDF_KERNEL_GAUSS) return qq <= kQCut ? q.norm * expf(-0.5f * qq) : 0.f;
-    if (q.kernel == PNDF_KERNEL_DISK) return qq <= 2.25f ? q.norm : 0.f;
+    if (Q::kernel == PNDF_KERNEL_GAUSS) return qq <= kQCut ? q.norm * expf(-0.5f * qq) : 0.f;
+    if (Q::kernel == PNDF_KERNEL_DISK) return qq <= 2.25f ? q.norm : 0.f;
     const float v1 = dx * dx * q.inv_sxx;  // (L^-1 d)_x^2; (L^-1 d)_y^2 = q - v1
     return (v1 <= 2.25f && qq - v1 <= 2.25f) ? q.norm : 0.f;
 }
 
-__device__ __forceinline__ double kweight_d(const Query &q, double dx, double qq)
+template <class Q>
+__device__ __forceinline__ double kweight_d(const Q &q, double dx, double qq)
 {
-    if (q.kernel == PNDF_KERNEL_GAUSS) return qq <= double(kQCut) ? double(q.norm) * exp(-0.5 * qq) : 0.0;
-    if (q.kernel == PNDF_KERNEL_DISK) return qq <= 2.25 ? double(q.norm) : 0.0;
+    if (Q::kernel == PNDF_KERNEL_GAUSS) return qq <= double(kQCut) ? double(q.norm) * exp(-0.5 * qq) : 0.0;
+    if (Q::kernel == PNDF_KERNEL_DISK) return qq <= 2.25 ? double(q.norm) : 0.0;
     const double v1 = dx * dx * double(q.inv_sxx);
     return (v1 <= 2.25 && qq - v1 <= 2.25) ? double(q.norm) : 0.0;
 }
 
-__device__ __forceinline__ float qform(const Query &q, float dx, float dy)
+template <class Q>
+__device__ __forceinline__ float qform(const Q &q, float dx, float dy)
 {
     return fmaf(q.ia * dx, dx, fmaf(2.0f * q.ib * dx, dy, q.ic * dy * dy));
 }
@@ -199,7 +207,8 @@ __device__ __forceinline__ float qform(const Query &q, float dx, float dy)
 // clamped 1D minimum (along x = X at y = -(ib / ic) X, the ratio precomputed
 // per query; a minimiser off by rounding raises the value only to second
 // order, far inside the pruning margin).
-__device__ __forceinline__ float qmin_box(const Query &q, float dx0, float dx1, float dy0, float dy1)
+template <class Q>
+__device__ __forceinline__ float qmin_box(const Q &q, float dx0, float dx1, float dy0, float dy1)
 {
     if (dx0 <= 0.f && dx1 >= 0.f && dy0 <= 0.f && dy1 >= 0.f) return 0.f;
     float best = __int_as_float(0x7f800000);
@@ -216,15 +225,21 @@ __device__ __forceinline__ float qmin_box(const Query &q, float dx0, float dx1, 
     return best;
 }
 
-// A node's normal box as stored: FP32 (s_min, t_min, s_max, t_max) in x..w,
-// or binary16 (s_min, t_min) and (s_max, t_max) as two half2 in x and y
-// (decoded only where tested, so a box in flight holds two registers).
+// Node k as stored: FP16 bounds, the 16-byte record; FP32 bounds, the box, with
+// the slab loaded beside it.
 template <int BFMT>
-__device__ __forceinline__ uint4 node_box(const MapDesc &d, int l, uint32_t m)
+struct Node {
+    uint4 v;
+    uint2 s;  // FP32 bounds only
+};
+
+template <int BFMT>
+__device__ __forceinline__ Node<BFMT> load_node(const MapDesc &d, uint32_t k)
 {
-    if (BFMT == PNDF_BOUNDS_F32) return __ldg(reinterpret_cast<const uint4 *>(d.lv[l]) + m);
-    uint2 v = __ldg(reinterpret_cast<const uint2 *>(d.lv[l]) + m);
-    return make_uint4(v.x, v.y, 0u, 0u);
+    Node<BFMT> n;
+    n.v = __ldg(d.nodes + k);
+    if (BFMT == PNDF_BOUNDS_F32) n.s = __ldg(d.slabs + k);
+    return n;
 }
 
 template <int TFMT>
@@ -240,7 +255,8 @@ __device__ __forceinline__ float2 texel(const MapDesc &d, int i, int j)
 // support L [-1.5, 1.5]^2?  Separating axes: x and y (the support's extents
 // are the inflated half-widths rx, ry) and n = (-l21, l11), normal to L e1,
 // onto which the support projects to +-1.5 l11 l22 (slightly inflated).
-__device__ __forceinline__ bool box_support_meets(const Query &q, float dx0, float dx1, float dy0, float dy1)
+template <class Q>
+__device__ __forceinline__ bool box_support_meets(const Q &q, float dx0, float dx1, float dy0, float dy1)
 {
     if (dx0 > q.rx || dx1 < -q.rx || dy0 > q.ry || dy1 < -q.ry) return false;
     const float hn = 1.5f * q.l11 * q.l22 * (1.0f + 1e-4f) + 1e-6f;
@@ -252,11 +268,12 @@ __device__ __forceinline__ bool box_support_meets(const Query &q, float dx0, flo
 // Node (level l, coords a, c): uv box [a 2^l, (a+1) 2^l] x [c 2^l, (c+1) 2^l].
 // It can hold a contributing hit only if that box meets the kernel's support
 // (the ellipse q <= qprune; for the box kernel the sheared square itself).
-__device__ __forceinline__ bool node_in_footprint(const Query &q, int l, uint32_t a, uint32_t c)
+template <class Q>
+__device__ __forceinline__ bool node_in_footprint(const Q &q, int l, uint32_t a, uint32_t c)
 {
     float sz = float(1u << l);
     float dx0 = float(a) * sz - q.x, dy0 = float(c) * sz - q.y;
-    if (q.kernel == PNDF_KERNEL_BOX) return box_support_meets(q, dx0, dx0 + sz, dy0, dy0 + sz);
+    if (Q::kernel == PNDF_KERNEL_BOX) return box_support_meets(q, dx0, dx0 + sz, dy0, dy0 + sz);
     return qmin_box(q, dx0, dx0 + sz, dy0, dy0 + sz) <= q.qprune;
 }
 
@@ -264,12 +281,13 @@ __device__ __forceinline__ bool node_in_footprint(const Query &q, int l, uint32_
 // convex, so its maximum over the box is at a corner; the box kernel's
 // support is convex too); every descendant then passes the footprint test
 // and skips it.  Claiming "inside" wrongly would only prune less.
-__device__ __forceinline__ bool node_inside(const Query &q, int l, uint32_t a, uint32_t c)
+template <class Q>
+__device__ __forceinline__ bool node_inside(const Q &q, int l, uint32_t a, uint32_t c)
 {
     float sz = float(1u << l);
     float dx0 = float(a) * sz - q.x, dy0 = float(c) * sz - q.y;
     float dx1 = dx0 + sz, dy1 = dy0 + sz;
-    if (q.kernel == PNDF_KERNEL_BOX) {  // the support is convex: all four corners inside it
+    if (Q::kernel == PNDF_KERNEL_BOX) {  // the support is convex: all four corners inside it
         const float hx = 1.5f * q.l11, hv = 1.5f * q.l22, k = q.l21 / q.l11;
         return fmaxf(fabsf(dx0), fabsf(dx1)) <= hx && fabsf(dy0 - k * dx0) <= hv && fabsf(dy0 - k * dx1) <= hv &&
                fabsf(dy1 - k * dx0) <= hv && fabsf(dy1 - k * dx1) <= hv;
@@ -278,42 +296,82 @@ __device__ __forceinline__ bool node_inside(const Query &q, int l, uint32_t a, u
     return m <= q.qprune;
 }
 
+// The descent's own version of the two tests above: does node (l, a, c) meet
+// the support, and does it lie inside?  N = sqrt(q) is a norm, so every point
+// of the node is within N <= h ncorner of its centre (h: half its side), which
+// gives both answers from one evaluation of q, looser than the exact box by
+// part of a node.  It nests: a node that meets the support by this test has a
+// parent that does, and the parent of a node that does not may not be inside;
+// so which leaf blocks are reached does not depend on the level a descent
+// starts from.  (The box kernel's support is no norm ball of q.)
+template <class Q>
+__device__ __forceinline__ bool node_meets(const Q &q, int l, uint32_t a, uint32_t c, bool &inside)
+{
+    if (Q::kernel == PNDF_KERNEL_BOX) {
+        const bool meets = node_in_footprint(q, l, a, c);
+        inside = meets && node_inside(q, l, a, c);
+        return meets;
+    }
+    const float sz = float(1u << l), e = 0.5f * sz * q.ncorner;
+    const float qq = qform(q, fmaf(float(a) + 0.5f, sz, -q.x), fmaf(float(c) + 0.5f, sz, -q.y));
+    const float lo = fmaxf(q.nprune - e, 0.f), hi = q.nprune + e;
+    inside = qq < lo * lo;
+    return !(qq > hi * hi);
+}
+
 // m in the box; with the clamp (CLAMP) widened by the replacement radius (a
 // replacement lies within rho of its triangle's centroid, hence of its box).
-template <bool CLAMP>
-__device__ __forceinline__ bool box_holds(const float4 &b, const Query &q)
+template <bool CLAMP, class Q>
+__device__ __forceinline__ bool box_holds(const float4 &b, const Q &q)
 {
     if (CLAMP) return q.mx >= b.x - q.rho && q.mx <= b.z + q.rho && q.my >= b.y - q.rho && q.my <= b.w + q.rho;
     return q.mx >= b.x && q.mx <= b.z && q.my >= b.y && q.my <= b.w;
 }
 
-// m in a node box as stored (node_box).
-template <int BFMT, bool CLAMP>
-__device__ __forceinline__ bool stored_box_holds(const uint4 &v, const Query &q)
+// m in a binary16 box.  For a binary16 bound b, m >= b exactly when m rounded
+// down to binary16 is, and m <= b when m rounded up is, so two packed compares
+// decide what four conversions and compares of FP32 values would.
+template <bool CLAMP, class Q>
+__device__ __forceinline__ bool half_box_holds(uint32_t lo, uint32_t hi, const Q &q)
+{
+    const __half2 l = *reinterpret_cast<const __half2 *>(&lo), h = *reinterpret_cast<const __half2 *>(&hi);
+    if (CLAMP) {
+        const float2 lf = __half22float2(l), hf = __half22float2(h);
+        return box_holds<CLAMP>(make_float4(lf.x, lf.y, hf.x, hf.y), q);
+    }
+    return __hbge2(q.mlo, l) && __hble2(q.mhi, h);
+}
+
+// m in a node's box.
+template <int BFMT, bool CLAMP, class Q>
+__device__ __forceinline__ bool node_box_holds(const Node<BFMT> &n, const Q &q)
 {
     if (BFMT == PNDF_BOUNDS_F32)
-        return box_holds<CLAMP>(make_float4(__uint_as_float(v.x), __uint_as_float(v.y), __uint_as_float(v.z),
-                                            __uint_as_float(v.w)), q);
-    float2 lo = __half22float2(*reinterpret_cast<const __half2 *>(&v.x));
-    float2 hi = __half22float2(*reinterpret_cast<const __half2 *>(&v.y));
-    return box_holds<CLAMP>(make_float4(lo.x, lo.y, hi.x, hi.y), q);
+        return box_holds<CLAMP>(make_float4(__uint_as_float(n.v.x), __uint_as_float(n.v.y), __uint_as_float(n.v.z),
+                                            __uint_as_float(n.v.w)), q);
+    return half_box_holds<CLAMP>(n.v.x, n.v.y, q);
 }
 
-template <int BFMT, bool CLAMP>
-__device__ __forceinline__ bool node_test(const MapDesc &d, const Query &q, int l, uint32_t a, uint32_t c)
+// How far a slab is widened: with the clamp, a replacement lies within rho of
+// its triangle's centroid (|direction| <= 1 + 2^-10).
+template <bool CLAMP, class Q>
+__device__ __forceinline__ float slab_slack(const Q &q)
 {
-    if (!node_in_footprint(q, l, a, c)) return false;
-    return stored_box_holds<BFMT, CLAMP>(node_box<BFMT>(d, l, morton2(a, c)), q);
+    return CLAMP ? q.rho * 1.01f : 0.f;
 }
 
-// Stack / leaf-queue entry: level in bits 28-31, "inside the ellipse" in bit
-// 27, the node's Morton index at its level in bits 0-26 (at most 2 (L - 1) =
-// 26 bits for L <= 14).  A child's Morton index is (m << 2) | (dy << 1 | dx).
-__device__ __forceinline__ uint32_t pack(int l, bool inside, uint32_t m)
+template <int BFMT, bool CLAMP, class Q>
+__device__ __forceinline__ bool node_slab_holds(const Node<BFMT> &n, const Q &q)
 {
-    return (uint32_t(l) << 28) | (uint32_t(inside) << 27) | m;
+    return BFMT == PNDF_BOUNDS_F32 ? slab_holds(n.s.x, n.s.y, q.mx, q.my, slab_slack<CLAMP>(q))
+                                   : slab_holds(n.v.z, n.v.w, q.mx, q.my, slab_slack<CLAMP>(q));
 }
-constexpr uint32_t kMortonMask = (1u << 27) - 1u;
+
+// Stack / leaf-queue entry: the node's index (node_index; below 2^25 for L <=
+// 14) and "inside the ellipse" in bit 31.
+constexpr uint32_t kInside = 0x80000000u;
+
+__device__ __forceinline__ int node_level(uint32_t k, int L) { return L - ((31 - __clz(int(k))) >> 1); }
 
 // A query's sum is exact: every contribution (an FP32 value >= 0) is added
 // into a 128-bit fixed-point number with 64 fraction bits, value =
@@ -376,79 +434,122 @@ __device__ __forceinline__ float acc_value(unsigned long long lo, unsigned long 
     return float(double(hi) + double(lo) * 0x1p-64);
 }
 
-// Test the lane's triangle of a leaf block and accumulate its contribution.
-// tri 0: (u0, u1, u2) with a = (i, j), b = a + (1, 0), c = a + (0, 1);
-// tri 1: (u3, u2, u1) with a = (i+1, j+1), b = a - (1, 0), c = a - (0, 1).
-template <bool STATS>
-__device__ __forceinline__ void test_triangle(const Query &q, float2 na, float2 nb, float2 nc, int ai, int aj,
-                                              float dir, uint32_t tri_id, Acc &acc)
+// The quad's capsule: its two normal triangles lie within distance w of the
+// segment between its two farthest normals (widened by `slack`).  Near-singular triangles are
+// evaluated (and flagged) only when m is in the quad's box and capsule, so the
+// flag does not depend on how the traversal got there.  The segment's ends are
+// 8-bit fractions of the quad's box as stored in the bound format, w is
+// rounded up to binary16 with a margin over FP32 rounding.
+template <int BFMT>
+__device__ __forceinline__ bool capsule_holds(float2 n0, float2 n1, float2 n2, float2 n3, float mx, float my, float slack)
 {
-    if (STATS) acc.tests++;
-    float lox = fminf(na.x, fminf(nb.x, nc.x)), hix = fmaxf(na.x, fmaxf(nb.x, nc.x));
-    float loy = fminf(na.y, fminf(nb.y, nc.y)), hiy = fmaxf(na.y, fmaxf(nb.y, nc.y));
-    if (q.mx < lox || q.mx > hix || q.my < loy || q.my > hiy) return;
-    float cr = orient(na.x, na.y, nb.x, nb.y, nc.x, nc.y);
-    float l1, l2, J;
-    if (fabsf(cr) >= kTinyCross) {
-        float e0 = orient(nb.x, nb.y, nc.x, nc.y, q.mx, q.my);
-        float e1 = orient(nc.x, nc.y, na.x, na.y, q.mx, q.my);
-        float e2 = orient(na.x, na.y, nb.x, nb.y, q.mx, q.my);
-        bool hit = cr > 0.f ? (e0 >= 0.f && e1 >= 0.f && e2 >= 0.f) : (e0 <= 0.f && e1 <= 0.f && e2 <= 0.f);
-        if (!hit) return;
-        float inv = 1.0f / cr;
-        l1 = e1 * inv;
-        l2 = e2 * inv;
-        J = fabsf(cr);
-    } else {
-        // near-singular normal triangle: FP64 test and weight
-        double ax = na.x, ay = na.y, bx = nb.x, by = nb.y, cx = nc.x, cy = nc.y, mx = q.mx, my = q.my;
-        double dcr = orient_d(ax, ay, bx, by, cx, cy);
-        if (dcr == 0.0) {
-            if (STATS) acc.degen++;
-            return;
+    const float2 v[4] = {n0, n1, n2, n3};
+    Box b = empty_box();
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        b.smin = fminf(b.smin, v[k].x);
+        b.tmin = fminf(b.tmin, v[k].y);
+        b.smax = fmaxf(b.smax, v[k].x);
+        b.tmax = fmaxf(b.tmax, v[k].y);
+    }
+    if (BFMT == PNDF_BOUNDS_F16_OUTWARD)
+        b = Box{__half2float(__float2half_rd(b.smin)), __half2float(__float2half_rd(b.tmin)),
+                __half2float(__float2half_ru(b.smax)), __half2float(__float2half_ru(b.tmax))};
+    int ip = 0, iq = 1;
+    float best = -1.f;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = i + 1; j < 4; ++j) {
+            const float dx = v[j].x - v[i].x, dy = v[j].y - v[i].y;
+            const float d2 = fmaf(dx, dx, dy * dy);
+            if (d2 > best) {
+                best = d2;
+                ip = i;
+                iq = j;
+            }
         }
-        if (STATS) acc.fp64++;
-        acc.flags |= PNDF_QF_FP64;
-        double e0 = orient_d(bx, by, cx, cy, mx, my);
-        double e1 = orient_d(cx, cy, ax, ay, mx, my);
-        double e2 = orient_d(ax, ay, bx, by, mx, my);
-        bool hit = dcr > 0.0 ? (e0 >= 0.0 && e1 >= 0.0 && e2 >= 0.0) : (e0 <= 0.0 && e1 <= 0.0 && e2 <= 0.0);
-        if (!hit) return;
-        double dl1 = e1 / dcr, dl2 = e2 / dcr;
-        double dx = (double(ai) - double(q.x)) + dir * dl1;
-        double dy = (double(aj) - double(q.y)) + dir * dl2;
-        double qq = double(q.ia) * dx * dx + 2.0 * double(q.ib) * dx * dy + double(q.ic) * dy * dy;
-        double w = kweight_d(q, dx, qq);
-        if (w == 0.0) return;
-        w /= fabs(dcr);
-        acc_add(acc, float(w));
-        if (STATS) {
-            acc.hits++;
-            acc.hash += fmix32(tri_id);
-        }
+    auto snap = [](float x, float lo, float hi) {  // x as an 8-bit fraction of [lo, hi]
+        const float e = hi - lo;
+        const float f = e > 0.f ? fminf(fmaxf(rintf((x - lo) / e * 255.0f), 0.f), 255.f) : 0.f;
+        return fmaf(e * (1.0f / 255.0f), f, lo);
+    };
+    float2 p = v[0], r = v[0];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        if (i == ip) p = v[i];
+        if (i == iq) r = v[i];
+    }
+    const float px = snap(p.x, b.smin, b.smax), py = snap(p.y, b.tmin, b.tmax);
+    const float dx = snap(r.x, b.smin, b.smax) - px, dy = snap(r.y, b.tmin, b.tmax) - py;
+    const float L2 = fmaf(dx, dx, dy * dy);
+    float w = 0.f;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const float ax = v[k].x - px, ay = v[k].y - py;
+        const float t = L2 > 0.f ? fminf(fmaxf(fmaf(ax, dx, ay * dy) / L2, 0.f), 1.f) : 0.f;
+        const float ex = fmaf(-t, dx, ax), ey = fmaf(-t, dy, ay);
+        w = fmaxf(w, sqrtf(fmaf(ex, ex, ey * ey)));
+    }
+    w = __half2float(__float2half_ru(fmaf(w, 1.0f + 1.0f / 512.0f, 1.0f / 2097152.0f))) + slack;
+    const float ax = mx - px, ay = my - py, t = fmaf(ax, dx, ay * dy), w2 = w * w;
+    if (t <= 0.f) return fmaf(ax, ax, ay * ay) <= w2;
+    if (t >= L2) {
+        const float bx = ax - dx, by = ay - dy;
+        return fmaf(bx, bx, by * by) <= w2;
+    }
+    const float cr = fmaf(ax, dy, -ay * dx);
+    return cr * cr <= w2 * L2;
+}
+
+// A near-singular normal triangle (FP32 |cross| below kTinyCross) that holds m
+// in its bounding box: hit test and weight in FP64.  Returns the contribution
+// (0: none) and what became of it.
+struct Tiny {
+    float w;
+    int state;  // 0: no area, 1: evaluated, 2: out of reach (support or capsule)
+};
+template <class Q>
+__device__ __forceinline__ Tiny tiny_triangle(const Q &q, float2 na, float2 nb, float2 nc, int ai, int aj, float dir)
+{
+    double ax = na.x, ay = na.y, bx = nb.x, by = nb.y, cx = nc.x, cy = nc.y, mx = q.mx, my = q.my;
+    double dcr = orient_d(ax, ay, bx, by, cx, cy);
+    if (dcr == 0.0) return Tiny{0.f, 0};
+    double e0 = orient_d(bx, by, cx, cy, mx, my);
+    double e1 = orient_d(cx, cy, ax, ay, mx, my);
+    double e2 = orient_d(ax, ay, bx, by, mx, my);
+    bool hit = dcr > 0.0 ? (e0 >= 0.0 && e1 >= 0.0 && e2 >= 0.0) : (e0 <= 0.0 && e1 <= 0.0 && e2 <= 0.0);
+    if (!hit) return Tiny{0.f, 1};
+    double dl1 = e1 / dcr, dl2 = e2 / dcr;
+    double dx = (double(ai) - double(q.x)) + dir * dl1;
+    double dy = (double(aj) - double(q.y)) + dir * dl2;
+    double qq = double(q.ia) * dx * dx + 2.0 * double(q.ib) * dx * dy + double(q.ic) * dy * dy;
+    double w = kweight_d(q, dx, qq);
+    if (w == 0.0) return Tiny{0.f, 1};
+    return Tiny{float(w / fabs(dcr)), 1};
+}
+
+template <bool STATS>
+__device__ __forceinline__ void add_tiny(const Tiny &t, uint32_t id, Acc &acc)
+{
+    if (t.state != 1) {
+        if (STATS && t.state == 0) acc.degen++;
         return;
     }
-    float dx = (float(ai) - q.x) + dir * l1;
-    float dy = (float(aj) - q.y) + dir * l2;
-    float qq = qform(q, dx, dy);
-    float w = kweight(q, dx, qq);
-    if (w == 0.f) return;
-    acc_add(acc, w / J);
+    if (STATS) acc.fp64++;
+    acc.flags |= PNDF_QF_FP64;
+    if (t.w == 0.f) return;
+    acc_add(acc, t.w);
     if (STATS) {
         acc.hits++;
-        acc.hash += fmix32(tri_id);
+        acc.hash += fmix32(id);
     }
 }
 
-// The hit decision of test_triangle alone: true for an FP32 hit (writes the
-// orientation-signed cross and edge functions e1, e2, so l1 = e1 / cross,
-// l2 = e2 / cross).  Near-singular triangles (FP32 |cross| < 2e-10) are
-// decided, weighted and accumulated here in FP64 and return false.
-template <bool STATS, bool CLAMP>
-__device__ __forceinline__ bool edge_test(const Query &q, float2 na, float2 nb, float2 nc, int ai, int aj, float dir,
-                                          uint32_t tri_id, Acc &acc, float &cr_o, float &e1_o, float &e2_o)
+// m in the closed bounding box of (a, b, c), with the clamp widened by rho.
+template <bool CLAMP, class Q>
+__device__ __forceinline__ bool tri_box_holds(const Q &q, float2 na, float2 nb, float2 nc)
 {
-    if (STATS) acc.tests++;
     float lox = fminf(na.x, fminf(nb.x, nc.x)), hix = fmaxf(na.x, fmaxf(nb.x, nc.x));
     float loy = fminf(na.y, fminf(nb.y, nc.y)), hiy = fmaxf(na.y, fmaxf(nb.y, nc.y));
     if (CLAMP) {
@@ -457,91 +558,62 @@ __device__ __forceinline__ bool edge_test(const Query &q, float2 na, float2 nb, 
         loy -= q.rho;
         hiy += q.rho;
     }
-    if (q.mx < lox || q.mx > hix || q.my < loy || q.my > hiy) return false;
-    float cr = orient(na.x, na.y, nb.x, nb.y, nc.x, nc.y);
-    if (CLAMP && fabsf(cr) < q.jac) {
-        // Eq. 6: the equilateral replacement (vertex k at 90 + 120 k degrees
-        // around the centroid g, radius rho), in vertex-relative form p = m - E0
-        const float gx = (na.x + nb.x + nc.x) * (1.0f / 3.0f), gy = (na.y + nb.y + nc.y) * (1.0f / 3.0f);
-        const float h = 0.8660254f * q.rho;  // E1 - E0 = rho (-sqrt3/2, -3/2), E2 - E0 = rho (sqrt3/2, -3/2)
-        const float2 b = make_float2(-h, -1.5f * q.rho), c = make_float2(h, -1.5f * q.rho);
-        const float2 p = make_float2(q.mx - gx, (q.my - gy) - q.rho);
-        const float ecr = dop(b.x, c.y, b.y, c.x);
-        const float e0 = dop(c.x - b.x, p.y - b.y, c.y - b.y, p.x - b.x);
-        const float e1 = dop(p.x, c.y, p.y, c.x);
-        const float e2 = dop(b.x, p.y, b.y, p.x);
-        cr_o = ecr;  // > 0: counter-clockwise
-        e1_o = e1;
-        e2_o = e2;
-        return e0 >= 0.f && e1 >= 0.f && e2 >= 0.f;
-    }
-    if (fabsf(cr) >= kTinyCross) {
-        float e0 = orient(nb.x, nb.y, nc.x, nc.y, q.mx, q.my);
-        float e1 = orient(nc.x, nc.y, na.x, na.y, q.mx, q.my);
-        float e2 = orient(na.x, na.y, nb.x, nb.y, q.mx, q.my);
-        bool hit = cr > 0.f ? (e0 >= 0.f && e1 >= 0.f && e2 >= 0.f) : (e0 <= 0.f && e1 <= 0.f && e2 <= 0.f);
-        cr_o = cr;
-        e1_o = e1;
-        e2_o = e2;
-        return hit;
-    }
-    test_triangle<STATS>(q, na, nb, nc, ai, aj, dir, tri_id, acc);  // FP64 branch
-    if (STATS) acc.tests--;
-    return false;
+    return !(q.mx < lox || q.mx > hix || q.my < loy || q.my > hiy);
 }
 
-// Hit ring: FP32 hits waiting for their footprint weight, as (cross, e1, e2,
-// tag): tag (i << 15) | (j << 1) | tri for a triangle of quad (i, j), or
-// kClusterTag | (l << 27) | (morton << 1) | tri for a cluster triangle of
-// node (l, morton).
-constexpr int kHitRing = 64;
-constexpr uint32_t kClusterTag = 0x80000000u;
-constexpr uint32_t kClusterMorton = (1u << 26) - 1u;
-
-// All 32 lanes: lane k < cnt weighs hit k of the ring (the tail of test_triangle).
-template <bool STATS>
-__device__ __forceinline__ void drain_hits(const Query &q, int n, int L, const float4 *hits, uint32_t hh, int cnt,
-                                           int lane, Acc &acc)
+// FP32 hit decision of a triangle with |cross| = |cr| >= kTinyCross.
+template <class Q>
+__device__ __forceinline__ bool edges_hold(const Q &q, float2 na, float2 nb, float2 nc, float cr, float &e1, float &e2)
 {
-    if (lane < cnt) {
-        float4 h = hits[(hh + uint32_t(lane)) & (kHitRing - 1)];
-        uint32_t pk = __float_as_uint(h.w);
-        const int tri = int(pk & 1u);
-        int gi, gj, l = 0;
-        if (pk & kClusterTag) {  // cluster triangle of node (l, I, J): uv scale 2^l
-            l = int((pk >> 27) & 15u);
-            uint32_t m = (pk >> 1) & kClusterMorton;
-            gi = int(compact1by1(m)) << l;
-            gj = int(compact1by1(m >> 1)) << l;
-        } else {
-            gi = int(pk >> 15);
-            gj = int((pk >> 1) & 0x3fffu);
-        }
-        const float a = float(1 << l);
-        float inv = 1.0f / h.x;
-        float l1 = h.y * inv, l2 = h.z * inv;
-        float dir = tri ? -a : a;
-        float dx = (float(gi + (tri << l)) - q.x) + dir * l1;
-        float dy = (float(gj + (tri << l)) - q.y) + dir * l2;
-        float qq = qform(q, dx, dy);
-        const float w = kweight(q, dx, qq);
-        if (w != 0.f) {
-            acc_add(acc, w * (a * a) / fabsf(h.x));
-            if (STATS) {
-                acc.hits++;
-                uint32_t id;
-                if (pk & kClusterTag) {
-                    uint32_t S = 1u << (L - l);
-                    id = kClusterTag | (uint32_t(l) << 27) |
-                         (((uint32_t(gj) >> l) * S + (uint32_t(gi) >> l)) << 1) | uint32_t(tri);
-                } else {
-                    id = 2u * (uint32_t(gj) * uint32_t(n - 1) + uint32_t(gi)) + uint32_t(tri);
-                }
-                acc.hash += fmix32(id);
-            }
-        }
+    const float e0 = orient(nb.x, nb.y, nc.x, nc.y, q.mx, q.my);
+    e1 = orient(nc.x, nc.y, na.x, na.y, q.mx, q.my);
+    e2 = orient(na.x, na.y, nb.x, nb.y, q.mx, q.my);
+    return cr > 0.f ? (e0 >= 0.f && e1 >= 0.f && e2 >= 0.f) : (e0 <= 0.f && e1 <= 0.f && e2 <= 0.f);
+}
+
+// Add the contribution of an FP32 hit: cross cr and edge functions e1, e2 (so
+// l1 = e1 / cr, l2 = e2 / cr) of triangle `tri` of the quad, or of the level-l
+// cluster, at (gi, gj); its uv legs are a = 2^l and the Jacobian cr / a^2.
+template <bool STATS, class Q>
+__device__ __forceinline__ void weigh(const Q &q, int gi, int gj, int l, int tri, float cr, float e1, float e2,
+                                      uint32_t id, Acc &acc)
+{
+    const float a = float(1 << l);
+    const float inv = 1.0f / cr;
+    const float dir = tri ? -a : a;
+    const float dx = (float(gi + (tri << l)) - q.x) + dir * (e1 * inv);
+    const float dy = (float(gj + (tri << l)) - q.y) + dir * (e2 * inv);
+    const float qq = qform(q, dx, dy);
+    const float w = kweight(q, dx, qq);
+    if (w == 0.f) return;
+    acc_add(acc, w * (a * a) / fabsf(cr));
+    if (STATS) {
+        acc.hits++;
+        acc.hash += fmix32(id);
     }
 }
+
+// Test triangle `tri` of quad (gi, gj) and add its contribution; tri 0: (u0,
+// u1, u2) with a = (i, j), b = a + (1, 0), c = a + (0, 1); tri 1: (u3, u2, u1)
+// with a = (i+1, j+1), b = a - (1, 0), c = a - (0, 1).
+template <bool STATS, class Q>
+__device__ __forceinline__ void test_triangle(const Q &q, float2 na, float2 nb, float2 nc, int gi, int gj, int tri,
+                                              uint32_t tri_id, Acc &acc)
+{
+    if (STATS) acc.tests++;
+    if (!tri_box_holds<false>(q, na, nb, nc)) return;
+    const float cr = orient(na.x, na.y, nb.x, nb.y, nc.x, nc.y);
+    if (fabsf(cr) >= kTinyCross) {
+        float e1, e2;
+        if (edges_hold(q, na, nb, nc, cr, e1, e2)) weigh<STATS>(q, gi, gj, 0, tri, cr, e1, e2, tri_id, acc);
+        return;
+    }
+    add_tiny<STATS>(tiny_triangle(q, na, nb, nc, gi + tri, gj + tri, tri ? -1.f : 1.f), tri_id, acc);
+}
+
+// Hit fingerprint ids of cluster triangles (stats): this bit, the level from
+// bit 27, the node's row-major index from bit 1 and the triangle.
+constexpr uint32_t kClusterTag = 0x80000000u;
 
 // Lanes 0..24 fetch the 5 x 5 texels of leaf block (a, c) (4 x 4 quads).
 template <int TFMT>
@@ -556,8 +628,8 @@ __device__ __forceinline__ float2 leaf_texel(const MapDesc &d, uint32_t a, uint3
 
 // All 32 lanes: test the 32 triangles of leaf block (a, c) whose texels the
 // lanes hold in tv (lane t: quad t >> 1, triangle t & 1).
-template <bool STATS>
-__device__ __forceinline__ void test_leaf(const MapDesc &d, const Query &q, uint32_t a, uint32_t c, float2 tv,
+template <bool STATS, class Q>
+__device__ __forceinline__ void test_leaf(const MapDesc &d, const Q &q, uint32_t a, uint32_t c, float2 tv,
                                           int lane, Acc &acc)
 {
     const int n = d.n;
@@ -578,81 +650,206 @@ __device__ __forceinline__ void test_leaf(const MapDesc &d, const Query &q, uint
     if (STATS && lane == 0) acc.leaves++;
     if (gi <= n - 2 && gj <= n - 2) {
         uint32_t id = 2u * (uint32_t(gj) * uint32_t(n - 1) + uint32_t(gi)) + uint32_t(tri);
-        test_triangle<STATS>(q, na, nb, nc, tri ? gi + 1 : gi, tri ? gj + 1 : gj, tri ? -1.f : 1.f, id, acc);
+        test_triangle<STATS>(q, na, nb, nc, gi, gj, tri, id, acc);
     }
 }
 
-// Survivor ring: quads whose level-0 box holds m, packed (i << 16) | j.
-constexpr int kRing = 256;
-// Capsule ring: box survivors whose capsule holds m too (at most 31 held
-// over between rounds plus one round's 32).
-constexpr int kCapRing = 64;
-// Leaf queue: up to 7 leaf blocks held over from the last step plus one
-// step's 64 children; cut cluster nodes fill it from the back (entry k at
+// Leaf queue: up to 15 leaf blocks held over from the last step plus one
+// step's children; cut cluster nodes fill it from the back (entry k at
 // kLeafQ - 1 - k), and a step's new leaf blocks and cut nodes number at most
-// 64 together, so the two ends never meet.
-constexpr int kLeafQ = 72;
-// Shared memory per warp: DFS stack, leaf queue, survivor ring, capsule
-// ring, hit ring (a multiple of four words, so the hit ring stays 16-byte
-// aligned).
-constexpr int kWarpSmemWords = kStackCap + kLeafQ + kRing + kCapRing + 4 * kHitRing;
-static_assert((kStackCap + kLeafQ + kRing + kCapRing) % 4 == 0, "hit ring alignment");
+// 4 kPop together, so the two ends never meet.
+constexpr int kLeafQ = 16 + 4 * kPop;
+// Group ring: 2 x 2-quad groups whose box and slab hold m (at most 31 held over
+// plus one pass's 64): Morton index at level 1 (at most 26 bits), kMarked where
+// the group holds a near-singular triangle.
+constexpr int kGroupRing = 128;
+constexpr uint32_t kMarked = 0x80000000u;
+// Triangle ring: triangles that may hold m (at most 31 held over plus 32):
+// (i << 15) | (j << 1) | tri of quad (i, j).
+constexpr int kTriRing = 64;
+// Hit ring, with the cluster cut only: cluster triangles that hold m (few of
+// those tested), waiting to be weighed 32 at a time, as (cross, e1, e2, (index
+// in the box array << 1) | tri); at most 31 held over plus 32.
+constexpr int kHitRing = 64;
+// Shared memory per warp: DFS stack, leaf queue, the rings.
+template <bool CLUSTER>
+constexpr int kWarpSmemWords = kStackCap + kLeafQ + kGroupRing + kTriRing + (CLUSTER ? 4 * kHitRing : 0);
+static_assert((kStackCap + kLeafQ + kGroupRing + kTriRing) % 4 == 0, "hit ring alignment");
 
-// Per-warp leaf state: box-survivor ring, capsule-survivor ring and hit ring
-// with their heads and counts.
+// A warp's shared memory and the rings' heads and counts.
 struct LeafState {
-    uint32_t *ring, *cring;
+    uint32_t *groups, *tris;
     float4 *hits;
-    uint32_t head, chead, hh;
-    int nsq, ncq, nh;
+    uint32_t ghead, thead, hhead;
+    int ng, nt, nh;
 };
 
-// All 32 lanes: lane k tests both triangles of capsule survivor k (k < cnt)
-// of the capsule ring, (u0, u1, u2) and (u3, u2, u1), its four texels loaded together;
-// hits are compacted into the hit ring and weighed 32 at a time.
-template <int TFMT, bool STATS, bool CLAMP>
-__device__ __forceinline__ void test_quads(const MapDesc &d, const Query &q, LeafState &ls, int cnt, int lane,
-                                           Acc &acc)
+// tiny_triangle of triangle `tri` of quad (gi, gj) when its leaf block meets the
+// support (exactly: node_meets lets some by) and m is in the quad's capsule; out of line, so that the rare path costs the common one neither
+// registers nor instruction fetches.
+template <int BFMT, int TFMT, bool CLAMP, class Q>
+__device__ __noinline__ Tiny tiny_in_capsule(const MapDesc &d, const Q &q, int gi, int gj, int tri)
+{
+    if (!node_in_footprint(q, kLeafLevel, uint32_t(gi) >> kLeafLevel, uint32_t(gj) >> kLeafLevel)) return Tiny{0.f, 2};
+    const float2 n0 = texel<TFMT>(d, gi, gj), n1 = texel<TFMT>(d, gi + 1, gj);
+    const float2 n2 = texel<TFMT>(d, gi, gj + 1), n3 = texel<TFMT>(d, gi + 1, gj + 1);
+    if (!capsule_holds<BFMT>(n0, n1, n2, n3, q.mx, q.my, CLAMP ? q.rho : 0.f)) return Tiny{0.f, 2};
+    return tri ? tiny_triangle(q, n3, n2, n1, gi + 1, gj + 1, -1.f) : tiny_triangle(q, n0, n1, n2, gi, gj, 1.f);
+}
+
+// All 32 lanes: lane k < cnt decides triangle k of the triangle ring and adds
+// its contribution.
+template <int BFMT, int TFMT, bool STATS, bool CLAMP, class Q>
+__device__ __forceinline__ void test_tris(const MapDesc &d, const Q &q, const LeafState &ls, int cnt, int lane,
+                                          Acc &acc)
+{
+    if (lane >= cnt) return;
+    const uint32_t pk = ls.tris[(ls.thead + uint32_t(lane)) & (kTriRing - 1)];
+    const int gi = int(pk >> 15), gj = int((pk >> 1) & 0x3fffu), tri = int(pk & 1u);
+    const float2 na = texel<TFMT>(d, gi + tri, gj + tri);
+    const float2 nb = texel<TFMT>(d, gi + 1 - tri, gj + tri), nc = texel<TFMT>(d, gi + tri, gj + 1 - tri);
+    const uint32_t id = 2u * (uint32_t(gj) * uint32_t(d.n - 1) + uint32_t(gi)) + uint32_t(tri);
+    if (STATS) acc.tests++;
+    if (!tri_box_holds<CLAMP>(q, na, nb, nc)) return;
+    const float cr = orient(na.x, na.y, nb.x, nb.y, nc.x, nc.y);
+    if (CLAMP && fabsf(cr) < q.jac) {
+        // Eq. 6: the equilateral replacement (vertex k at 90 + 120 k degrees
+        // around the centroid g, radius rho), in vertex-relative form p = m - E0
+        const float gx = (na.x + nb.x + nc.x) * (1.0f / 3.0f), gy = (na.y + nb.y + nc.y) * (1.0f / 3.0f);
+        const float h = 0.8660254f * q.rho;  // E1 - E0 = rho (-sqrt3/2, -3/2), E2 - E0 = rho (sqrt3/2, -3/2)
+        const float2 b = make_float2(-h, -1.5f * q.rho), c = make_float2(h, -1.5f * q.rho);
+        const float2 p = make_float2(q.mx - gx, (q.my - gy) - q.rho);
+        const float ecr = diff_prod(b.x, c.y, b.y, c.x);  // > 0: counter-clockwise
+        const float e0 = diff_prod(c.x - b.x, p.y - b.y, c.y - b.y, p.x - b.x);
+        const float e1 = diff_prod(p.x, c.y, p.y, c.x);
+        const float e2 = diff_prod(b.x, p.y, b.y, p.x);
+        if (e0 >= 0.f && e1 >= 0.f && e2 >= 0.f) weigh<STATS>(q, gi, gj, 0, tri, ecr, e1, e2, id, acc);
+        return;
+    }
+    if (fabsf(cr) >= kTinyCross) {
+        float e1, e2;
+        if (edges_hold(q, na, nb, nc, cr, e1, e2)) weigh<STATS>(q, gi, gj, 0, tri, cr, e1, e2, id, acc);
+        return;
+    }
+    add_tiny<STATS>(tiny_in_capsule<BFMT, TFMT, CLAMP>(d, q, gi, gj, tri), id, acc);
+}
+
+// The 3 x 3 texels of group (i, j) (i, j even), rows j..j + 2; past the map's
+// last row or column the last one again.  With an even n a row's first two
+// FP32 (FP16) texels are one aligned 16-byte (8-byte) load.
+template <int TFMT>
+__device__ __forceinline__ void group_texels(const MapDesc &d, int i, int j, float2 (&t)[3][3])
+{
+    const int n = d.n;
+    const int i2 = min(i + 2, n - 1);
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+        const int jr = min(j + r, n - 1);
+        const size_t row = size_t(jr) * n;
+        if ((n & 1) == 0) {  // i + 1 <= n - 1
+            if (TFMT == PNDF_TEXEL_F32X2) {
+                const float4 v = __ldg(reinterpret_cast<const float4 *>(reinterpret_cast<const float2 *>(d.texels) + row + i));
+                t[r][0] = make_float2(v.x, v.y);
+                t[r][1] = make_float2(v.z, v.w);
+            } else {
+                const uint2 v = __ldg(reinterpret_cast<const uint2 *>(reinterpret_cast<const __half2 *>(d.texels) + row + i));
+                t[r][0] = __half22float2(*reinterpret_cast<const __half2 *>(&v.x));
+                t[r][1] = __half22float2(*reinterpret_cast<const __half2 *>(&v.y));
+            }
+        } else {
+            t[r][0] = texel<TFMT>(d, i, jr);
+            t[r][1] = texel<TFMT>(d, min(i + 1, n - 1), jr);
+        }
+        t[r][2] = texel<TFMT>(d, i2, jr);
+    }
+}
+
+// All 32 lanes: lane k < cnt takes group k of the group ring and finds the
+// triangles of its four quads that may hold m.  With d_u = n_u - m, edge u -> v
+// has m on its left when d_u x d_v > 0, so the group's 16 edges (12 sides, 4
+// diagonals), two operations each, decide all eight triangles.  A triangle is
+// dropped only when two of its edges differ in sign by more than `eps`; with M
+// the largest |d| component, the rounding of these edge functions (2^-21 M^2)
+// and of the exact test's (2^-21 M^2: differences of at most 2 M, each
+// relative to 2^-24) add up to 2^-20 M^2, and eps is four times that.  The
+// survivors (few beside the hits) are listed and decided 32 at a time.
+template <int BFMT, int TFMT, bool STATS, bool CLAMP, class Q>
+__device__ __forceinline__ void test_groups(const MapDesc &d, const Q &q, LeafState &ls, int cnt, int lane, Acc &acc)
 {
     const unsigned lt = (1u << lane) - 1u;
-    bool h0 = false, h1 = false;
-    float4 v0 = make_float4(0.f, 0.f, 0.f, 0.f), v1 = v0;
+    uint32_t cand = 0, base = 0;
     if (lane < cnt) {
-        uint32_t pk = ls.cring[(ls.chead + uint32_t(lane)) & (kCapRing - 1)];
-        int gi = int(pk >> 16), gj = int(pk & 0xffffu);
-        float2 n0 = texel<TFMT>(d, gi, gj), n1 = texel<TFMT>(d, gi + 1, gj);
-        float2 n2 = texel<TFMT>(d, gi, gj + 1), n3 = texel<TFMT>(d, gi + 1, gj + 1);
-        uint32_t id = 2u * (uint32_t(gj) * uint32_t(d.n - 1) + uint32_t(gi));
-        uint32_t hp = (uint32_t(gi) << 15) | (uint32_t(gj) << 1);
-        float cr, e1, e2;
-        h0 = edge_test<STATS, CLAMP>(q, n0, n1, n2, gi, gj, 1.f, id, acc, cr, e1, e2);
-        if (h0) v0 = make_float4(cr, e1, e2, __uint_as_float(hp));
-        h1 = edge_test<STATS, CLAMP>(q, n3, n2, n1, gi + 1, gj + 1, -1.f, id + 1u, acc, cr, e1, e2);
-        if (h1) v1 = make_float4(cr, e1, e2, __uint_as_float(hp | 1u));
-    }
+        const uint32_t g = ls.groups[(ls.ghead + uint32_t(lane)) & (kGroupRing - 1)];
+        const uint32_t m = g & ~kMarked;
+        const int i = int(compact1by1(m)) * 2, j = int(compact1by1(m >> 1)) * 2;
+        base = (uint32_t(i) << 15) | (uint32_t(j) << 1);
+        float2 t[3][3];
+        group_texels<TFMT>(d, i, j, t);
+        float M = 0.f;
 #pragma unroll
-    for (int t = 0; t < 2; ++t) {  // at most 31 + 32 entries queue between drains
-        bool h = t ? h1 : h0;
-        unsigned m = __ballot_sync(kFull, h);
-        if (h) ls.hits[(ls.hh + uint32_t(ls.nh) + __popc(m & lt)) & (kHitRing - 1)] = t ? v1 : v0;
-        ls.nh += __popc(m);
+        for (int r = 0; r < 3; ++r)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                t[r][c].x -= q.mx;
+                t[r][c].y -= q.my;
+                M = fmaxf(M, fmaxf(fabsf(t[r][c].x), fabsf(t[r][c].y)));
+            }
+        const float eps = M * M * 0x1p-18f;
+        auto edge = [](const float2 &u, const float2 &v) { return fmaf(u.x, v.y, -(u.y * v.x)); };
+        float H[3][2], V[2][3];
+#pragma unroll
+        for (int r = 0; r < 3; ++r)
+#pragma unroll
+            for (int c = 0; c < 2; ++c) H[r][c] = edge(t[r][c], t[r][c + 1]);
+#pragma unroll
+        for (int r = 0; r < 2; ++r)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) V[r][c] = edge(t[r][c], t[r + 1][c]);
+        auto may = [&](float a, float b, float c) {
+            const bool out = fminf(a, fminf(b, c)) < -eps && fmaxf(a, fmaxf(b, c)) > eps;
+            // with the clamp, also whatever its cross (the edges' sum) may send to the replacement
+            return !out || (CLAMP && !(fabsf(a + b + c) >= q.jac + eps));
+        };
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int r = k >> 1, c = k & 1;
+            const float dg = edge(t[r][c + 1], t[r + 1][c]);
+            cand |= uint32_t(may(H[r][c], dg, -V[r][c])) << (2 * k);              // u0 u1 u2
+            cand |= uint32_t(may(-H[r + 1][c], -dg, V[r][c + 1])) << (2 * k + 1);  // u3 u2 u1
+        }
+        if (g & kMarked) cand = 0xffu;
+        // quads past the map's last row or column of quads do not exist
+        if (i + 1 > d.n - 2) cand &= 0x33u;
+        if (j + 1 > d.n - 2) cand &= 0x0fu;
+        if (STATS) acc.quads += 4;
+    }
+    unsigned m = __ballot_sync(kFull, cand != 0u);
+    while (m) {
+        if (cand) {
+            const uint32_t b = uint32_t(__ffs(int(cand)) - 1);
+            cand &= cand - 1u;
+            ls.tris[(ls.thead + uint32_t(ls.nt) + __popc(m & lt)) & (kTriRing - 1)] =
+                base + ((b & 2u) << 14) + ((b & 4u) >> 1) + (b & 1u);
+        }
+        ls.nt += __popc(m);
         __syncwarp();
-        if (ls.nh >= 32) {
-            drain_hits<STATS>(q, d.n, d.L, ls.hits, ls.hh, 32, lane, acc);
-            ls.hh += 32;
-            ls.nh -= 32;
+        if (ls.nt >= 32) {
+            test_tris<BFMT, TFMT, STATS, CLAMP>(d, q, ls, 32, lane, acc);
+            ls.thead += 32;
+            ls.nt -= 32;
             __syncwarp();
         }
+        m = __ballot_sync(kFull, cand != 0u);
     }
 }
 
 // Cluster triangle test (Sec. 4.2) in vertex-relative form: p = m - A,
-// b = B - A, c = C - A.  Same rule as edge_test (closed bounding box, edge
+// b = B - A, c = C - A.  Same rule as for a fine triangle (closed bounding box, edge
 // functions sign-consistent with the orientation); the Jacobian of the
 // cluster map is cross / 4^l, applied when the hit is weighed.  Triangles
 // with FP32 |cross| < 2e-10 are decided and weighed here in FP64.
-template <bool STATS>
-__device__ __forceinline__ bool cluster_edge_test(const Query &q, float2 p, float2 b, float2 c, int l, int ai,
+template <bool STATS, class Q>
+__device__ __forceinline__ bool cluster_edge_test(const Q &q, float2 p, float2 b, float2 c, int l, int ai,
                                                   int aj, float dir, uint32_t id, Acc &acc, float &cr_o, float &e1_o,
                                                   float &e2_o)
 {
@@ -660,11 +857,11 @@ __device__ __forceinline__ bool cluster_edge_test(const Query &q, float2 p, floa
     if (p.x < fminf(0.f, fminf(b.x, c.x)) || p.x > fmaxf(0.f, fmaxf(b.x, c.x)) ||
         p.y < fminf(0.f, fminf(b.y, c.y)) || p.y > fmaxf(0.f, fmaxf(b.y, c.y)))
         return false;
-    float cr = dop(b.x, c.y, b.y, c.x);
+    float cr = diff_prod(b.x, c.y, b.y, c.x);
     if (fabsf(cr) >= kTinyCross) {
-        float e0 = dop(c.x - b.x, p.y - b.y, c.y - b.y, p.x - b.x);
-        float e1 = dop(p.x, c.y, p.y, c.x);
-        float e2 = dop(b.x, p.y, b.y, p.x);
+        float e0 = diff_prod(c.x - b.x, p.y - b.y, c.y - b.y, p.x - b.x);
+        float e1 = diff_prod(p.x, c.y, p.y, c.x);
+        float e2 = diff_prod(b.x, p.y, b.y, p.x);
         bool hit = cr > 0.f ? (e0 >= 0.f && e1 >= 0.f && e2 >= 0.f) : (e0 <= 0.f && e1 <= 0.f && e2 <= 0.f);
         cr_o = cr;
         e1_o = e1;
@@ -699,182 +896,110 @@ __device__ __forceinline__ bool cluster_edge_test(const Query &q, float2 p, floa
     return false;
 }
 
+// All 32 lanes: lane k < cnt weighs hit k of the hit ring.
+template <bool STATS, class Q>
+__device__ __forceinline__ void weigh_clusters(const MapDesc &d, const Q &q, const LeafState &ls, int cnt, int lane,
+                                               Acc &acc)
+{
+    if (lane >= cnt) return;
+    const float4 h = ls.hits[(ls.hhead + uint32_t(lane)) & (kHitRing - 1)];
+    const uint32_t k = __float_as_uint(h.w) >> 1;
+    const int tri = int(__float_as_uint(h.w) & 1u), l = node_level(k, d.L);
+    const uint32_t m = k - node_index(d.L, l, 0);
+    const uint32_t I = compact1by1(m), J = compact1by1(m >> 1);
+    const uint32_t id = kClusterTag | (uint32_t(l) << 27) | (((J << (d.L - l)) + I) << 1) | uint32_t(tri);
+    weigh<STATS>(q, int(I << l), int(J << l), l, tri, h.x, h.y, h.z, id, acc);
+}
+
 // All 32 lanes: lane k < cnt tests the two cluster triangles of the cut node
-// in last[-k] (level, Morton): lower (c00, c10, c01) at uv (O, O + (a, 0),
-// O + (0, a)), upper (c11, c01, c10) at (O + (a, a), O + (0, a), O + (a, 0)),
-// a = 2^l; hits join the hit ring.
-template <bool STATS>
-__device__ __forceinline__ void test_clusters(const MapDesc &d, const ClusterDesc &cd, const Query &q,
+// in last[-k] (index in the box array): lower (c00, c10, c01) at uv (O, O + (a,
+// 0), O + (0, a)), upper (c11, c01, c10) at (O + (a, a), O + (0, a), O + (a,
+// 0)), a = 2^l; hits join the hit ring.
+template <bool STATS, class Q>
+__device__ __forceinline__ void test_clusters(const MapDesc &d, const ClusterDesc &cd, const Q &q,
                                               const uint32_t *last, int cnt, LeafState &ls, int lane, Acc &acc)
 {
     const unsigned lt = (1u << lane) - 1u;
     bool h0 = false, h1 = false;
     float4 v0 = make_float4(0.f, 0.f, 0.f, 0.f), v1 = v0;
     if (lane < cnt) {
-        uint32_t ent = last[-lane];
-        int l = int(ent >> 28);
-        uint32_t m = ent & kMortonMask;
-        const float4 *rec = cd.cl[l] + 2 * size_t(m);
+        const uint32_t k = last[-lane];
+        const int l = node_level(k, d.L);
+        const uint32_t m = k - node_index(d.L, l, 0);
+        const float4 *rec = cd.cl + 2 * size_t(k);
         float4 r0 = __ldg(rec), r1 = __ldg(rec + 1);
         int ox = int(compact1by1(m)) << l, oy = int(compact1by1(m >> 1)) << l;
         int a = 1 << l;
         float2 p = make_float2(q.mx - r0.x, q.my - r0.y);
         float2 d10 = make_float2(r0.z, r0.w), d01 = make_float2(r1.x, r1.y), d11 = make_float2(r1.z, r1.w);
-        uint32_t tag = kClusterTag | (uint32_t(l) << 27) | (m << 1);
         // hit fingerprint id (stats): row-major node index at its level
         uint32_t id = kClusterTag | (uint32_t(l) << 27) |
                       (((uint32_t(oy >> l) << (d.L - l)) + uint32_t(ox >> l)) << 1);
         float cr, e1, e2;
         if (STATS) acc.clusters++;
         h0 = cluster_edge_test<STATS>(q, p, d10, d01, l, ox, oy, float(a), id, acc, cr, e1, e2);
-        if (h0) v0 = make_float4(cr, e1, e2, __uint_as_float(tag));
+        if (h0) v0 = make_float4(cr, e1, e2, __uint_as_float(k << 1));
         float2 pu = make_float2(p.x - d11.x, p.y - d11.y);
         float2 bu = make_float2(d01.x - d11.x, d01.y - d11.y), cu = make_float2(d10.x - d11.x, d10.y - d11.y);
         h1 = cluster_edge_test<STATS>(q, pu, bu, cu, l, ox + a, oy + a, -float(a), id | 1u, acc, cr, e1, e2);
-        if (h1) v1 = make_float4(cr, e1, e2, __uint_as_float(tag | 1u));
+        if (h1) v1 = make_float4(cr, e1, e2, __uint_as_float((k << 1) | 1u));
     }
 #pragma unroll
     for (int t = 0; t < 2; ++t) {
         bool h = t ? h1 : h0;
         unsigned mk = __ballot_sync(kFull, h);
-        if (h) ls.hits[(ls.hh + uint32_t(ls.nh) + __popc(mk & lt)) & (kHitRing - 1)] = t ? v1 : v0;
+        if (h) ls.hits[(ls.hhead + uint32_t(ls.nh) + __popc(mk & lt)) & (kHitRing - 1)] = t ? v1 : v0;
         ls.nh += __popc(mk);
         __syncwarp();
         if (ls.nh >= 32) {
-            drain_hits<STATS>(q, d.n, d.L, ls.hits, ls.hh, 32, lane, acc);
-            ls.hh += 32;
+            weigh_clusters<STATS>(d, q, ls, 32, lane, acc);
+            ls.hhead += 32;
             ls.nh -= 32;
             __syncwarp();
         }
     }
 }
 
-// Four level-0 boxes (Morton-consecutive quads) in one 32-byte (FP16) or
-// 64-byte (FP32) load; returns bit u set when box u holds m.
-template <int BFMT, bool CLAMP>
-__device__ __forceinline__ unsigned quad_boxes_hold(const MapDesc &d, uint32_t first, const Query &q)
-{
-    const float mx = q.mx, my = q.my, rho = CLAMP ? q.rho : 0.f;
-    unsigned bits = 0;
-    if (BFMT == PNDF_BOUNDS_F32) {
-        const float4 *p = reinterpret_cast<const float4 *>(d.lv[0]) + first;
-        float4 b[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) b[u] = __ldg(p + u);
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-            bits |= CLAMP ? unsigned(mx >= b[u].x - rho && mx <= b[u].z + rho && my >= b[u].y - rho &&
-                                     my <= b[u].w + rho) << u
-                          : unsigned(mx >= b[u].x && mx <= b[u].z && my >= b[u].y && my <= b[u].w) << u;
-    } else {
-        const uint4 *p = reinterpret_cast<const uint4 *>(reinterpret_cast<const uint2 *>(d.lv[0]) + first);
-        uint4 v0 = __ldg(p), v1 = __ldg(p + 1);
-        uint32_t w[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            float2 lo = __half22float2(*reinterpret_cast<__half2 *>(&w[2 * u]));
-            float2 hi = __half22float2(*reinterpret_cast<__half2 *>(&w[2 * u + 1]));
-            bits |= CLAMP ? unsigned(mx >= lo.x - rho && mx <= hi.x + rho && my >= lo.y - rho && my <= hi.y + rho) << u
-                          : unsigned(mx >= lo.x && mx <= hi.x && my >= lo.y && my <= hi.y) << u;
-        }
-    }
-    return bits;
-}
-
-// A stored node box decoded to (s_min, t_min, s_max, t_max).
-template <int BFMT>
-__device__ __forceinline__ float4 box_floats(const uint4 &v)
-{
-    if (BFMT == PNDF_BOUNDS_F32)
-        return make_float4(__uint_as_float(v.x), __uint_as_float(v.y), __uint_as_float(v.z), __uint_as_float(v.w));
-    float2 lo = __half22float2(*reinterpret_cast<const __half2 *>(&v.x));
-    float2 hi = __half22float2(*reinterpret_cast<const __half2 *>(&v.y));
-    return make_float4(lo.x, lo.y, hi.x, hi.y);
-}
-
-// All 32 lanes: lane k takes box survivors k and k + 32 of the ring (those
-// below cnt <= 64; both quads' boxes and capsule codes are loaded before
-// either is used), tests m against each quad's capsule, and the survivors
-// are compacted into the capsule ring, whose quads are tested 32 at a time.
-template <int BFMT, int TFMT, bool STATS, bool CLAMP>
-__device__ __forceinline__ void capsule_round(const MapDesc &d, const Query &q, LeafState &ls, int cnt, int lane,
-                                              Acc &acc)
-{
-    const unsigned lt = (1u << lane) - 1u;
-    bool pass[2] = {false, false};
-    uint32_t pk[2] = {0u, 0u};
-    uint4 bx[2];
-    uint2 code[2];
-#pragma unroll
-    for (int r = 0; r < 2; ++r)
-        if (lane + 32 * r < cnt) {
-            pk[r] = ls.ring[(ls.head + uint32_t(lane + 32 * r)) & (kRing - 1)];
-            const uint32_t mq = morton2(pk[r] >> 16, pk[r] & 0xffffu);
-            bx[r] = node_box<BFMT>(d, 0, mq);
-            code[r] = __ldg(d.qcap + mq);
-        }
-#pragma unroll
-    for (int r = 0; r < 2; ++r)
-        if (lane + 32 * r < cnt) {
-            const float4 b = box_floats<BFMT>(bx[r]);
-            const Capsule c = decode_capsule(b.x, b.y, b.z, b.w, code[r]);
-            pass[r] = capsule_holds(c, q.mx, q.my, CLAMP ? c.w + q.rho : c.w);
-        }
-#pragma unroll
-    for (int r = 0; r < 2; ++r) {
-        const unsigned m = __ballot_sync(kFull, pass[r]);
-        if (pass[r]) ls.cring[(ls.chead + uint32_t(ls.ncq) + __popc(m & lt)) & (kCapRing - 1)] = pk[r];
-        ls.ncq += __popc(m);
-        __syncwarp();
-        if (ls.ncq >= 32) {
-            test_quads<TFMT, STATS, CLAMP>(d, q, ls, 32, lane, acc);
-            ls.chead += 32;
-            ls.ncq -= 32;
-            __syncwarp();
-        }
-    }
-}
-
-// All 32 lanes: filter the queued leaf blocks' quads by their level-0 boxes
-// (lane t: quads 4 (t & 3) .. 4 (t & 3) + 3 of block p + (t >> 2), eight
-// blocks per pass), compact the survivors into the ring with ballot/popc and
-// test them 32 quads (64 triangles) at a time.
-template <int BFMT, int TFMT, bool STATS, bool CLAMP>
-__device__ __forceinline__ void process_leaves(const MapDesc &d, const Query &q, const uint32_t *lq, int nleaf,
+// All 32 lanes: filter the queued leaf blocks' 2 x 2-quad groups by box and
+// slab (lane t: group t & 3 of blocks p + (t >> 2) and p + 8 + (t >> 2), sixteen
+// blocks per pass, both records in flight), compact the survivors into the
+// ring and test them 32 groups (256 triangles) at a time.
+template <int BFMT, int TFMT, bool STATS, bool CLAMP, class Q>
+__device__ __forceinline__ void process_leaves(const MapDesc &d, const Q &q, const uint32_t *lq, int nleaf,
                                                LeafState &ls, int lane, Acc &acc)
 {
     const unsigned lt = (1u << lane) - 1u;
-    for (int p = 0; p < nleaf; p += 8) {
-        const int blk = p + (lane >> 2);
-        unsigned bits = 0;
-        uint32_t base = 0;
-        if (blk < nleaf) {
-            uint32_t m = lq[blk] & kMortonMask;
-            // the lane's four quads are the 2 x 2 quad group (lane & 3) of the
-            // block (Morton order): (i0 + u & 1, j0 + u >> 1) for u = 0..3
-            const uint32_t i0 = compact1by1(m) * kLeafQuads + ((uint32_t(lane) & 1u) << 1);
-            const uint32_t j0 = compact1by1(m >> 1) * kLeafQuads + (uint32_t(lane) & 2u);
-            base = (i0 << 16) | j0;
-            bits = quad_boxes_hold<BFMT, CLAMP>(d, (m << 4) | (uint32_t(lane & 3) << 2), q);
-            if (STATS) {
-                acc.quads += 4;
-                if ((lane & 3) == 0) acc.leaves++;
+    const uint32_t morton_mask = (1u << (2 * (d.L - kLeafLevel))) - 1u;
+    for (int p = 0; p < nleaf; p += 16) {
+        uint32_t g[2];
+        uint4 rec[2];
+        bool pass[2];
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            const int blk = p + 8 * r + (lane >> 2);
+            pass[r] = blk < nleaf;
+            if (pass[r]) {
+                g[r] = ((lq[blk] & morton_mask) << 2) | uint32_t(lane & 3);
+                rec[r] = __ldg(d.groups + g[r]);
+                if (STATS && (lane & 3) == 0) acc.leaves++;
             }
         }
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            bool pass = (bits >> u) & 1u;
-            unsigned m = __ballot_sync(kFull, pass);
-            if (pass)
-                ls.ring[(ls.head + uint32_t(ls.nsq) + __popc(m & lt)) & (kRing - 1)] =
-                    base + ((uint32_t(u) & 1u) << 16) + (uint32_t(u) >> 1);
-            ls.nsq += __popc(m);
+        for (int r = 0; r < 2; ++r) {
+            if (pass[r]) {
+                pass[r] = half_box_holds<CLAMP>(rec[r].x, rec[r].y, q) &&
+                          slab_holds(rec[r].z, rec[r].w, q.mx, q.my, slab_slack<CLAMP>(q));
+                if (slab_marked(rec[r].w)) g[r] |= kMarked;
+            }
+            const unsigned m = __ballot_sync(kFull, pass[r]);
+            if (pass[r]) ls.groups[(ls.ghead + uint32_t(ls.ng) + __popc(m & lt)) & (kGroupRing - 1)] = g[r];
+            ls.ng += __popc(m);
         }
         __syncwarp();
-        while (ls.nsq >= 64) {
-            capsule_round<BFMT, TFMT, STATS, CLAMP>(d, q, ls, 64, lane, acc);
-            ls.head += 64;
-            ls.nsq -= 64;
+        while (ls.ng >= 32) {
+            test_groups<BFMT, TFMT, STATS, CLAMP>(d, q, ls, 32, lane, acc);
+            ls.ghead += 32;
+            ls.ng -= 32;
             __syncwarp();
         }
     }
@@ -896,7 +1021,8 @@ __device__ __forceinline__ void node_range(float x, float r, float sz, int S, in
     a1 = int(f1);
 }
 
-__device__ __forceinline__ int entry_level(const Query &q, int L)
+template <class Q>
+__device__ __forceinline__ int entry_level(const Q &q, int L)
 {
     float r = fmaxf(q.rx, q.ry);
     int l = kLeafLevel;
@@ -911,53 +1037,74 @@ __device__ __forceinline__ int entry_level(const Query &q, int L)
 // children's), so a leaf block is reached from any level above it exactly
 // when every node test on its path passes: the hit set, and with the exact
 // sum the result, does not depend on the level the descent starts from.
-template <int BFMT, int TFMT, bool STATS, bool CLUSTER, bool CLAMP>
-__device__ __forceinline__ void eval_range(const MapDesc &d, const ClusterDesc &cd, const Query &q, int e, int a0,
-                                           int a1, int c0, int c1, int lane, uint32_t *stk, uint32_t *lq,
-                                           uint32_t *ring, float4 *hits, Acc &acc)
+template <int BFMT, int TFMT, bool STATS, bool CLUSTER, bool CLAMP, class Q>
+__device__ __forceinline__ void eval_range(const MapDesc &d, const ClusterDesc &cd, const Q &q, int e, int a0,
+                                           int a1, int c0, int c1, int lane, uint32_t *smem, Acc &acc)
 {
+    uint32_t *stk = smem, *lq = smem + kStackCap;
     int top = 0, nleaf = 0, ncl = 0;
     const unsigned lt = (1u << lane) - 1u;
+    const uint32_t leaf0 = node_index(d.L, kLeafLevel, 0);  // from here on a node is a leaf block
+    // With the cut, a slab above the leaf level says nothing: it holds the
+    // texels' normals, but a descendant may be cut and its cluster lie outside.
+    // Below an uncut leaf block only exact triangles follow.
+    auto in_slab = [&](const Node<BFMT> &n, uint32_t k) {
+        return (CLUSTER && k < leaf0) || node_slab_holds<BFMT, CLAMP>(n, q);
+    };
+    // the cut of Sec. 4.2, e <= r_x r_y tau, of a node that holds m; a node is cut
+    // only if its uv box meets the support exactly (node_meets lets some by),
+    // else nothing below it contributes
+    auto cut_here = [&](uint32_t k, float ev, bool ins, bool &pass) {
+        if (STATS) acc.cchecks++;
+        if (!(ev <= q.theta)) return false;
+        if (!ins) {
+            const int l = node_level(k, d.L);
+            const uint32_t m = k - node_index(d.L, l, 0);
+            pass = node_in_footprint(q, l, compact1by1(m), compact1by1(m >> 1));
+        }
+        return pass;
+    };
+    // node k, child of a parent that was not inside: meets the support?  (and is it inside?)
+    auto in_footprint = [&](uint32_t k, bool &ins) {
+        if (ins) return true;
+        const int l = node_level(k, d.L);
+        const uint32_t m = k - node_index(d.L, l, 0);
+        return node_meets(q, l, compact1by1(m), compact1by1(m >> 1), ins);
+    };
     // entry nodes: at most 4 x 4
     {
         int a = a0 + (lane & 3), c = c0 + (lane >> 2);
         bool valid = lane < 16 && a <= a1 && c <= c1;
-        bool pass = valid && node_test<BFMT, CLAMP>(d, q, e, a, c);
-        bool inside = pass && node_inside(q, e, a, c);
+        const uint32_t k = node_index(d.L, e, valid ? morton2(a, c) : 0u);
+        const Node<BFMT> n = load_node<BFMT>(d, k);
+        bool inside = false;
+        bool pass = valid && node_meets(q, e, a, c, inside) && node_box_holds<BFMT, CLAMP>(n, q);
         bool cut = false;
         if (STATS) acc.nodes += valid ? 1u : 0u;
-        if (CLUSTER && pass) {  // the cut of Sec. 4.2: e <= r_x r_y tau
-            cut = __ldg(cd.ce[e] + morton2(a, c)) <= q.theta;
-            if (STATS) acc.cchecks++;
-        }
-        unsigned m = __ballot_sync(kFull, pass && !cut);
+        if (CLUSTER && pass) cut = cut_here(k, __ldg(cd.ce + k), inside, pass);
+        if (pass && !cut) pass = in_slab(n, k);
+        unsigned mp = __ballot_sync(kFull, pass && !cut);
         unsigned mc = __ballot_sync(kFull, cut);
-        if (pass && !cut) {
-            int pos = __popc(m & lt);
-            uint32_t ent = pack(e, inside, morton2(a, c));
-            if (e == kLeafLevel)
-                lq[pos] = ent;
-            else
-                stk[pos] = ent;
-        }
-        if (CLUSTER && cut) lq[kLeafQ - 1 - __popc(mc & lt)] = pack(e, false, morton2(a, c));
+        if (pass && !cut) (e == kLeafLevel ? lq : stk)[__popc(mp & lt)] = k | (inside ? kInside : 0u);
+        if (CLUSTER && cut) lq[kLeafQ - 1 - __popc(mc & lt)] = k;
         if (e == kLeafLevel)
-            nleaf = __popc(m);
+            nleaf = __popc(mp);
         else
-            top = __popc(m);
+            top = __popc(mp);
         ncl = __popc(mc);
         __syncwarp();
     }
     bool overflow = false;
-    LeafState ls{ring, ring + kRing, hits, 0u, 0u, 0u, 0, 0, 0};
+    uint32_t *rings = lq + kLeafQ;
+    LeafState ls{rings, rings + kGroupRing, reinterpret_cast<float4 *>(rings + kGroupRing + kTriRing), 0u, 0u, 0u, 0, 0, 0};
     while (true) {
-        // leaf blocks are filtered eight to a pass (four lanes each): while
-        // the stack still holds nodes only whole passes run, and the rest
-        // (fewer than 8) waits at the front of the queue for the next step
-        const int nrun = top == 0 ? nleaf : (nleaf & ~7);
+        // leaf blocks are filtered sixteen to a pass (four lanes each, twice):
+        // while the stack still holds nodes only whole passes run, and the rest
+        // (fewer than 16) waits at the front of the queue for the next step
+        const int nrun = top == 0 ? nleaf : (nleaf & ~15);
         process_leaves<BFMT, TFMT, STATS, CLAMP>(d, q, lq, nrun, ls, lane, acc);
         if (nrun > 0 && nrun < nleaf) {
-            const int rest = nleaf - nrun;  // < 8 <= nrun: source and target do not overlap
+            const int rest = nleaf - nrun;  // < 16 <= nrun: source and target do not overlap
             uint32_t v = lane < rest ? lq[nrun + lane] : 0u;
             if (lane < rest) lq[lane] = v;
             __syncwarp();
@@ -972,65 +1119,61 @@ __device__ __forceinline__ void eval_range(const MapDesc &d, const ClusterDesc &
             ncl = 0;
         }
         if (top == 0) break;
-        // pop up to 16 nodes; lane k tests child (k & 3) of popped nodes
-        // (k >> 2) and (k >> 2) + 8, so two box loads per lane are in flight
-        int npop = min(top, 16);
+        // pop up to kPop nodes; lane k tests child (k & 3) of popped nodes
+        // (k >> 2) + 8 r, so kPer loads per lane are in flight
+        int npop = min(top, kPop);
         top -= npop;
-        bool pass[2], ins[2], cut[2] = {false, false};
-        int cl[2];
-        uint32_t cm[2];
-        uint4 bx[2];
-        float ev[2];
+        bool pass[kPer], ins[kPer], cut[kPer];
+        uint32_t ck[kPer];
+        Node<BFMT> nd[kPer];
+        float ev[kPer];
 #pragma unroll
-        for (int r = 0; r < 2; ++r) {
+        for (int r = 0; r < kPer; ++r) {
             int slot = (lane >> 2) + 8 * r;
             uint32_t ent = slot < npop ? stk[top + slot] : 0u;
-            cl[r] = int(ent >> 28) - 1;
-            cm[r] = ((ent & kMortonMask) << 2) | uint32_t(lane & 3);
-            ins[r] = (ent >> 27) & 1u;
+            ck[r] = (ent << 2) | uint32_t(lane & 3);  // shifts "inside" out
+            ins[r] = (ent & kInside) != 0u;
             pass[r] = slot < npop;
+            cut[r] = false;
             if (STATS && slot < npop) acc.nodes++;
         }
-        // both box loads issue before the uv tests, which hide their latency
-        // (895.9 ms against 915.2 ms per 4M-query flake step, same bits)
+        // All loads are in flight before either is tested; the uv box,
+        // the costly test, only for the few children that hold m (98 ms against
+        // 105 ms with the uv box first, 1M flake queries).
 #pragma unroll
-        for (int r = 0; r < 2; ++r)
+        for (int r = 0; r < kPer; ++r)
             if (pass[r]) {
-                bx[r] = node_box<BFMT>(d, cl[r], cm[r]);
-                if (CLUSTER) ev[r] = __ldg(cd.ce[cl[r]] + cm[r]);
+                nd[r] = load_node<BFMT>(d, ck[r]);
+                if (CLUSTER) ev[r] = __ldg(cd.ce + ck[r]);
             }
 #pragma unroll
-        for (int r = 0; r < 2; ++r)
-            if (pass[r] && !ins[r]) {
-                // parent straddles the ellipse: test this child's uv box
-                uint32_t a = compact1by1(cm[r]), c = compact1by1(cm[r] >> 1);
-                pass[r] = node_in_footprint(q, cl[r], a, c);
-                ins[r] = pass[r] && node_inside(q, cl[r], a, c);
-            }
-#pragma unroll
-        for (int r = 0; r < 2; ++r) {
-            pass[r] = pass[r] && stored_box_holds<BFMT, CLAMP>(bx[r], q);
-            if (CLUSTER && pass[r]) {  // the cut of Sec. 4.2: e <= r_x r_y tau
-                cut[r] = ev[r] <= q.theta;
-                if (STATS) acc.cchecks++;
+        for (int r = 0; r < kPer; ++r) {
+            pass[r] = pass[r] && node_box_holds<BFMT, CLAMP>(nd[r], q);
+            if (CLUSTER) {
+                pass[r] = pass[r] && in_footprint(ck[r], ins[r]);
+                if (pass[r]) cut[r] = cut_here(ck[r], ev[r], ins[r], pass[r]);
+                if (pass[r] && !cut[r]) pass[r] = in_slab(nd[r], ck[r]);
+            } else {
+                pass[r] = pass[r] && in_slab(nd[r], ck[r]) && in_footprint(ck[r], ins[r]);
             }
         }
         __syncwarp();
 #pragma unroll
-        for (int r = 0; r < 2; ++r) {
-            bool to_leaf = pass[r] && !cut[r] && cl[r] == kLeafLevel;
-            bool to_stack = pass[r] && !cut[r] && cl[r] > kLeafLevel;
+        for (int r = 0; r < kPer; ++r) {
+            const bool keep = pass[r] && !cut[r];
+            bool to_leaf = keep && ck[r] >= leaf0;
+            bool to_stack = keep && ck[r] < leaf0;
             unsigned ml = __ballot_sync(kFull, to_leaf);
             unsigned ms = __ballot_sync(kFull, to_stack);
             if (CLUSTER) {
                 unsigned mc = __ballot_sync(kFull, cut[r]);
-                if (cut[r]) lq[kLeafQ - 1 - ncl - __popc(mc & lt)] = pack(cl[r], false, cm[r]);
+                if (cut[r]) lq[kLeafQ - 1 - ncl - __popc(mc & lt)] = ck[r];
                 ncl += __popc(mc);
             }
-            if (to_leaf) lq[nleaf + __popc(ml & lt)] = pack(cl[r], ins[r], cm[r]);
+            if (to_leaf) lq[nleaf + __popc(ml & lt)] = ck[r];
             if (to_stack) {
                 int pos = top + __popc(ms & lt);
-                if (pos < kStackCap) stk[pos] = pack(cl[r], ins[r], cm[r]);
+                if (pos < kStackCap) stk[pos] = ck[r] | (ins[r] ? kInside : 0u);
             }
             nleaf += __popc(ml);
             top += __popc(ms);
@@ -1041,9 +1184,9 @@ __device__ __forceinline__ void eval_range(const MapDesc &d, const ClusterDesc &
         }
         __syncwarp();
     }
-    if (ls.nsq > 0) capsule_round<BFMT, TFMT, STATS, CLAMP>(d, q, ls, ls.nsq, lane, acc);  // nsq < 64 here
-    if (ls.ncq > 0) test_quads<TFMT, STATS, CLAMP>(d, q, ls, ls.ncq, lane, acc);  // ncq < 32 here
-    if (ls.nh > 0) drain_hits<STATS>(q, d.n, d.L, ls.hits, ls.hh, ls.nh, lane, acc);  // nh < 32 here
+    if (ls.ng > 0) test_groups<BFMT, TFMT, STATS, CLAMP>(d, q, ls, ls.ng, lane, acc);  // ng < 32 here
+    if (ls.nt > 0) test_tris<BFMT, TFMT, STATS, CLAMP>(d, q, ls, ls.nt, lane, acc);    // nt < 32 here
+    if (CLUSTER && ls.nh > 0) weigh_clusters<STATS>(d, q, ls, ls.nh, lane, acc);  // nh < 32 here
     if (overflow) acc.flags |= PNDF_QF_OVERFLOW;
 }
 
@@ -1083,13 +1226,19 @@ __device__ __forceinline__ void warp_total(Acc &acc, unsigned long long &lo, uns
 // instantiation).
 template <int BFMT, int TFMT, bool STATS, bool FLAT, bool CLUSTER, int KERN>
 __device__ void eval_one(const MapDesc &d, const ClusterDesc &cd, float tau, float jac_eps, const pndf_query &rec,
-                         int lane, uint32_t *stk, uint32_t *lq, uint32_t *ring, float4 *hits, float &D_out,
-                         uint32_t &flags_out, pndf_query_stats *st_out)
+                         int lane, uint32_t *wsm, Query<KERN> &q, float &D_out, uint32_t &flags_out,
+                         pndf_query_stats *st_out)
 {
     constexpr bool CLAMP = KERN == kKernGaussClamp;
-    Query q = make_query(rec, KERN, jac_eps);
     Acc acc = {};
     acc_zero();
+    {
+        Query<KERN> r = make_query<KERN>(rec, jac_eps);
+        if (CLUSTER) r.theta *= tau;  // r_x r_y tau with the support's half-widths
+        __syncwarp();
+        if (lane == 0) q = r;
+        __syncwarp();
+    }
     if (!q.valid) {
         if (lane == 0) {
             D_out = __int_as_float(0x7fc00000);
@@ -1099,7 +1248,6 @@ __device__ void eval_one(const MapDesc &d, const ClusterDesc &cd, float tau, flo
         }
         return;
     }
-    if (CLUSTER) q.theta *= tau;  // r_x r_y tau with the support's half-widths
     const int L = d.L;
     if (FLAT) {
         // every leaf block meeting the 4-sigma box, no pruning
@@ -1118,7 +1266,7 @@ __device__ void eval_one(const MapDesc &d, const ClusterDesc &cd, float tau, flo
         int a0, a1, c0, c1;
         node_range(q.x, q.rx, sz, S, a0, a1);
         node_range(q.y, q.ry, sz, S, c0, c1);
-        eval_range<BFMT, TFMT, STATS, CLUSTER, CLAMP>(d, cd, q, e, a0, a1, c0, c1, lane, stk, lq, ring, hits, acc);
+        eval_range<BFMT, TFMT, STATS, CLUSTER, CLAMP>(d, cd, q, e, a0, a1, c0, c1, lane, wsm, acc);
     }
     unsigned long long lo, hi;
     uint32_t fl;
@@ -1174,7 +1322,8 @@ struct SplitPlan {
     int resident_warps;
 };
 
-__device__ __forceinline__ float split_estimate(const Query &q)
+template <class Q>
+__device__ __forceinline__ float split_estimate(const Q &q)
 {
     return q.valid ? 64.f + 4.f * q.rx * q.ry : 64.f;
 }
@@ -1185,7 +1334,7 @@ __global__ void split_work(const pndf_query *__restrict__ qs, int64_t nq, float 
     __shared__ double red[256];
     double acc = 0.0;
     for (int64_t k = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; k < nq; k += int64_t(gridDim.x) * blockDim.x)
-        acc += double(split_estimate(make_query(qs[k], KERN, jac_eps)));
+        acc += double(split_estimate(make_query<KERN>(qs[k], jac_eps)));
     red[threadIdx.x] = acc;
     __syncthreads();
     for (int o = 128; o > 0; o >>= 1) {
@@ -1196,7 +1345,8 @@ __global__ void split_work(const pndf_query *__restrict__ qs, int64_t nq, float 
 }
 
 // Tiles of level l over the support's bounding box: ceil(nx / 4) ceil(ny / 4).
-__device__ __forceinline__ uint32_t split_tiles(const Query &q, int L, int l, int &a0, int &a1, int &c0, int &c1)
+template <class Q>
+__device__ __forceinline__ uint32_t split_tiles(const Q &q, int L, int l, int &a0, int &a1, int &c0, int &c1)
 {
     const int S = 1 << (L - l);
     const float sz = float(1u << l);
@@ -1214,7 +1364,8 @@ __device__ __forceinline__ float split_target(const SplitPlan &p)
 // Whether query q is divided at target wt, and into which tiles: the deepest
 // level (>= kSplitMinLevel) whose tile count stays <= kSplitMaxTiles, or the
 // first going down whose count reaches estimate / wt; at least two tiles.
-__device__ __forceinline__ bool split_choice(const Query &q, int L, float wt, int &level, uint32_t &tiles)
+template <class Q>
+__device__ __forceinline__ bool split_choice(const Q &q, int L, float wt, int &level, uint32_t &tiles)
 {
     const float w = split_estimate(q);
     if (!q.valid || !(w > 2.f * wt)) return false;
@@ -1257,7 +1408,7 @@ __global__ void split_plan(MapDesc d, const pndf_query *__restrict__ qs, int64_t
 {
     const float wt = split_target(p);
     for (int64_t k = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; k < nq; k += int64_t(gridDim.x) * blockDim.x) {
-        const Query q = make_query(qs[k], KERN, jac_eps);
+        const auto q = make_query<KERN>(qs[k], jac_eps);
         int level;
         uint32_t tiles;
         p.marker[k] = split_choice(q, d.L, wt, level, tiles) && split_reserve(p, uint32_t(k), 0, level, tiles);
@@ -1279,7 +1430,8 @@ __device__ __forceinline__ int tile_entry(const SplitPlan &p, int n_entries, uns
     return lo;
 }
 
-__device__ __forceinline__ void tile_range(const Query &q, int L, int l, uint32_t j, int &a0, int &a1, int &c0, int &c1)
+template <class Q>
+__device__ __forceinline__ void tile_range(const Q &q, int L, int l, uint32_t j, int &a0, int &a1, int &c0, int &c1)
 {
     int b0, b1, d0, d1;
     split_tiles(q, L, l, b0, b1, d0, d1);
@@ -1337,14 +1489,12 @@ __global__ void __launch_bounds__(256, PNDF_TRAVERSE_MIN_CTAS)
 {
     extern __shared__ uint32_t smem[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    uint32_t *stk = smem + warp * kWarpSmemWords;
-    uint32_t *lq = stk + kStackCap;
-    uint32_t *ring = lq + kLeafQ;
-    float4 *hits = reinterpret_cast<float4 *>(ring + kRing + kCapRing);
+    uint32_t *wsm = smem + warp * kWarpSmemWords<CLUSTER>;
     // the divided queries' tiles take the first s_ntiles work indices
     __shared__ unsigned long long s_ntiles;
     __shared__ int s_entries;
     __shared__ uint32_t s_dest[8][2];  // per warp: query, entry (-1: whole query)
+    __shared__ Query<KERN> s_query[8];
     if (threadIdx.x == 0) {
         int n = 0;
         unsigned long long t = 0ull;
@@ -1365,8 +1515,8 @@ __global__ void __launch_bounds__(256, PNDF_TRAVERSE_MIN_CTAS)
             const int64_t qi = order ? int64_t(order[k]) : int64_t(k);
             float Dv;
             uint32_t fv;
-            eval_one<BFMT, TFMT, STATS, FLAT, CLUSTER, KERN>(d, cd, tau, jac_eps, qs[qi], lane, stk, lq, ring, hits, Dv,
-                                                             fv, stats ? stats + qi : nullptr);
+            eval_one<BFMT, TFMT, STATS, FLAT, CLUSTER, KERN>(d, cd, tau, jac_eps, qs[qi], lane, wsm, s_query[warp], Dv, fv,
+                                                             stats ? stats + qi : nullptr);
             if (lane == 0) {
                 D[qi] = Dv;
                 if (flags) flags[qi] = fv;
@@ -1377,13 +1527,13 @@ __global__ void __launch_bounds__(256, PNDF_TRAVERSE_MIN_CTAS)
         constexpr bool CLAMP = KERN == kKernGaussClamp;
         int ei = -1;  // the divided query's entry, or -1 for a whole query
         uint32_t qi;
-        Query q;
+        Query<KERN> q;
         int e, a0, a1, c0, c1;
         if (k < s_ntiles) {
             ei = tile_entry(sp, s_entries, k);
             const SplitEntry &E = sp.entries[ei];
             qi = __ldg(&E.qi);
-            q = make_query(qs[qi], KERN, jac_eps);
+            q = make_query<KERN>(qs[qi], jac_eps);
             e = __ldg(&E.level);
             tile_range(q, d.L, e, uint32_t(k - __ldg(&E.base)), a0, a1, c0, c1);
         } else {
@@ -1391,7 +1541,7 @@ __global__ void __launch_bounds__(256, PNDF_TRAVERSE_MIN_CTAS)
             if (k >= (unsigned long long)nq) break;
             qi = order ? order[k] : uint32_t(k);
             if (s_entries > 0 && sp.marker[qi]) continue;  // evaluated as tiles
-            q = make_query(qs[qi], KERN, jac_eps);
+            q = make_query<KERN>(qs[qi], jac_eps);
             if (!q.valid) {
                 if (lane == 0) {
                     D[qi] = __int_as_float(0x7fc00000);
@@ -1407,13 +1557,16 @@ __global__ void __launch_bounds__(256, PNDF_TRAVERSE_MIN_CTAS)
             node_range(q.y, q.ry, sz, 1 << (d.L - e), c0, c1);
         }
         // where the result goes waits in shared memory during the descent
+        __syncwarp();
         if (lane == 0) {
             s_dest[warp][0] = qi;
             s_dest[warp][1] = uint32_t(ei);
+            s_query[warp] = q;
         }
+        __syncwarp();
         Acc acc = {};
         acc_zero();
-        eval_range<BFMT, TFMT, STATS, false, CLAMP>(d, cd, q, e, a0, a1, c0, c1, lane, stk, lq, ring, hits, acc);
+        eval_range<BFMT, TFMT, STATS, false, CLAMP>(d, cd, s_query[warp], e, a0, a1, c0, c1, lane, wsm, acc);
         unsigned long long lo, hi;
         uint32_t fl;
         warp_total<STATS>(acc, lo, hi, fl);
@@ -1444,7 +1597,7 @@ __global__ void __launch_bounds__(256, PNDF_TRAVERSE_MIN_CTAS)
 // blocks, so they share L1/L2 lines.  The order never changes a result.
 __device__ __forceinline__ uint32_t sort_key(const MapDesc &d, const pndf_query &r, int mode, int sub)
 {
-    Query q = make_query(r);
+    const auto q = make_query<PNDF_KERNEL_GAUSS>(r);
     if (!q.valid) return 0u;
     int e = entry_level(q, d.L);
     int tb, mb;  // bits per axis for the tile and the normal bin
@@ -1574,7 +1727,7 @@ cudaError_t launch_traverse(const MapDesc &d, const ClusterDesc &cd, float tau, 
     if (FLAT || CLUSTER) sp.entries = nullptr;  // whole queries only (the cut depends on the entry level)
     auto kern = traverse_kernel<BFMT, TFMT, STATS, FLAT, CLUSTER, KERN>;
     int threads = warps * 32;
-    size_t smem = size_t(warps) * kWarpSmemWords * sizeof(uint32_t);
+    size_t smem = size_t(warps) * kWarpSmemWords<CLUSTER> * sizeof(uint32_t);
     int dev = 0, sms = 0, occ = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -1777,7 +1930,7 @@ __global__ void serve_split_work(const uint32_t *__restrict__ table, const pndf_
     for (uint32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < total; k += gridDim.x * blockDim.x) {
         const pndf_segment &sg = segs[serve_segment(prefix, nsegs, k)];
         const int64_t j = int64_t(sg.first) + int64_t(k - prefix[&sg - segs]);
-        acc += double(split_estimate(make_query(sg.q[sg.order ? int64_t(sg.order[j]) : j], KERN, jac_eps)));
+        acc += double(split_estimate(make_query<KERN>(sg.q[sg.order ? int64_t(sg.order[j]) : j], jac_eps)));
     }
     red[threadIdx.x] = acc;
     __syncthreads();
@@ -1802,7 +1955,7 @@ __global__ void serve_split_plan(const MapDesc *__restrict__ maps, const uint32_
         const pndf_segment &sg = segs[i];
         const int64_t j = int64_t(sg.first) + int64_t(k - prefix[i]);
         const uint32_t qi = sg.order ? sg.order[j] : uint32_t(j);
-        const Query q = make_query(sg.q[qi], KERN, jac_eps);
+        const auto q = make_query<KERN>(sg.q[qi], jac_eps);
         int level;
         uint32_t tiles;
         if (split_choice(q, maps[sg.map].L, wt, level, tiles) && !split_reserve(p, qi, i, level, tiles))
@@ -1823,6 +1976,7 @@ __global__ void __launch_bounds__(256, PNDF_TRAVERSE_MIN_CTAS)
     __shared__ int s_entries;
     __shared__ float s_wt;
     __shared__ uint32_t s_dest[8][3];  // per warp: segment, query, entry (-1: whole query)
+    __shared__ Query<KERN> s_query[8];
     const int nsegs = int(table[0]);
     // the segment prefix sums, searched once per query, in shared memory when they fit
     const bool prefix_in_smem = nsegs < kServePrefixSmem;
@@ -1850,10 +2004,7 @@ __global__ void __launch_bounds__(256, PNDF_TRAVERSE_MIN_CTAS)
     }
     __syncthreads();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    uint32_t *stk = smem + warp * kWarpSmemWords;
-    uint32_t *lq = stk + kStackCap;
-    uint32_t *ring = lq + kLeafQ;
-    float4 *hits = reinterpret_cast<float4 *>(ring + kRing + kCapRing);
+    uint32_t *wsm = smem + warp * kWarpSmemWords<CLUSTER>;
     const uint32_t *prefix = prefix_in_smem ? sprefix : table + 1;
     const uint32_t total = prefix[nsegs];
     while (true) {
@@ -1869,7 +2020,7 @@ __global__ void __launch_bounds__(256, PNDF_TRAVERSE_MIN_CTAS)
             float Dv;
             uint32_t fv;
             eval_one<BFMT, TFMT, false, false, CLUSTER, KERN>(smaps[sg.map], clusters[sg.map], tau, jac_eps, sg.q[qi],
-                                                               lane, stk, lq, ring, hits, Dv, fv, nullptr);
+                                                               lane, wsm, s_query[warp], Dv, fv, nullptr);
             if (lane == 0) {
                 sg.D[qi] = Dv;
                 if (sg.flags) sg.flags[qi] = fv;
@@ -1881,14 +2032,14 @@ __global__ void __launch_bounds__(256, PNDF_TRAVERSE_MIN_CTAS)
         int ei = -1;
         int i;
         uint32_t qi;
-        Query q;
+        Query<KERN> q;
         int e, a0, a1, c0, c1;
         if (k < s_ntiles) {
             ei = tile_entry(sp, s_entries, k);
             const SplitEntry &E = sp.entries[ei];
             i = __ldg(&E.pad);
             qi = __ldg(&E.qi);
-            q = make_query(segs[i].q[qi], KERN, jac_eps);
+            q = make_query<KERN>(segs[i].q[qi], jac_eps);
             e = __ldg(&E.level);
             tile_range(q, smaps[segs[i].map].L, e, uint32_t(k - __ldg(&E.base)), a0, a1, c0, c1);
         } else {
@@ -1897,7 +2048,7 @@ __global__ void __launch_bounds__(256, PNDF_TRAVERSE_MIN_CTAS)
             i = serve_segment(prefix, nsegs, uint32_t(k));
             const int64_t j = int64_t(segs[i].first) + int64_t(uint32_t(k) - prefix[i]);
             qi = segs[i].order ? segs[i].order[j] : uint32_t(j);
-            q = make_query(segs[i].q[qi], KERN, jac_eps);
+            q = make_query<KERN>(segs[i].q[qi], jac_eps);
             const int L = smaps[segs[i].map].L;
             if (!q.valid) {
                 if (lane == 0) {
@@ -1918,16 +2069,18 @@ __global__ void __launch_bounds__(256, PNDF_TRAVERSE_MIN_CTAS)
             node_range(q.y, q.ry, sz, 1 << (L - e), c0, c1);
         }
         // where the result goes waits in shared memory during the descent
+        __syncwarp();
         if (lane == 0) {
             s_dest[warp][0] = uint32_t(i);
             s_dest[warp][1] = qi;
             s_dest[warp][2] = uint32_t(ei);
+            s_query[warp] = q;
         }
+        __syncwarp();
         const int map = segs[i].map;
         Acc acc = {};
         acc_zero();
-        eval_range<BFMT, TFMT, false, false, CLAMP>(smaps[map], kNoClusters, q, e, a0, a1, c0, c1, lane, stk, lq, ring,
-                                                    hits, acc);
+        eval_range<BFMT, TFMT, false, false, CLAMP>(smaps[map], kNoClusters, s_query[warp], e, a0, a1, c0, c1, lane, wsm, acc);
         unsigned long long lo, hi;
         uint32_t fl;
         warp_total<false>(acc, lo, hi, fl);
@@ -1954,7 +2107,7 @@ cudaError_t launch_serve_t(const ServeVariant &v, const MapDesc *maps, const Clu
 {
     auto kern = serve_kernel<BFMT, TFMT, CLUSTER, KERN>;
     int threads = warps * 32;
-    size_t smem = size_t(warps) * kWarpSmemWords * sizeof(uint32_t);
+    size_t smem = size_t(warps) * kWarpSmemWords<CLUSTER> * sizeof(uint32_t);
     int dev = 0, sms = 0, occ = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -1986,7 +2139,7 @@ template <int BFMT, int TFMT, bool CLUSTER, int KERN>
 cudaError_t serve_smem_t(int warps)
 {
     return cudaFuncSetAttribute(serve_kernel<BFMT, TFMT, CLUSTER, KERN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                warps * kWarpSmemWords * int(sizeof(uint32_t)));
+                                warps * kWarpSmemWords<CLUSTER> * int(sizeof(uint32_t)));
 }
 
 template <int BFMT, int TFMT>
