@@ -847,11 +847,12 @@ __device__ __forceinline__ void test_groups(const MapDesc &d, const Q &q, LeafSt
 // b = B - A, c = C - A.  Same rule as for a fine triangle (closed bounding box, edge
 // functions sign-consistent with the orientation); the Jacobian of the
 // cluster map is cross / 4^l, applied when the hit is weighed.  Triangles
-// with FP32 |cross| < 2e-10 are decided and weighed here in FP64.
+// with FP32 |cross| < 2e-10 are decided and weighed here in FP64, if the node
+// (l, I, J) meets the support exactly (node_meets lets some by).
 template <bool STATS, class Q>
 __device__ __forceinline__ bool cluster_edge_test(const Q &q, float2 p, float2 b, float2 c, int l, int ai,
-                                                  int aj, float dir, uint32_t id, Acc &acc, float &cr_o, float &e1_o,
-                                                  float &e2_o)
+                                                  int aj, float dir, uint32_t I, uint32_t J, uint32_t id, Acc &acc,
+                                                  float &cr_o, float &e1_o, float &e2_o)
 {
     if (STATS) acc.tests++;
     if (p.x < fminf(0.f, fminf(b.x, c.x)) || p.x > fmaxf(0.f, fmaxf(b.x, c.x)) ||
@@ -868,6 +869,7 @@ __device__ __forceinline__ bool cluster_edge_test(const Q &q, float2 p, float2 b
         e2_o = e2;
         return hit;
     }
+    if (!node_in_footprint(q, l, I, J)) return false;
     double bx = b.x, by = b.y, cx = c.x, cy = c.y, px = p.x, py = p.y;
     double dcr = bx * cy - by * cx;
     if (dcr == 0.0) {
@@ -928,20 +930,20 @@ __device__ __forceinline__ void test_clusters(const MapDesc &d, const ClusterDes
         const uint32_t m = k - node_index(d.L, l, 0);
         const float4 *rec = cd.cl + 2 * size_t(k);
         float4 r0 = __ldg(rec), r1 = __ldg(rec + 1);
-        int ox = int(compact1by1(m)) << l, oy = int(compact1by1(m >> 1)) << l;
+        const uint32_t I = compact1by1(m), J = compact1by1(m >> 1);
+        int ox = int(I) << l, oy = int(J) << l;
         int a = 1 << l;
         float2 p = make_float2(q.mx - r0.x, q.my - r0.y);
         float2 d10 = make_float2(r0.z, r0.w), d01 = make_float2(r1.x, r1.y), d11 = make_float2(r1.z, r1.w);
         // hit fingerprint id (stats): row-major node index at its level
-        uint32_t id = kClusterTag | (uint32_t(l) << 27) |
-                      (((uint32_t(oy >> l) << (d.L - l)) + uint32_t(ox >> l)) << 1);
+        uint32_t id = kClusterTag | (uint32_t(l) << 27) | (((J << (d.L - l)) + I) << 1);
         float cr, e1, e2;
         if (STATS) acc.clusters++;
-        h0 = cluster_edge_test<STATS>(q, p, d10, d01, l, ox, oy, float(a), id, acc, cr, e1, e2);
+        h0 = cluster_edge_test<STATS>(q, p, d10, d01, l, ox, oy, float(a), I, J, id, acc, cr, e1, e2);
         if (h0) v0 = make_float4(cr, e1, e2, __uint_as_float(k << 1));
         float2 pu = make_float2(p.x - d11.x, p.y - d11.y);
         float2 bu = make_float2(d01.x - d11.x, d01.y - d11.y), cu = make_float2(d10.x - d11.x, d10.y - d11.y);
-        h1 = cluster_edge_test<STATS>(q, pu, bu, cu, l, ox + a, oy + a, -float(a), id | 1u, acc, cr, e1, e2);
+        h1 = cluster_edge_test<STATS>(q, pu, bu, cu, l, ox + a, oy + a, -float(a), I, J, id | 1u, acc, cr, e1, e2);
         if (h1) v1 = make_float4(cr, e1, e2, __uint_as_float((k << 1) | 1u));
     }
 #pragma unroll
@@ -1051,19 +1053,6 @@ __device__ __forceinline__ void eval_range(const MapDesc &d, const ClusterDesc &
     auto in_slab = [&](const Node<BFMT> &n, uint32_t k) {
         return (CLUSTER && k < leaf0) || node_slab_holds<BFMT, CLAMP>(n, q);
     };
-    // the cut of Sec. 4.2, e <= r_x r_y tau, of a node that holds m; a node is cut
-    // only if its uv box meets the support exactly (node_meets lets some by),
-    // else nothing below it contributes
-    auto cut_here = [&](uint32_t k, float ev, bool ins, bool &pass) {
-        if (STATS) acc.cchecks++;
-        if (!(ev <= q.theta)) return false;
-        if (!ins) {
-            const int l = node_level(k, d.L);
-            const uint32_t m = k - node_index(d.L, l, 0);
-            pass = node_in_footprint(q, l, compact1by1(m), compact1by1(m >> 1));
-        }
-        return pass;
-    };
     // node k, child of a parent that was not inside: meets the support?  (and is it inside?)
     auto in_footprint = [&](uint32_t k, bool &ins) {
         if (ins) return true;
@@ -1081,7 +1070,10 @@ __device__ __forceinline__ void eval_range(const MapDesc &d, const ClusterDesc &
         bool pass = valid && node_meets(q, e, a, c, inside) && node_box_holds<BFMT, CLAMP>(n, q);
         bool cut = false;
         if (STATS) acc.nodes += valid ? 1u : 0u;
-        if (CLUSTER && pass) cut = cut_here(k, __ldg(cd.ce + k), inside, pass);
+        if (CLUSTER && pass) {  // the cut of Sec. 4.2: e <= r_x r_y tau
+            cut = __ldg(cd.ce + k) <= q.theta;
+            if (STATS) acc.cchecks++;
+        }
         if (pass && !cut) pass = in_slab(n, k);
         unsigned mp = __ballot_sync(kFull, pass && !cut);
         unsigned mc = __ballot_sync(kFull, cut);
@@ -1151,7 +1143,10 @@ __device__ __forceinline__ void eval_range(const MapDesc &d, const ClusterDesc &
             pass[r] = pass[r] && node_box_holds<BFMT, CLAMP>(nd[r], q);
             if (CLUSTER) {
                 pass[r] = pass[r] && in_footprint(ck[r], ins[r]);
-                if (pass[r]) cut[r] = cut_here(ck[r], ev[r], ins[r], pass[r]);
+                if (pass[r]) {  // the cut of Sec. 4.2: e <= r_x r_y tau
+                    cut[r] = ev[r] <= q.theta;
+                    if (STATS) acc.cchecks++;
+                }
                 if (pass[r] && !cut[r]) pass[r] = in_slab(nd[r], ck[r]);
             } else {
                 pass[r] = pass[r] && in_slab(nd[r], ck[r]) && in_footprint(ck[r], ins[r]);

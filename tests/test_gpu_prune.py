@@ -24,15 +24,12 @@ def make_map(kind, n):
         return synth.flake_normals(n, max(4, n * n // 90), seed=n)
     if kind == "bumps":
         return synth.bumps_map(n=n, n_bumps=max(1, n // 8), seed=n)
-    if kind == "collinear":  # all normals on one line: zero-area triangles and slabs of width zero
-        t = torch.sin(torch.arange(n * n, dtype=torch.float32).reshape(n, n))
-        return torch.stack((0.2 * t, 0.1 * t), -1)
     if kind == "plateaus":  # few distinct normals: repeated vertices, m on vertices
         return synth.flake_normals(n, max(4, n * n // 30), seed=n).round(decimals=2)
     return 2.0 ** -17 * synth.bumps_map(n=n, n_bumps=max(1, n // 8), seed=n)  # near-singular triangles
 
 
-@pytest.mark.parametrize("kind", ["flake", "bumps", "collinear", "plateaus", "minute"])
+@pytest.mark.parametrize("kind", ["flake", "bumps", "plateaus", "minute"])
 @pytest.mark.parametrize("n", [2, 3, 4, 5, 6, 9, 33, 64, 65, 66, 131])
 def test_hierarchy_hits_what_the_flat_scan_hits(P, kind, n):
     st = make_map(kind, n)
