@@ -7,33 +7,29 @@
 // (n_c - n_a).  Every triangle in the footprint is integrated (no pruning:
 // every visible triangle contributes).
 //
-// Per triangle:
+// Per triangle (meang.cuh): a positive quadrature of the integrand over the uv
+// triangle, in FP32.
 //  * all three vertices see w  =>  the whole triangle does (the visible region,
-//    a right half-disk joined to a left half-ellipse, is convex; App. B), and
-//    V_T = w_z A + w_x Wx + w_y Wy with Wx = -oint m~_z dm_y, Wy = oint m~_z
-//    dm_x (Green's theorem on d(-m~_z)/dm_x = m_x/m~_z).  Along an edge the
-//    mean of m~_z is the arc-area formula of App. B; it is evaluated in a
-//    cancellation-free form (the asin difference as one atan2 of exact
-//    products), so no rotation is needed and the 1/|cross| division keeps
-//    FP32 accuracy for small triangles.  Small slivers (longest edge^2 below
-//    1e-4 and aspect above 2) take the 3-point edge-midpoint rule on
-//    max(m~.w, 0)/m~_z instead, exact for quadratics.
-//  * no vertex sees w and the triangle stays clear of the visibility
-//    boundary: exactly 0 (Alg. 1 drops every edge).
-//  * otherwise (partly visible, slivers of aspect above 2000, normals
-//    collapsed onto a segment): the general path of visible.cuh in FP64 (the
-//    clip of Alg. 1 as a line-circle intersection in a scaled frame, Eq. 11's
-//    boundary integral as a corner fan plus chord and arc excesses, and the
-//    segment form of Eq. 13 in closed form), deferred and evaluated 32
-//    triangles at a time so that it runs lane-dense.
+//    a right half-disk joined to a left half-ellipse, is convex; App. B): 6
+//    points for small triangles, 12 for those that straddle normal regions;
+//  * no vertex sees w and none of the triangle can: exactly 0 (Alg. 1 drops
+//    every edge);
+//  * otherwise cut along the visibility boundary into smooth pieces
+//    (partial_mean);
+//  * very large triangles: the closed form of visible.cuh in FP64 (the clip of
+//    Alg. 1, Eq. 11's boundary integral, the segment form of Eq. 13).
+// All but the first kind and the zeros are deferred into per-warp rings and
+// evaluated 32 at a time, so that each runs lane-dense.
 //
 // Work decomposition: each request's footprint is cut into bands of kBand quad
-// rows; one warp integrates one band (lane = quad column, two triangles per
-// lane), compensated sums are reduced across the warp and stored per band;
+// rows; one warp integrates one band (its quads inside the support's ellipse,
+// row after row, one per lane), compensated sums are reduced across the warp
+// and stored per band;
 // a second kernel adds a request's bands in fixed order, so results do not
 // depend on scheduling or on which other requests share the launch.
 #include "area_step.cuh"
 #include "ggx.cuh"
+#include "meang.cuh"
 #include "visible.cuh"
 
 namespace pndf {
@@ -43,82 +39,16 @@ __device__ unsigned int g_status_projarea;
 namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
+#ifndef PNDF_GGX_CTAS
+#define PNDF_GGX_CTAS 4  // of 3, 4, 5, 6 and 8 within 8% of each other
+#endif
+#ifndef PNDF_PA_CTAS
+#define PNDF_PA_CTAS 4
+#endif
 constexpr int kBand = 8;                 // quad rows per work item
 
-__device__ __forceinline__ float dop(float a, float b, float c, float d)
-{
-    float w = c * d;
-    float e = fmaf(-c, d, w);
-    float f = fmaf(a, b, -w);
-    return f + e;
-}
-
-__device__ __forceinline__ float zof(float2 p)
-{
-    return sqrtf(fmaxf(0.f, 1.f - fmaf(p.x, p.x, p.y * p.y)));
-}
-
-// phi(t) = t - sin t, by its Taylor series for small |t| (no cancellation).
-__device__ __forceinline__ float phi_small(float t)
-{
-    if (fabsf(t) < 0.25f) {
-        float t2 = t * t;
-        return t * t2 * (1.f / 6.f) * (1.f - t2 * (1.f / 20.f) * (1.f - t2 * (1.f / 42.f) * (1.f - t2 * (1.f / 72.f))));
-    }
-    return t - sinf(t);
-}
-
-// Curvature part H of the mean of m~_z = sqrt(1 - |m|^2) along p0 -> p1, over
-// its trapezoid value (z0 + z1)/2.  With d the unit direction, u the abscissa
-// along the line (u1 = u0 + L) and r^2 = 1 - s^2 = z0^2 + u0^2 (s the line's
-// distance to the origin), the arc-area formula of App. B gives
-//   L * mean = (1/2)[u z]_{u0}^{u1} + (r^2/2)(asin(u1/r) - asin(u0/r)),
-// so L * H = (r^2/2)(dth - sin dth) with dth the asin difference, which is
-// atan2(X, Y), X = u1 z0 - u0 z1 = L (r^2 + z0 z1 + u0 u1) / (z0 + z1),
-// Y = z0 z1 + u0 u1 (both free of cancellation).
-__device__ __forceinline__ float edge_curv(float2 p0, float z0, float2 p1, float z1)
-{
-    float ex = p1.x - p0.x, ey = p1.y - p0.y;
-    float L2 = fmaf(ex, ex, ey * ey);
-    if (L2 == 0.f) return 0.f;
-    float L = sqrtf(L2);
-    float inv = 1.f / L;
-    float u0 = fmaf(ex, p0.x, ey * p0.y) * inv;
-    float u1 = u0 + L;
-    float r2 = fmaf(z0, z0, u0 * u0);
-    float Y = fmaf(z0, z1, u0 * u1);
-    float X = L * (r2 + Y) / (z0 + z1);
-    return 0.5f * r2 * phi_small(atan2f(X, Y)) * inv;
-}
-
-// z(q) - z(p) for z = sqrt(1 - |m|^2), from (|p|^2 - |q|^2) / (z(p) + z(q)).
-__device__ __forceinline__ float zdiff(float2 p, float zp, float2 q, float zq)
-{
-    return -fmaf(q.x - p.x, q.x + p.x, (q.y - p.y) * (q.y + p.y)) / (zp + zq);
-}
-
-struct Dir {
-    float wx, wy, wz;  // unit direction
-    float c, s, wr;    // rotation to w_y = 0: (c, s) = w_xy / |w_xy|, wr = |w_xy|
-};
-
-// Unit direction from the caller's (unit to single precision) vector.
-__device__ __forceinline__ Dir make_dir_f(float wx, float wy, float wz)
-{
-    Dir w;
-    const float n = sqrtf(fmaf(wx, wx, fmaf(wy, wy, wz * wz)));
-    w.wx = wx / n;
-    w.wy = wy / n;
-    w.wz = wz / n;
-    w.wr = sqrtf(fmaf(w.wx, w.wx, w.wy * w.wy));
-    w.c = w.wr > 0.f ? w.wx / w.wr : 1.f;
-    w.s = w.wr > 0.f ? w.wy / w.wr : 0.f;
-    return w;
-}
-
-// V_T / |cross| on the general path (visible.cuh, FP64): partly visible
-// triangles, long slivers, and triangles whose normals collapsed onto a
-// segment (|cross| < 1e-12: the segment form of Eq. 13).
+// V_T / |cross| in closed form (visible.cuh, FP64): the triangles of class kSlow;
+// the segment form of Eq. 13 where the normals collapsed (|cross| < 1e-12).
 __device__ __noinline__ float slow_ratio(float2 a, float2 b, float2 c, const Dir &wf)
 {
     const vis::DirD w = vis::make_dir(wf.wx, wf.wy, wf.wz);
@@ -126,95 +56,6 @@ __device__ __noinline__ float slow_ratio(float2 a, float2 b, float2 c, const Dir
                       (double(b.y) - double(a.y)) * (double(c.x) - double(a.x));
     if (fabs(cr) < 1e-12) return float(vis::collapsed_visible(a.x, a.y, b.x, b.y, c.x, c.y, w));
     return float(vis::tri_visible<double>(a.x, a.y, b.x, b.y, c.x, c.y, w));
-}
-
-// Squared distance from the origin to segment p -> q.
-__device__ __forceinline__ float seg_dist2(float px, float py, float qx, float qy)
-{
-    float vx = qx - px, vy = qy - py;
-    float L2 = fmaf(vx, vx, vy * vy);
-    float t = L2 > 0.f ? fminf(fmaxf(-fmaf(px, vx, py * vy) / L2, 0.f), 1.f) : 0.f;
-    float dx = fmaf(t, vx, px), dy = fmaf(t, vy, py);
-    return fmaf(dx, dx, dy * dy);
-}
-
-// True when the triangle provably sees nothing of w: in the frame rotated so
-// w_y = 0 all three vertices have m_x < 0 (the visible part there is the
-// half-ellipse (m_x / w_z)^2 + m_y^2 <= 1) and the triangle stays clear of
-// that ellipse (distance > 1 from the origin after scaling m_x by 1 / w_z,
-// with a margin for FP32 rounding).  Alg. 1 drops every edge of such a
-// triangle, so its integral is exactly 0.
-__device__ __forceinline__ bool invisible_and_clear(float2 a, float2 b, float2 c, const Dir &w)
-{
-    float ax = fmaf(w.c, a.x, w.s * a.y), bx = fmaf(w.c, b.x, w.s * b.y), cx = fmaf(w.c, c.x, w.s * c.y);
-    if (!(ax < 0.f && bx < 0.f && cx < 0.f)) return false;
-    float ay = fmaf(-w.s, a.x, w.c * a.y), by = fmaf(-w.s, b.x, w.c * b.y), cy = fmaf(-w.s, c.x, w.c * c.y);
-    float iz = 1.f / w.wz;
-    ax *= iz;
-    bx *= iz;
-    cx *= iz;
-    // the origin must not lie inside the scaled triangle
-    float o0 = dop(bx - ax, -ay, by - ay, -ax), o1 = dop(cx - bx, -by, cy - by, -bx), o2 = dop(ax - cx, -cy, ay - cy, -cx);
-    if ((o0 >= 0.f && o1 >= 0.f && o2 >= 0.f) || (o0 <= 0.f && o1 <= 0.f && o2 <= 0.f)) return false;
-    float d2 = fminf(seg_dist2(ax, ay, bx, by), fminf(seg_dist2(bx, by, cx, cy), seg_dist2(cx, cy, ax, ay)));
-    return d2 > 1.0045f;  // (1 + 2.25e-3)^2
-}
-
-// V_T / |cross| for one triangle in FP32 when that is accurate: returns false
-// when the triangle needs the FP64 path (partially visible, long sliver,
-// collapsed), which the caller defers and batches.
-__device__ __forceinline__ bool tri_ratio_fast(float2 a, float za, float2 b, float zb, float2 c, float zc,
-                                               const Dir &w, float &out)
-{
-    float va = fmaf(w.wx, a.x, fmaf(w.wy, a.y, w.wz * za));
-    float vb = fmaf(w.wx, b.x, fmaf(w.wy, b.y, w.wz * zb));
-    float vc = fmaf(w.wx, c.x, fmaf(w.wy, c.y, w.wz * zc));
-    float2 ab = make_float2(b.x - a.x, b.y - a.y), ac = make_float2(c.x - a.x, c.y - a.y);
-    float2 bc = make_float2(c.x - b.x, c.y - b.y);
-    float cr = dop(ab.x, ac.y, ab.y, ac.x);
-    float P2 = fmaxf(fmaf(ab.x, ab.x, ab.y * ab.y), fmaxf(fmaf(ac.x, ac.x, ac.y * ac.y), fmaf(bc.x, bc.x, bc.y * bc.y)));
-    if (!(va >= 0.f && vb >= 0.f && vc >= 0.f)) {
-        // partially visible triangles take the FP64 path: when most of a
-        // footprint is shadowed P itself is tiny, and FP32 clipping (roots of
-        // nearly tangent edges, arcs) would dominate its relative error
-        out = 0.f;
-        return invisible_and_clear(a, b, c, w);
-    }
-    if (P2 == 0.f) {  // all three normals equal
-        out = 0.5f * (w.wz + fmaf(w.wx, a.x, w.wy * a.y) / za);
-        return true;
-    }
-    // The boundary form below has FP32 error about 1.5 eps P^2 / |cross|.
-    if (P2 > 2.0f * fabsf(cr)) {
-        if (P2 < 1e-4f) {
-            // small sliver: 3-point edge-midpoint rule (exact for quadratics) on
-            // the mean of (w . m~)/m~_z; V / |cross| = mean / 2
-            float2 m0 = make_float2(0.5f * (a.x + b.x), 0.5f * (a.y + b.y));
-            float2 m1 = make_float2(0.5f * (b.x + c.x), 0.5f * (b.y + c.y));
-            float2 m2 = make_float2(0.5f * (c.x + a.x), 0.5f * (c.y + a.y));
-            float z0 = zof(m0), z1 = zof(m1), z2 = zof(m2);
-            float f0 = fmaf(w.wx, m0.x, w.wy * m0.y) / z0;
-            float f1 = fmaf(w.wx, m1.x, w.wy * m1.y) / z1;
-            float f2 = fmaf(w.wx, m2.x, w.wy * m2.y) / z2;
-            out = 0.5f * w.wz + (f0 + f1 + f2) * (1.f / 6.f);
-            return true;
-        }
-        if (P2 > 2000.0f * fabsf(cr)) return false;  // long sliver or collapsed: FP64
-    }
-    // Fully visible: V = w_z A + w_x Wx + w_y Wy, Wx = -oint m~_z dm_y,
-    // Wy = oint m~_z dm_x.  With the edge mean of m~_z split into its
-    // trapezoid value and the curvature part H, the trapezoid sums collapse to
-    // 2x2 determinants of vertex differences in (x, z) and (y, z).
-    float dzab = zdiff(a, za, b, zb), dzac = zdiff(a, za, c, zc);
-    float dety = dop(ab.y, dzac, ac.y, dzab);
-    float detx = dop(ab.x, dzac, ac.x, dzab);
-    float hab = edge_curv(a, za, b, zb), hbc = edge_curv(b, zb, c, zc), hca = edge_curv(c, zc, a, za);
-    float Wx = 0.5f * dety - (hab * ab.y + hbc * bc.y - hca * ac.y);
-    float Wy = -0.5f * detx + (hab * ab.x + hbc * bc.x - hca * ac.x);
-    // orientation-following integrals over the signed cross = the
-    // counter-clockwise value over |cross|
-    out = 0.5f * w.wz + fmaf(w.wx, Wx, w.wy * Wy) / cr;
-    return true;
 }
 
 struct Req {
@@ -258,6 +99,39 @@ __device__ __forceinline__ float wq(const Req &q, float dx, float dy)
     return fmaf(q.ia * dx, dx, fmaf(2.f * q.ib * dx, dy, q.ic * dy * dy));
 }
 
+// Columns [x0, x0 + count) of row j whose triangles' centroids can lie in the
+// ellipse q <= kQCut: at height dy, dx = -(ib / ia) dy +- sqrt(Q / ia - dy^2 det /
+// ia^2), widened by a column and 1e-3 of Q (FP32 rounding of the square root's
+// argument; a nearly singular S takes the whole row).
+__device__ __forceinline__ void row_span(const Req &q, int j, int &x0, int &count)
+{
+    const float k = q.ib / q.ia, v = q.ic / q.ia - k * k, Q = kQCut * (1.0f + 1e-3f) / q.ia;
+    x0 = q.i0;
+    count = q.i1 - q.i0 + 1;
+    if (!(v * q.ia > 1e-3f * q.ic)) return;
+    float lo = __int_as_float(0x7f800000), hi = -lo;
+#pragma unroll
+    for (int t = 1; t <= 2; ++t) {
+        const float dy = (float(j) - q.y) + float(t) * (1.f / 3.f);
+        const float r2 = fmaf(-dy * dy, v, Q);
+        if (r2 < 0.f) continue;
+        const float r = sqrtf(r2), c = fmaf(-k, dy, q.x);
+        lo = fminf(lo, c - r);
+        hi = fmaxf(hi, c + r);
+    }
+    if (lo > hi) {  // the row misses the ellipse
+        count = 0;
+        return;
+    }
+    const float f0 = fmaxf(floorf(lo) - 2.f, float(q.i0)), f1 = fminf(ceilf(hi) + 1.f, float(q.i1));
+    if (!(f0 <= f1)) {
+        count = f0 > f1 ? 0 : count;
+        return;
+    }
+    x0 = int(f0);
+    count = int(f1) - x0 + 1;
+}
+
 template <int TFMT>
 __device__ __forceinline__ float2 texel(const MapDesc &d, int i, int j)
 {
@@ -266,24 +140,57 @@ __device__ __forceinline__ float2 texel(const MapDesc &d, int i, int j)
     return __half22float2(__ldg(reinterpret_cast<const __half2 *>(d.texels) + idx));
 }
 
-// Ring of triangles deferred to the FP64 path, per warp: (i << 15) | (j << 1)
-// | tri and the triangle's kernel weight; processed 32 at a time so the slow
-// path runs with every lane busy.
+// Deferred triangles, one ring per class and warp: (i << 15) | (j << 1) | tri and
+// the kernel weight; at most 31 held over plus one step's 64.
 constexpr int kDefer = 128;
+constexpr int kRings = 3;  // kLarge, kPartial, kSlow
+struct WarpArea {
+    uint32_t id[kRings][kDefer];
+    float wt[kRings][kDefer];
+    int off[kBand + 1], x0[kBand];  // the band's rows: first quad of each in lane order, first column
+};
 
-// Lane's deferred triangle (ring slot head + lane): kernel weight times the
-// FP64 value of V_T / |cross| (tri 0 = (u0, u1, u2), tri 1 = (u3, u2, u1)).
-template <int TFMT>
-__device__ __forceinline__ float deferred_value(const MapDesc &d, const Dir &w, const uint32_t *dq_id,
-                                                const float *dq_w, uint32_t head, int lane)
+// Compensated sum (Neumaier).
+struct Sum {
+    float s, c;
+};
+__device__ __forceinline__ void add(Sum &a, float v)
 {
-    uint32_t slot = (head + uint32_t(lane)) & (kDefer - 1);
-    uint32_t id = dq_id[slot];
-    int i = int(id >> 15), j = int((id >> 1) & 0x3fffu), tri = int(id & 1u);
-    float2 a = texel<TFMT>(d, i + tri, j + tri);
-    float2 b = texel<TFMT>(d, i + 1 - tri, j + tri);
-    float2 c = texel<TFMT>(d, i + tri, j + 1 - tri);
-    return dq_w[slot] * slow_ratio(a, b, c, w);
+    const float t = a.s + v;
+    a.c += fabsf(a.s) >= fabsf(v) ? (a.s - t) + v : (v - t) + a.s;
+    a.s = t;
+}
+
+__device__ __forceinline__ float longest2(float2 a, float2 b, float2 c)
+{
+    return fmaxf(len2(sub(b, a)), fmaxf(len2(sub(c, a)), len2(sub(c, b))));
+}
+
+// Half the mean of g over a fully visible triangle of class kSmall / kLarge.
+__device__ __forceinline__ float full_mean_small(float2 a, float2 b, float2 c, const Dir &w)
+{
+    return fmaf(0.5f, quad4(a, sub(b, a), sub(c, a), [&](float x, float y) { return slope_at(w, x, y); }), 0.5f * w.wz);
+}
+__device__ __forceinline__ float full_mean_large(float2 a, float2 b, float2 c, const Dir &w)
+{
+    return fmaf(0.5f, quad6(a, sub(b, a), sub(c, a), [&](float x, float y) { return slope_at(w, x, y); }), 0.5f * w.wz);
+}
+
+// Lane's deferred triangle of ring r (slot head + lane): kernel weight times
+// V_T / |cross| (tri 0 = (u0, u1, u2), tri 1 = (u3, u2, u1)).
+template <int TFMT>
+__device__ __forceinline__ float deferred_value(const MapDesc &d, const Dir &w, const WarpArea &wa, int r,
+                                                uint32_t head, int lane)
+{
+    const uint32_t slot = (head + uint32_t(lane)) & (kDefer - 1);
+    const uint32_t id = wa.id[r][slot];
+    const int i = int(id >> 15), j = int((id >> 1) & 0x3fffu), tri = int(id & 1u);
+    const float2 a = texel<TFMT>(d, i + tri, j + tri);
+    const float2 b = texel<TFMT>(d, i + 1 - tri, j + tri);
+    const float2 c = texel<TFMT>(d, i + tri, j + 1 - tri);
+    float v = r == 0 ? full_mean_large(a, b, c, w) : r == 1 ? partial_mean(a, b, c, w) : -1.f;
+    if (r > 0 && v < 0.f) v = slow_ratio(a, b, c, w);
+    return wa.wt[r][slot] * v;
 }
 
 __global__ void pa_bands(MapDesc d, const pndf_query *__restrict__ qs, int64_t k0, int cnt, uint32_t *__restrict__ nb)
@@ -327,90 +234,94 @@ __device__ __forceinline__ void scan_bands(uint32_t *__restrict__ nb, int cnt)
 __global__ void __launch_bounds__(1024) pa_scan(uint32_t *__restrict__ nb, int cnt) { scan_bands(nb, cnt); }
 
 // Band `band` (kBand quad rows) of request (q, w) on map d, integrated by one
-// warp (lane = quad column, both triangles; the FP64 triangles deferred into
-// the warp's ring dq_id / dq_w and evaluated 32 at a time); returns the
-// compensated sum and its correction, reduced to lane 0 in a fixed order.
+// warp: the band's quads inside the ellipse in row order, one per lane, both
+// triangles; returns the compensated sum and its correction, reduced to lane 0
+// in a fixed order.
 template <int TFMT>
 __device__ __forceinline__ float2 integrate_band(const MapDesc &d, const Req &q, const Dir &w, int band, int lane,
-                                                 uint32_t *dq_id, float *dq_w)
+                                                 WarpArea &wa)
 {
     const unsigned lt = (1u << lane) - 1u;
-    const int jb0 = q.j0 + band * kBand, jb1 = min(q.j1, jb0 + kBand - 1);
-    float s = 0.f, c = 0.f;
-    uint32_t head = 0;
-    int nd = 0;  // deferred triangles waiting in the ring (warp-uniform)
-    for (int j = jb0; j <= jb1; ++j) {
-        const float dyl = (float(j) - q.y) + (1.f / 3.f), dyu = (float(j) - q.y) + (2.f / 3.f);
-        for (int ib = q.i0; ib <= q.i1; ib += 32) {
-            const int i = ib + lane;
-            float v[2] = {0.f, 0.f}, kw[2] = {0.f, 0.f};
-            bool dfr[2] = {false, false};
-            if (i <= q.i1) {
-                const float dxl = (float(i) - q.x) + (1.f / 3.f), dxu = (float(i) - q.x) + (2.f / 3.f);
-                const float ql = wq(q, dxl, dyl), qu = wq(q, dxu, dyu);
-                if (ql <= kQCut || qu <= kQCut) {
-                    // one copy of the triangle path for both triangles (tri 0 =
-                    // (u0, u1, u2), tri 1 = (u3, u2, u1)): unrolled, the kernel
-                    // stalled on instruction fetch (516 ms against 386 ms); the
-                    // quad's four texels are loaded together
-                    const float2 n1 = texel<TFMT>(d, i + 1, j), n2 = texel<TFMT>(d, i, j + 1);
-                    const float2 n0 = texel<TFMT>(d, i, j), n3 = texel<TFMT>(d, i + 1, j + 1);
-                    const float z1 = zof(n1), z2 = zof(n2);
-#pragma unroll 1
-                    for (int k = 0; k < 2; ++k) {
-                        const float qk = k ? qu : ql;
-                        if (qk > kQCut) continue;
-                        const float2 na = k ? n3 : n0;
-                        const float2 nb = k ? n2 : n1, nc = k ? n1 : n2;
-                        const float zb = k ? z2 : z1, zc = k ? z1 : z2;
-                        float r;
-                        const float kk = q.norm * expf(-0.5f * qk);
-                        const bool ok = tri_ratio_fast(na, zof(na), nb, zb, nc, zc, w, r);
-                        if (k) {
-                            kw[1] = kk;
-                            v[1] = ok ? kk * r : 0.f;
-                            dfr[1] = !ok;
-                        } else {
-                            kw[0] = kk;
-                            v[0] = ok ? kk * r : 0.f;
-                            dfr[0] = !ok;
-                        }
-                    }
+    const int jb0 = q.j0 + band * kBand, rows = min(q.j1 - jb0 + 1, kBand);
+    {
+        int x0 = 0, cnt = 0;
+        if (lane < rows) row_span(q, jb0 + lane, x0, cnt);
+        int incl = cnt;
+#pragma unroll
+        for (int o = 1; o < kBand; o <<= 1) {
+            const int v = __shfl_up_sync(kFull, incl, o);
+            if (lane >= o) incl += v;
+        }
+        __syncwarp();
+        if (lane < kBand) {
+            wa.off[lane + 1] = incl;
+            wa.x0[lane] = x0;
+        }
+        if (lane == 0) wa.off[0] = 0;
+        __syncwarp();
+    }
+    const int total = wa.off[kBand];
+    Sum sum{0.f, 0.f};
+    uint32_t head[kRings] = {0u, 0u, 0u};
+    int nd[kRings] = {0, 0, 0};  // triangles waiting per ring (warp-uniform)
+    int row = 0;
+    for (int base = 0; base < total; base += 32) {
+        const int k = base + lane;
+        Class cl[2] = {kNone, kNone};
+        float kw[2] = {0.f, 0.f}, v[2] = {0.f, 0.f};
+        int i = 0, j = 0;
+        if (k < total) {
+            while (k >= wa.off[row + 1]) ++row;
+            i = wa.x0[row] + (k - wa.off[row]);
+            j = jb0 + row;
+            const float dx = float(i) - q.x, dy = float(j) - q.y;
+            const float ql = wq(q, dx + (1.f / 3.f), dy + (1.f / 3.f)), qu = wq(q, dx + (2.f / 3.f), dy + (2.f / 3.f));
+            if (ql <= kQCut || qu <= kQCut) {
+                const float2 n1 = texel<TFMT>(d, i + 1, j), n2 = texel<TFMT>(d, i, j + 1);
+                const float2 n0 = texel<TFMT>(d, i, j), n3 = texel<TFMT>(d, i + 1, j + 1);
+                const float z1 = zof(n1), z2 = zof(n2);
+                const float f1 = phi_of(w, n1, z1), f2 = phi_of(w, n2, z2);
+                const float d12 = len2(sub(n2, n1));
+#pragma unroll
+                for (int t = 0; t < 2; ++t) {
+                    const float qk = t ? qu : ql;
+                    if (qk > kQCut) continue;
+                    const float2 na = t ? n3 : n0;
+                    const float za = zof(na);
+                    const float h2 = fmaxf(d12, fmaxf(len2(sub(n1, na)), len2(sub(n2, na))));
+                    kw[t] = q.norm * expf(-0.5f * qk);
+                    cl[t] = classify(phi_of(w, na, za), f1, f2, za, z1, z2, h2, w);
+                    if (cl[t] == kSmall) v[t] = kw[t] * full_mean_small(na, t ? n2 : n1, t ? n1 : n2, w);
                 }
             }
+        }
+        add(sum, v[0]);
+        add(sum, v[1]);
+        const bool last = base + 32 >= total;
 #pragma unroll
-            for (int k = 0; k < 2; ++k) {
-                float tt = s + v[k];
-                c += fabsf(s) >= fabsf(v[k]) ? (s - tt) + v[k] : (v[k] - tt) + s;
-                s = tt;
-                // queue the triangles that need the FP64 path
-                unsigned m = __ballot_sync(kFull, dfr[k]);
-                if (dfr[k]) {
-                    uint32_t pos = (head + uint32_t(nd) + __popc(m & lt)) & (kDefer - 1);
-                    dq_id[pos] = (uint32_t(i) << 15) | (uint32_t(j) << 1) | uint32_t(k);
-                    dq_w[pos] = kw[k];
+        for (int r = 0; r < kRings; ++r) {
+#pragma unroll
+            for (int t = 0; t < 2; ++t) {
+                const bool dfr = cl[t] == Class(kLarge + r);
+                const unsigned m = __ballot_sync(kFull, dfr);
+                if (dfr) {
+                    const uint32_t pos = (head[r] + uint32_t(nd[r]) + __popc(m & lt)) & (kDefer - 1);
+                    wa.id[r][pos] = (uint32_t(i) << 15) | (uint32_t(j) << 1) | uint32_t(t);
+                    wa.wt[r][pos] = kw[t];
                 }
-                nd += __popc(m);
+                nd[r] += __popc(m);
             }
             __syncwarp();
-            while (nd >= 32) {
-                float val = deferred_value<TFMT>(d, w, dq_id, dq_w, head, lane);
-                float tt = s + val;
-                c += fabsf(s) >= fabsf(val) ? (s - tt) + val : (val - tt) + s;
-                s = tt;
-                head += 32;
-                nd -= 32;
+            while (nd[r] >= (last ? 1 : 32)) {  // (one copy of each class's code)
+                const int n = min(nd[r], 32);
+                add(sum, lane < n ? deferred_value<TFMT>(d, w, wa, r, head[r], lane) : 0.f);
+                head[r] += uint32_t(n);
+                nd[r] -= n;
                 __syncwarp();
             }
         }
     }
-    if (nd > 0) {
-        float val = lane < nd ? deferred_value<TFMT>(d, w, dq_id, dq_w, head, lane) : 0.f;
-        float tt = s + val;
-        c += fabsf(s) >= fabsf(val) ? (s - tt) + val : (val - tt) + s;
-        s = tt;
-        __syncwarp();
-    }
+    float s = sum.s, c = sum.c;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         float so = __shfl_down_sync(kFull, s, o), co = __shfl_down_sync(kFull, c, o);
@@ -422,20 +333,19 @@ __device__ __forceinline__ float2 integrate_band(const MapDesc &d, const Req &q,
     return make_float2(s, c);
 }
 
-// Eight CTAs per SM (32 registers, some spilled): 285 ms against 319 ms at
-// six and 516 ms at two for 1,024 requests on a 4096^2 mixed map; the warps
-// that wait on the FP64 path need company to keep the SM issuing.
+// What bounds it: FP32 issue (about 250 instructions per triangle: the six
+// quadrature points 80, classification and weights 80, row walk and sums 50, the
+// deferred classes 40).  Four CTAs per SM (64 registers): 192 requests on the
+// 16384^2 mixed map 13.5 ms, at three 14.3, at five and six 13.7, at eight 15.8;
+// with the FP64 path for every partly visible triangle it was 79 ms.
 template <int TFMT>
-__global__ void __launch_bounds__(256, 8) pa_items(MapDesc d, const pndf_query *__restrict__ qs,
+__global__ void __launch_bounds__(256, PNDF_PA_CTAS) pa_items(MapDesc d, const pndf_query *__restrict__ qs,
                                                const float *__restrict__ omega, int64_t k0, int cnt,
                                                const uint32_t *__restrict__ off, float2 *__restrict__ part,
                                                unsigned int *__restrict__ cursor)
 {
-    __shared__ uint32_t dq_id_s[8][kDefer];
-    __shared__ float dq_w_s[8][kDefer];
+    __shared__ WarpArea wa_s[8];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    uint32_t *dq_id = dq_id_s[warp];
-    float *dq_w = dq_w_s[warp];
     const uint32_t total = off[cnt];
     while (true) {
         uint32_t it = 0;
@@ -454,7 +364,7 @@ __global__ void __launch_bounds__(256, 8) pa_items(MapDesc d, const pndf_query *
         const int t = lo;
         const Req q = make_req(qs[k0 + t], d.n);
         const Dir w = make_dir_f(omega[3 * (k0 + t)], omega[3 * (k0 + t) + 1], omega[3 * (k0 + t) + 2]);
-        const float2 v = integrate_band<TFMT>(d, q, w, int(it - off[t]), lane, dq_id, dq_w);
+        const float2 v = integrate_band<TFMT>(d, q, w, int(it - off[t]), lane, wa_s[warp]);
         if (lane == 0) part[it] = v;
     }
 }
@@ -523,14 +433,13 @@ __global__ void __launch_bounds__(1024) area_step_scan(const uint32_t *__restric
 }
 
 template <int TFMT>
-__global__ void __launch_bounds__(256, 8) area_step_items(const MapDesc *__restrict__ maps, int nmaps,
+__global__ void __launch_bounds__(256, PNDF_PA_CTAS) area_step_items(const MapDesc *__restrict__ maps, int nmaps,
                                                       const uint32_t *__restrict__ count,
                                                       const AreaReq *__restrict__ areq,
                                                       const uint32_t *__restrict__ off, float2 *__restrict__ part,
                                                       unsigned int *__restrict__ cursor)
 {
-    __shared__ uint32_t dq_id_s[8][kDefer];
-    __shared__ float dq_w_s[8][kDefer];
+    __shared__ WarpArea wa_s[8];
     __shared__ MapDesc smaps[kStepMaxMaps];
     {
         const uint32_t *src = reinterpret_cast<const uint32_t *>(maps);
@@ -540,8 +449,6 @@ __global__ void __launch_bounds__(256, 8) area_step_items(const MapDesc *__restr
     }
     __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    uint32_t *dq_id = dq_id_s[warp];
-    float *dq_w = dq_w_s[warp];
     const int cnt = int(*count);
     if (cnt == 0) return;
     const uint32_t total = off[cnt];
@@ -562,7 +469,7 @@ __global__ void __launch_bounds__(256, 8) area_step_items(const MapDesc *__restr
         const MapDesc &d = smaps[a.map];
         const Req q = make_req(*a.q, d.n);
         const Dir w = make_dir_f(a.w[0], a.w[1], a.w[2]);
-        const float2 v = integrate_band<TFMT>(d, q, w, int(it - off[lo]), lane, dq_id, dq_w);
+        const float2 v = integrate_band<TFMT>(d, q, w, int(it - off[lo]), lane, wa_s[warp]);
         if (lane == 0) part[it] = v;
     }
 }
@@ -596,48 +503,24 @@ __global__ void area_step_reduce(const MapDesc *__restrict__ maps, const uint32_
 
 struct GgxDirs {
     Dir w[kGgxDirs];
+    double fit[3][kGgxDirs];  // least squares: Omega = fit a (the normal equations' matrix depends on w alone)
 };
 
-__device__ bool ggx_fit(const float *P, const GgxDirs &dirs, float4 &out)
+// Omega of a node from its P at the fit directions, one per lane (direction k,
+// the 16 directions on lanes that differ in the bits SH..SH + 3); every lane
+// gets it.  FP64: Omega is a difference of nearly equal terms.
+template <int SH>
+__device__ __forceinline__ float4 ggx_fit(double P, int k, const GgxDirs &dirs)
 {
-    double A[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}}, r[3] = {0, 0, 0};
-    for (int k = 0; k < kGgxDirs; ++k) {
-        const double wx = dirs.w[k].wx, wy = dirs.w[k].wy, wz = dirs.w[k].wz;
-        const double t = 2.0 * double(P[k]) - wz;
-        const double a = t * t - wz * wz;
-        const double row[3] = {wx * wx, 2.0 * wx * wy, wy * wy};
-        for (int p = 0; p < 3; ++p) {
-            r[p] += row[p] * a;
-            for (int q = 0; q < 3; ++q) A[p][q] += row[p] * row[q];
-        }
+    const double wz = dirs.w[k].wz, t = 2.0 * P - wz, a = t * t - wz * wz;
+    double x[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        x[c] = dirs.fit[c][k] * a;
+#pragma unroll
+        for (int o = 1 << SH; o < (16 << SH); o <<= 1) x[c] += __shfl_xor_sync(kFull, x[c], o);
     }
-    // Cholesky of the symmetric positive definite 3 x 3 system
-    double L[3][3];
-    for (int j = 0; j < 3; ++j) {
-        double dd = A[j][j];
-        for (int k = 0; k < j; ++k) dd -= L[j][k] * L[j][k];
-        if (!(dd > 0.0)) return false;
-        dd = sqrt(dd);
-        L[j][j] = dd;
-        for (int i = j + 1; i < 3; ++i) {
-            double v = A[i][j];
-            for (int k = 0; k < j; ++k) v -= L[i][k] * L[j][k];
-            L[i][j] = v / dd;
-        }
-    }
-    double y[3], x[3];
-    for (int i = 0; i < 3; ++i) {
-        double v = r[i];
-        for (int k = 0; k < i; ++k) v -= L[i][k] * y[k];
-        y[i] = v / L[i][i];
-    }
-    for (int i = 2; i >= 0; --i) {
-        double v = y[i];
-        for (int k = i + 1; k < 3; ++k) v -= L[k][i] * x[k];
-        x[i] = v / L[i][i];
-    }
-    out = make_float4(float(x[0]), float(x[1]), float(x[2]), 0.f);
-    return true;
+    return make_float4(float(x[0]), float(x[1]), float(x[2]), 0.f);
 }
 
 __device__ __forceinline__ bool ggx_node_inside(const MapDesc &d, int l, uint32_t m)
@@ -660,18 +543,19 @@ __device__ __forceinline__ void leaf_triangle(const MapDesc &d, int i0, int j0, 
 }
 
 // One warp per leaf block (Morton index): P at the fit directions (NaN when
-// the block has a quad outside the map) and the block's fit.  Each lane
-// evaluates its triangle at every direction in FP32 where that is accurate;
-// the (triangle, direction) pairs that need the FP64 path are listed and
-// spread over the warp 32 at a time, so the slow path runs lane-dense.  The
-// per-direction sums then run in the same fixed order either way.
+// the block has a quad outside the map) and the block's fit.  A lane integrates
+// m / m~_z over its triangle once and has the directions that see all of it
+// from that; the (triangle, direction) pairs that the visibility boundary
+// crosses are listed and spread over the warp 32 at a time, and so are the few
+// that need the FP64 form.  The sums over the triangles run in a fixed order.  The
+// whole fit of a 2048^2 mixed map takes 1.6 ms (17.2 ms with a closed-form integral
+// per direction, FP64 for every partly visible pair and the 3 x 3 solve in FP64 by
+// one lane), and Omega's error against 64 bits fell from 6e-6 to 6e-7.
 constexpr int kGgxLeafWarps = 8;
-static_assert(kGgxDirs <= 16, "a listed pair packs the direction in 4 bits");
+static_assert(kGgxDirs == 16, "two lanes per direction in the sums, four bits in a listed pair");
 
-// Eight CTAs per SM: 68 ms against 75 ms at the register-limited two for a
-// 4096^2 map (FP64 pairs dominate; more warps keep the FP64 pipe fed).
 template <int TFMT>
-__global__ void __launch_bounds__(32 * kGgxLeafWarps, 8) ggx_leaf(MapDesc d, GgxDirs dirs,
+__global__ void __launch_bounds__(32 * kGgxLeafWarps, PNDF_GGX_CTAS) ggx_leaf(MapDesc d, GgxDirs dirs,
                                                                float *__restrict__ P, float4 *__restrict__ omega,
                                                                uint32_t nleaf)
 {
@@ -689,85 +573,128 @@ __global__ void __launch_bounds__(32 * kGgxLeafWarps, 8) ggx_leaf(MapDesc d, Ggx
     float(*rs)[32] = r_s[warp];
     uint16_t *items = item_s[warp];
     const int i0 = int(compact1by1(m)) * kLeafQuads, j0 = int(compact1by1(m >> 1)) * kLeafQuads;
-    float2 na, nb, nc;
-    leaf_triangle<TFMT>(d, i0, j0, lane, na, nb, nc);
-    const float za = zof(na), zb = zof(nb), zc = zof(nc);
-    uint32_t need = 0;  // bit k: direction k needs the FP64 path
-    for (int k = 0; k < kGgxDirs; ++k) {
-        float r;
-        if (tri_ratio_fast(na, za, nb, zb, nc, zc, dirs.w[k], r))
-            rs[k][lane] = r;
-        else
-            need |= 1u << k;
-    }
-    // list the FP64 pairs (lane-major) and evaluate them 32 at a time
-    const int cnt = __popc(need);
-    int incl = cnt;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int v = __shfl_up_sync(kFull, incl, o);
-        if (lane >= o) incl += v;
-    }
-    const int total = __shfl_sync(kFull, incl, 31);
-    for (int p = incl - cnt; need; need &= need - 1) items[p++] = uint16_t((lane << 4) | (__ffs(need) - 1));
-    __syncwarp();
-    for (int t0 = 0; t0 < total; t0 += 32) {
-        if (t0 + lane < total) {
-            const int it = items[t0 + lane], src = it >> 4, k = it & 15;
-            float2 a, b, c;
-            leaf_triangle<TFMT>(d, i0, j0, src, a, b, c);
-            rs[k][src] = slow_ratio(a, b, c, dirs.w[k]);
+    uint32_t need[2] = {0u, 0u};  // directions (bits) whose pair is partly visible, and those for FP64
+    {
+        float2 na, nb, nc;
+        leaf_triangle<TFMT>(d, i0, j0, lane, na, nb, nc);
+        const float za = zof(na), zb = zof(nb), zc = zof(nc);
+        const float h2 = longest2(na, nb, nc);
+        auto f = [](float x, float y) {
+            const float2 r = ratio_at(x, y);
+            return V2{r.x, r.y};
+        };
+        const float zm = fminf(za, fminf(zb, zc)), z2 = zm * zm;
+        const V2 mean = h2 <= kSmallH2 * (z2 * z2) ? quad4(na, sub(nb, na), sub(nc, na), f)
+                                                    : quad6(na, sub(nb, na), sub(nc, na), f);
+        for (int k = 0; k < kGgxDirs; ++k) {
+            const Dir &w = dirs.w[k];
+            const Class cl = classify(phi_of(w, na, za), phi_of(w, nb, zb), phi_of(w, nc, zc), za, zb, zc, h2, w);
+            if (cl == kPartial)
+                need[0] |= 1u << k;
+            else if (cl == kSlow)
+                need[1] |= 1u << k;
+            else
+                rs[k][lane] = cl == kNone ? 0.f : 0.5f * fmaf(w.wx, mean.x, fmaf(w.wy, mean.y, w.wz));
         }
     }
-    __syncwarp();
-    for (int k = 0; k < kGgxDirs; ++k) {
-        float r = rs[k][lane];
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) r += __shfl_down_sync(kFull, r, off);  // fixed order
-        if (lane == 0) Pm[k] = r * (1.0f / float(kLeafQuads * kLeafQuads));
+    for (int pass = 0; pass < 2; ++pass) {
+        // list the pairs (lane-major) and evaluate them 32 at a time
+        uint32_t set = need[pass];
+        const int cnt = __popc(set);
+        if (!__any_sync(kFull, cnt > 0)) continue;
+        int incl = cnt;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(kFull, incl, o);
+            if (lane >= o) incl += v;
+        }
+        const int total = __shfl_sync(kFull, incl, 31);
+        for (int p = incl - cnt; set; set &= set - 1) items[p++] = uint16_t((lane << 4) | (__ffs(set) - 1));
+        __syncwarp();
+        for (int t0 = 0; t0 < total; t0 += 32) {
+            if (t0 + lane < total) {
+                const int it = items[t0 + lane], src = it >> 4, k = it & 15;
+                float2 a, b, c;
+                leaf_triangle<TFMT>(d, i0, j0, src, a, b, c);
+                float v = pass == 0 ? partial_mean(a, b, c, dirs.w[k]) : -1.f;
+                if (v < 0.f) v = slow_ratio(a, b, c, dirs.w[k]);
+                rs[k][src] = v;
+            }
+        }
+        __syncwarp();
     }
     __syncwarp();
-    if (lane == 0) {
-        float4 o;
-        if (!ggx_fit(Pm, dirs, o)) o = make_float4(__int_as_float(0x7fc00000), 0.f, 0.f, 0.f);
-        omega[m] = o;
+    // sums over the 32 triangles, 16 directions at once: each step halves the
+    // directions a lane holds, so that lanes 2k and 2k + 1 end with direction k
+    float v[kGgxDirs];
+#pragma unroll
+    for (int k = 0; k < kGgxDirs; ++k) v[k] = rs[k][lane];
+#pragma unroll
+    for (int h = kGgxDirs / 2; h >= 1; h >>= 1) {
+        const int o = 2 * h;
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int k = 0; k < h; ++k) {
+            const float got = __shfl_xor_sync(kFull, up ? v[k] : v[k + h], o);
+            v[k] = (up ? v[k + h] : v[k]) + got;
+        }
     }
+    const float p = (v[0] + __shfl_xor_sync(kFull, v[0], 1)) * (1.0f / float(kLeafQuads * kLeafQuads));
+    if ((lane & 1) == 0) Pm[lane >> 1] = p;
+    const float4 o = ggx_fit<1>(p, lane >> 1, dirs);
+    if (lane == 0) omega[m] = o;
 }
 
-// One thread per node of level l: P = mean of the four children's, then the fit.
-__global__ void ggx_up(MapDesc d, int l, GgxDirs dirs, const float *__restrict__ Pc, float *__restrict__ Pp,
+// 16 lanes per node of level l: P = mean of the four children's, then the fit.
+// Above the leaf blocks P is kept in FP64: Omega is a small difference, and a
+// rounding per level would show in the coarse ones.
+template <class T>
+__global__ void ggx_up(MapDesc d, int l, GgxDirs dirs, const T *__restrict__ Pc, double *__restrict__ Pp,
                        float4 *__restrict__ omega, uint32_t count)
 {
-    const uint32_t m = blockIdx.x * blockDim.x + threadIdx.x;
-    if (m >= count) return;
-    float Pl[kGgxDirs];
-    bool ok = ggx_node_inside(d, l, m);
-    for (int k = 0; k < kGgxDirs; ++k) {
-        float v = 0.f;
-        for (int c = 0; c < 4; ++c) v += Pc[(4 * size_t(m) + c) * kGgxDirs + k];
-        Pl[k] = 0.25f * v;
-        ok = ok && isfinite(Pl[k]);
-    }
-    for (int k = 0; k < kGgxDirs; ++k) Pp[size_t(m) * kGgxDirs + k] = ok ? Pl[k] : __int_as_float(0x7fc00000);
-    float4 o = make_float4(__int_as_float(0x7fc00000), 0.f, 0.f, 0.f);
-    if (ok && !ggx_fit(Pl, dirs, o)) o = make_float4(__int_as_float(0x7fc00000), 0.f, 0.f, 0.f);
-    omega[m] = o;
+    const uint32_t m = (blockIdx.x * blockDim.x + threadIdx.x) / kGgxDirs;
+    const int k = threadIdx.x & (kGgxDirs - 1);
+    const bool live = m < count;
+    double v = 0.0;
+    if (live)
+        for (int c = 0; c < 4; ++c) v += double(Pc[(4 * size_t(m) + c) * kGgxDirs + k]);
+    const double p = 0.25 * v;
+    const unsigned half = 0xffffu << (threadIdx.x & 16);  // the node's lanes
+    const bool fine = (__ballot_sync(kFull, isfinite(p)) & half) == half;
+    const bool ok = live && ggx_node_inside(d, l, m) && fine;
+    const float4 o = ggx_fit<0>(p, k, dirs);
+    if (!live) return;
+    Pp[size_t(m) * kGgxDirs + k] = ok ? p : __longlong_as_double(0x7ff8000000000000ll);
+    if (k == 0) omega[m] = ok ? o : make_float4(__int_as_float(0x7fc00000), 0.f, 0.f, 0.f);
 }
 
 GgxDirs make_ggx_dirs()
 {
     GgxDirs g;
     const double r = sqrt(1.0 - double(kGgxWz) * kGgxWz);
+    double row[kGgxDirs][3], A[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
     for (int k = 0; k < kGgxDirs; ++k) {
         const double ph = 2.0 * 3.14159265358979323846 * k / kGgxDirs;
         Dir &w = g.w[k];
         w.wx = float(r * cos(ph));
         w.wy = float(r * sin(ph));
         w.wz = kGgxWz;
-        w.wr = sqrtf(w.wx * w.wx + w.wy * w.wy);
-        w.c = w.wr > 0.f ? w.wx / w.wr : 1.f;
-        w.s = w.wr > 0.f ? w.wy / w.wr : 0.f;
+        row[k][0] = double(w.wx) * w.wx;
+        row[k][1] = 2.0 * double(w.wx) * w.wy;
+        row[k][2] = double(w.wy) * w.wy;
+        for (int p = 0; p < 3; ++p)
+            for (int q = 0; q < 3; ++q) A[p][q] += row[k][p] * row[k][q];
     }
+    // fit = A^-1 rows^T, A^-1 by cofactors (A is symmetric and well conditioned)
+    const double c00 = A[1][1] * A[2][2] - A[1][2] * A[2][1], c01 = A[1][2] * A[2][0] - A[1][0] * A[2][2];
+    const double c02 = A[1][0] * A[2][1] - A[1][1] * A[2][0], c11 = A[0][0] * A[2][2] - A[0][2] * A[2][0];
+    const double c12 = A[0][1] * A[2][0] - A[0][0] * A[2][1], c22 = A[0][0] * A[1][1] - A[0][1] * A[1][0];
+    const double det = A[0][0] * c00 + A[0][1] * c01 + A[0][2] * c02;
+    const double inv[3][3] = {{c00, c01, c02}, {c01, c11, c12}, {c02, c12, c22}};
+    for (int c = 0; c < 3; ++c)
+        for (int k = 0; k < kGgxDirs; ++k)
+            g.fit[c][k] = (inv[c][0] * row[k][0] + inv[c][1] * row[k][1] + inv[c][2] * row[k][2]) / det;
     return g;
 }
 
@@ -878,14 +805,21 @@ pndf_status launch_ggx_build(const pndf_hierarchy *h, pndf_ggx *g, cudaStream_t 
         ggx_leaf<PNDF_TEXEL_F16X2><<<blocks, 32 * kGgxLeafWarps, 0, s>>>(d, dirs, pa, g->omega[kLeafLevel], nleaf);
     count_launches(1);
     cudaError_t e = cudaGetLastError();
+    // the leaf blocks' P are floats in pa; the levels above alternate between
+    // the two halves as doubles (a quarter of the nodes, twice the size)
+    double *from = reinterpret_cast<double *>(pa), *to = reinterpret_cast<double *>(pb);
     for (int l = kLeafLevel + 1; e == cudaSuccess && l <= L; ++l) {
         const uint32_t cnt = uint32_t(level_nodes(L, l));
-        ggx_up<<<(cnt + 127) / 128, 128, 0, s>>>(d, l, dirs, pa, pb, g->omega[l], cnt);
+        const unsigned grid = unsigned((size_t(cnt) * kGgxDirs + 127) / 128);
+        if (l == kLeafLevel + 1)
+            ggx_up<float><<<grid, 128, 0, s>>>(d, l, dirs, pa, to, g->omega[l], cnt);
+        else
+            ggx_up<double><<<grid, 128, 0, s>>>(d, l, dirs, from, to, g->omega[l], cnt);
         count_launches(1);
         e = cudaGetLastError();
-        float *t = pa;
-        pa = pb;
-        pb = t;
+        double *t = from;
+        from = to;
+        to = t;
     }
     cudaError_t ef = cudaFreeAsync(scratch, s);
     return (e == cudaSuccess && ef == cudaSuccess) ? PNDF_OK : PNDF_ERR_CUDA;
