@@ -13,7 +13,8 @@
 //
 // A triangle the boundary w . m~ = 0 crosses is cut along it into straight and
 // curved pieces, each again a positive smooth integral (partial_mean).  Larger
-// triangles go to the closed form in FP64 (visible.cuh).
+// triangles are split in four at their edges' midpoints; what is still too
+// large goes to the closed form in FP64 (visible.cuh).
 #pragma once
 
 namespace pndf {
@@ -97,7 +98,7 @@ __device__ __forceinline__ float len2(float2 v) { return fmaf(v.x, v.x, v.y * v.
 __device__ __forceinline__ float2 sub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
 
 // How a triangle is integrated.
-enum Class : int { kNone, kSmall, kLarge, kPartial, kSlow };
+enum Class : int { kNone, kSmall, kLarge, kPartial, kSplit };
 
 // Class of a triangle with phi = w . m~ and m~_z at its vertices, longest edge
 // squared h2.  m~_z is concave with second derivative at most 1 / m~_z^3, so
@@ -109,9 +110,9 @@ __device__ __forceinline__ Class classify(float fa, float fb, float fc, float za
 {
     const float zm = fminf(za, fminf(zb, zc)), z2 = zm * zm;
     const float s2 = z2 * z2;  // h^2 = h2 / s2
-    if (fminf(fa, fminf(fb, fc)) >= 0.f) return h2 <= kSmallH2 * s2 ? kSmall : h2 <= kLargeH2 * s2 ? kLarge : kSlow;
+    if (fminf(fa, fminf(fb, fc)) >= 0.f) return h2 <= kSmallH2 * s2 ? kSmall : h2 <= kLargeH2 * s2 ? kLarge : kSplit;
     if (fmaf(fmaxf(fa, fmaxf(fb, fc)) + 5e-7f, 6.f * z2 * zm, w.wz * h2) < 0.f) return kNone;
-    return h2 <= kLargeH2 * s2 ? kPartial : kSlow;
+    return h2 <= kLargeH2 * s2 ? kPartial : kSplit;
 }
 
 // Where the segment m + t d leaves (m visible) or enters (m not visible) the
@@ -166,7 +167,7 @@ __constant__ float kGw5[5] = {0.118463442528095f, 0.239314335249683f, 0.28444444
 // error against 64 bits, FP32 rounding included, 2e-9 (h up to 0.4) to 2e-8
 // (0.8).  Clipped in FP64, the same 2% of all triangles kept the kernel's FP64
 // pipe 53% busy and took most of its time.
-__device__ __forceinline__ float partial_mean(float2 a, float2 b, float2 c, const Dir &w)
+__device__ __noinline__ float partial_mean(float2 a, float2 b, float2 c, const Dir &w)
 {
     float fa = phi_of(w, a, zof(a)), fb = phi_of(w, b, zof(b)), fc = phi_of(w, c, zof(c));
     const bool va = fa >= 0.f, vb = fb >= 0.f, vc = fc >= 0.f;

@@ -16,8 +16,9 @@
 //    every edge);
 //  * otherwise cut along the visibility boundary into smooth pieces
 //    (partial_mean);
-//  * very large triangles: the closed form of visible.cuh in FP64 (the clip of
-//    Alg. 1, Eq. 11's boundary integral, the segment form of Eq. 13).
+//  * larger triangles are split in four, each part classified again; a part that
+//    is still too large takes the closed form of visible.cuh in FP64 (the clip
+//    of Alg. 1, Eq. 11's boundary integral, the segment form of Eq. 13).
 // All but the first kind and the zeros are deferred into per-warp rings and
 // evaluated 32 at a time, so that each runs lane-dense.
 //
@@ -47,7 +48,7 @@ constexpr unsigned kFull = 0xffffffffu;
 #endif
 constexpr int kBand = 8;                 // quad rows per work item
 
-// V_T / |cross| in closed form (visible.cuh, FP64): the triangles of class kSlow;
+// V_T / |cross| in closed form (visible.cuh, FP64), for the largest triangles;
 // the segment form of Eq. 13 where the normals collapsed (|cross| < 1e-12).
 __device__ __noinline__ float slow_ratio(float2 a, float2 b, float2 c, const Dir &wf)
 {
@@ -143,7 +144,7 @@ __device__ __forceinline__ float2 texel(const MapDesc &d, int i, int j)
 // Deferred triangles, one ring per class and warp: (i << 15) | (j << 1) | tri and
 // the kernel weight; at most 31 held over plus one step's 64.
 constexpr int kDefer = 128;
-constexpr int kRings = 3;  // kLarge, kPartial, kSlow
+constexpr int kRings = 3;  // kLarge, kPartial, kSplit
 struct WarpArea {
     uint32_t id[kRings][kDefer];
     float wt[kRings][kDefer];
@@ -176,6 +177,37 @@ __device__ __forceinline__ float full_mean_large(float2 a, float2 b, float2 c, c
     return fmaf(0.5f, quad6(a, sub(b, a), sub(c, a), [&](float x, float y) { return slope_at(w, x, y); }), 0.5f * w.wz);
 }
 
+// V_T / |cross| of a triangle of class kPartial.
+__device__ __forceinline__ float partial_ratio(float2 a, float2 b, float2 c, const Dir &w)
+{
+    const float v = partial_mean(a, b, c, w);
+    return v < 0.f ? slow_ratio(a, b, c, w) : v;
+}
+
+// V_T / |cross| of a triangle of class kSplit: the mean over its four parts.
+__device__ __noinline__ float split_ratio(float2 a, float2 b, float2 c, const Dir &w)
+{
+    const float2 ab = make_float2(0.5f * (a.x + b.x), 0.5f * (a.y + b.y));
+    const float2 bc = make_float2(0.5f * (b.x + c.x), 0.5f * (b.y + c.y));
+    const float2 ca = make_float2(0.5f * (c.x + a.x), 0.5f * (c.y + a.y));
+    float sum = 0.f;
+#pragma unroll 1
+    for (int k = 0; k < 4; ++k) {
+        const float2 p = k == 0 ? a : k == 1 ? ab : k == 2 ? ca : ab;
+        const float2 q = k == 0 ? ab : k == 1 ? b : k == 2 ? bc : bc;
+        const float2 r = k == 0 ? ca : k == 1 ? bc : k == 2 ? c : ca;
+        const float zp = zof(p), zq = zof(q), zr = zof(r);
+        const Class cl = classify(phi_of(w, p, zp), phi_of(w, q, zq), phi_of(w, r, zr), zp, zq, zr, longest2(p, q, r), w);
+        if (cl == kSmall || cl == kLarge)
+            sum += full_mean_large(p, q, r, w);
+        else if (cl == kPartial)
+            sum += partial_ratio(p, q, r, w);
+        else if (cl == kSplit)
+            sum += slow_ratio(p, q, r, w);
+    }
+    return 0.25f * sum;
+}
+
 // Lane's deferred triangle of ring r (slot head + lane): kernel weight times
 // V_T / |cross| (tri 0 = (u0, u1, u2), tri 1 = (u3, u2, u1)).
 template <int TFMT>
@@ -188,8 +220,7 @@ __device__ __forceinline__ float deferred_value(const MapDesc &d, const Dir &w, 
     const float2 a = texel<TFMT>(d, i + tri, j + tri);
     const float2 b = texel<TFMT>(d, i + 1 - tri, j + tri);
     const float2 c = texel<TFMT>(d, i + tri, j + 1 - tri);
-    float v = r == 0 ? full_mean_large(a, b, c, w) : r == 1 ? partial_mean(a, b, c, w) : -1.f;
-    if (r > 0 && v < 0.f) v = slow_ratio(a, b, c, w);
+    const float v = r == 0 ? full_mean_large(a, b, c, w) : r == 1 ? partial_ratio(a, b, c, w) : split_ratio(a, b, c, w);
     return wa.wt[r][slot] * v;
 }
 
@@ -337,7 +368,9 @@ __device__ __forceinline__ float2 integrate_band(const MapDesc &d, const Req &q,
 // quadrature points 80, classification and weights 80, row walk and sums 50, the
 // deferred classes 40).  Four CTAs per SM (64 registers): 192 requests on the
 // 16384^2 mixed map 13.5 ms, at three 14.3, at five and six 13.7, at eight 15.8;
-// with the FP64 path for every partly visible triangle it was 79 ms.
+// with the FP64 path for every partly visible triangle it was 79 ms.  Splitting the
+// larger triangles instead of taking them in FP64: 1000 small footprints on a
+// scratch map, whose grooves have many, 0.49 -> 0.34 ms.
 template <int TFMT>
 __global__ void __launch_bounds__(256, PNDF_PA_CTAS) pa_items(MapDesc d, const pndf_query *__restrict__ qs,
                                                const float *__restrict__ omega, int64_t k0, int cnt,
@@ -547,8 +580,8 @@ __device__ __forceinline__ void leaf_triangle(const MapDesc &d, int i0, int j0, 
 // m / m~_z over its triangle once and has the directions that see all of it
 // from that; the (triangle, direction) pairs that the visibility boundary
 // crosses are listed and spread over the warp 32 at a time, and so are the few
-// that need the FP64 form.  The sums over the triangles run in a fixed order.  The
-// whole fit of a 2048^2 mixed map takes 1.6 ms (17.2 ms with a closed-form integral
+// to be split.  The sums over the triangles run in a fixed order.  The
+// whole fit of a 2048^2 mixed map takes 1.1 ms (17.2 ms with a closed-form integral
 // per direction, FP64 for every partly visible pair and the 3 x 3 solve in FP64 by
 // one lane), and Omega's error against 64 bits fell from 6e-6 to 6e-7.
 constexpr int kGgxLeafWarps = 8;
@@ -573,7 +606,7 @@ __global__ void __launch_bounds__(32 * kGgxLeafWarps, PNDF_GGX_CTAS) ggx_leaf(Ma
     float(*rs)[32] = r_s[warp];
     uint16_t *items = item_s[warp];
     const int i0 = int(compact1by1(m)) * kLeafQuads, j0 = int(compact1by1(m >> 1)) * kLeafQuads;
-    uint32_t need[2] = {0u, 0u};  // directions (bits) whose pair is partly visible, and those for FP64
+    uint32_t need[2] = {0u, 0u};  // directions (bits) whose pair is partly visible, and those to split
     {
         float2 na, nb, nc;
         leaf_triangle<TFMT>(d, i0, j0, lane, na, nb, nc);
@@ -591,7 +624,7 @@ __global__ void __launch_bounds__(32 * kGgxLeafWarps, PNDF_GGX_CTAS) ggx_leaf(Ma
             const Class cl = classify(phi_of(w, na, za), phi_of(w, nb, zb), phi_of(w, nc, zc), za, zb, zc, h2, w);
             if (cl == kPartial)
                 need[0] |= 1u << k;
-            else if (cl == kSlow)
+            else if (cl == kSplit)
                 need[1] |= 1u << k;
             else
                 rs[k][lane] = cl == kNone ? 0.f : 0.5f * fmaf(w.wx, mean.x, fmaf(w.wy, mean.y, w.wz));
@@ -617,9 +650,7 @@ __global__ void __launch_bounds__(32 * kGgxLeafWarps, PNDF_GGX_CTAS) ggx_leaf(Ma
                 const int it = items[t0 + lane], src = it >> 4, k = it & 15;
                 float2 a, b, c;
                 leaf_triangle<TFMT>(d, i0, j0, src, a, b, c);
-                float v = pass == 0 ? partial_mean(a, b, c, dirs.w[k]) : -1.f;
-                if (v < 0.f) v = slow_ratio(a, b, c, dirs.w[k]);
-                rs[k][src] = v;
+                rs[k][src] = pass == 0 ? partial_ratio(a, b, c, dirs.w[k]) : split_ratio(a, b, c, dirs.w[k]);
             }
         }
         __syncwarp();
