@@ -62,25 +62,43 @@ __host__ __device__ constexpr double hat(int a, double s, double t)
                         : (a == 0 ? 0.0 : a == 1 ? 1.0 - t : a == 2 ? 1.0 - s : s + t - 1.0);
 }
 
-// Cholesky solve of G c = R (G packed symmetric).  False if G is not
+// 1 / x for x > 0: the FP32 reciprocal (relative error below 2^-22) and one
+// cubic step, three FP64 operations where a division takes about twelve.
+__host__ __device__ __forceinline__ double inv_pos(double x)
+{
+#ifdef __CUDA_ARCH__
+    if (x > 1e-30 && x < 1e30) {
+        const double r = double(__fdividef(1.0f, float(x)));
+        const double e = fma(-x, r, 1.0);
+        return fma(r, fma(e, e, e), r);
+    }
+#endif
+    return 1.0 / x;
+}
+
+// Solve of G c = R (G packed symmetric) by L D L^T.  False if G is not
 // numerically positive definite.
 __host__ __device__ bool solve_spd(const double Gp[10], const double R[4][2], double c[4][2])
 {
-    double L[4][4];
+    double L[4][4], inv[4];  // unit lower triangle; 1 / D
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
+        double u[4];  // L[j][k] D[k]
         double d = Gp[sym(j, j)];
 #pragma unroll
-        for (int k = 0; k < j; ++k) d -= L[j][k] * L[j][k];
+        for (int k = 0; k < j; ++k) {
+            u[k] = L[j][k];            // still multiplied by D[k]
+            L[j][k] = u[k] * inv[k];
+            d -= u[k] * L[j][k];
+        }
         if (!(d > 0.0)) return false;
-        d = sqrt(d);
-        L[j][j] = d;
+        inv[j] = inv_pos(d);
 #pragma unroll
         for (int i = j + 1; i < 4; ++i) {
             double v = Gp[sym(i, j)];
 #pragma unroll
             for (int k = 0; k < j; ++k) v -= L[i][k] * L[j][k];
-            L[i][j] = v / d;
+            L[i][j] = v;  // times D[j] until row i is reached
         }
     }
 #pragma unroll
@@ -88,17 +106,16 @@ __host__ __device__ bool solve_spd(const double Gp[10], const double R[4][2], do
         double y[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            double v = R[i][r];
+            y[i] = R[i][r];
 #pragma unroll
-            for (int k = 0; k < i; ++k) v -= L[i][k] * y[k];
-            y[i] = v / L[i][i];
+            for (int k = 0; k < i; ++k) y[i] -= L[i][k] * y[k];
         }
 #pragma unroll
         for (int i = 3; i >= 0; --i) {
-            double v = y[i];
+            double v = y[i] * inv[i];
 #pragma unroll
             for (int k = i + 1; k < 4; ++k) v -= L[k][i] * c[k][r];
-            c[i][r] = v / L[i][i];
+            c[i][r] = v;
         }
     }
     return true;
@@ -118,11 +135,11 @@ __device__ __forceinline__ float2 texel_at(const MapDesc &d, int i, int j)
     return __half22float2(__ldg(reinterpret_cast<const __half2 *>(d.texels) + idx));
 }
 
-// Fit of leaf block (I, J) (4 x 4 quads), all of whose quads lie in the map.
-// Returns false if the normal equations are singular.
-// Fit of a leaf block (4 x 4 quads) from its 5 x 5 texels tx[y][x].
-// Returns false if the normal equations are singular.
-__host__ __device__ bool leaf_fit_texels(const float2 (&tx)[kLeafQuads + 1][kLeafQuads + 1], QF &out)
+// Fit of a leaf block (4 x 4 quads) from its 5 x 5 texels tx[y][x].  The 32
+// triangles' weights wait in wt (element t at wt[t * stride]) between the two
+// passes.  Returns false if the normal equations are singular.
+__host__ __device__ __forceinline__ bool leaf_fit_texels(const float2 (&tx)[kLeafQuads + 1][kLeafQuads + 1], QF &out,
+                                                         double *wt, int stride)
 {
     constexpr int Q = kLeafQuads;
     double G[10], R[4][2];
@@ -149,7 +166,8 @@ __host__ __device__ bool leaf_fit_texels(const float2 (&tx)[kLeafQuads + 1][kLea
                     for (int k = 0; k < 3; ++k) h[v][k] = hat(base + k, double(x) / Q, double(y) / Q);
                 }
                 const double cr = (nx[1] - nx[0]) * (ny[2] - ny[0]) - (ny[1] - ny[0]) * (nx[2] - nx[0]);
-                const double w = (1.0 / 24.0) / fmax(fabs(cr), kJacEps);
+                const double w = (1.0 / 24.0) * inv_pos(fmax(fabs(cr), kJacEps));
+                wt[((qj * Q + qi) * 2 + tri) * stride] = w;
                 const double sx = nx[0] + nx[1] + nx[2], sy = ny[0] + ny[1] + ny[2];
 #pragma unroll
                 for (int k = 0; k < 3; ++k) {
@@ -190,8 +208,7 @@ __host__ __device__ bool leaf_fit_texels(const float2 (&tx)[kLeafQuads + 1][kLea
                     dx[v] = ax - nx[v];
                     dy[v] = ay - ny[v];
                 }
-                const double cr = (nx[1] - nx[0]) * (ny[2] - ny[0]) - (ny[1] - ny[0]) * (nx[2] - nx[0]);
-                const double w = (1.0 / 24.0) / fmax(fabs(cr), kJacEps);
+                const double w = wt[((qj * Q + qi) * 2 + tri) * stride];
                 const double sx = dx[0] + dx[1] + dx[2], sy = dy[0] + dy[1] + dy[2];
                 F += w * (dx[0] * dx[0] + dx[1] * dx[1] + dx[2] * dx[2] + dy[0] * dy[0] + dy[1] * dy[1] +
                           dy[2] * dy[2] + sx * sx + sy * sy);
@@ -204,7 +221,7 @@ __host__ __device__ bool leaf_fit_texels(const float2 (&tx)[kLeafQuads + 1][kLea
 
 // Fit of leaf block (I, J), all of whose quads lie in the map.
 template <int TFMT>
-__device__ bool leaf_fit(const MapDesc &d, uint32_t I, uint32_t J, QF &out)
+__device__ __forceinline__ bool leaf_fit(const MapDesc &d, uint32_t I, uint32_t J, QF &out, double *wt, int stride)
 {
     constexpr int Q = kLeafQuads;
     const int i0 = int(I) * Q, j0 = int(J) * Q;
@@ -213,7 +230,7 @@ __device__ bool leaf_fit(const MapDesc &d, uint32_t I, uint32_t J, QF &out)
     for (int y = 0; y <= Q; ++y)
 #pragma unroll
         for (int x = 0; x <= Q; ++x) tx[y][x] = texel_at<TFMT>(d, i0 + x, j0 + y);
-    return leaf_fit_texels(tx, out);
+    return leaf_fit_texels(tx, out, wt, stride);
 }
 
 // Child (ox, oy) of a parent: P[j][a] = parent hat a at child corner j, in
@@ -411,6 +428,7 @@ constexpr int kTileThreads = 1 << (2 * kTileLevels);  // 256 leaf blocks
 template <int TFMT, int BFMT>
 __global__ void __launch_bounds__(kTileThreads, 2) cluster_tiles(MapDesc d, ClusterDesc cd, QF *__restrict__ out6)
 {
+    extern __shared__ double wt_s[];  // [32][kTileThreads]
     __shared__ QF part[16];
     __shared__ bool part_ok[16];
     const int tid = threadIdx.x;
@@ -420,7 +438,8 @@ __global__ void __launch_bounds__(kTileThreads, 2) cluster_tiles(MapDesc d, Clus
     QF m;
     bool ok = false;
     if (m2 < n2) {
-        ok = node_inside_map(d, kLeafLevel, m2) && leaf_fit<TFMT>(d, compact1by1(m2), compact1by1(m2 >> 1), m);
+        ok = node_inside_map(d, kLeafLevel, m2) && leaf_fit<TFMT>(d, compact1by1(m2), compact1by1(m2 >> 1), m, wt_s + tid,
+                                                             kTileThreads);
         fit_store<BFMT>(d, cd, kLeafLevel, m2, ok, m);
     }
     if (!ok) {  // keep the shuffled sums finite; such a node's ancestors are never fitted
@@ -509,9 +528,12 @@ cudaError_t launch_clusters_t(pndf_hierarchy *h, cudaStream_t s)
     const unsigned blocks = L >= top_tile ? unsigned(level_nodes(L, top_tile)) : 1u;
     QF *a = static_cast<QF *>(h->moments);
     QF *b = a ? a + level_nodes(L, top_tile) : nullptr;
-    cluster_tiles<TFMT, BFMT><<<blocks, kTileThreads, 0, s>>>(d, h->c, L > top_tile ? a : nullptr);
+    constexpr size_t smem = 32 * kTileThreads * sizeof(double);  // 64 KB, past the 48 KB a launch gets by default
+    cudaError_t e = cudaFuncSetAttribute(cluster_tiles<TFMT, BFMT>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    if (e != cudaSuccess) return e;
+    cluster_tiles<TFMT, BFMT><<<blocks, kTileThreads, smem, s>>>(d, h->c, L > top_tile ? a : nullptr);
     count_launches(1);
-    cudaError_t e = cudaGetLastError();
+    e = cudaGetLastError();
     for (int l = top_tile + 1; e == cudaSuccess && l <= L; ++l) {
         const uint32_t cnt = uint32_t(level_nodes(L, l));
         cluster_up<BFMT><<<(cnt + 127) / 128, 128, 0, s>>>(d, h->c, l, a, l < L ? b : nullptr, cnt);
