@@ -41,6 +41,9 @@ namespace pndf {
 namespace {
 
 constexpr double kJacEps = 1e-6;
+#ifndef PNDF_CL_CTAS
+#define PNDF_CL_CTAS 2
+#endif
 
 // A node's quadratic form at its optimum: Gram matrix G (symmetric, upper
 // triangle packed: 00 01 02 03 11 12 13 22 23 33), optimal corners g
@@ -67,8 +70,9 @@ __host__ __device__ constexpr double hat(int a, double s, double t)
 __host__ __device__ __forceinline__ double inv_pos(double x)
 {
 #ifdef __CUDA_ARCH__
-    if (x > 1e-30 && x < 1e30) {
-        const double r = double(__fdividef(1.0f, float(x)));
+    const float xf = float(x);
+    if (xf > 1e-30f && xf < 1e30f) {
+        const double r = double(__fdividef(1.0f, xf));
         const double e = fma(-x, r, 1.0);
         return fma(r, fma(e, e, e), r);
     }
@@ -135,84 +139,126 @@ __device__ __forceinline__ float2 texel_at(const MapDesc &d, int i, int j)
     return __half22float2(__ldg(reinterpret_cast<const __half2 *>(d.texels) + idx));
 }
 
-// Fit of a leaf block (4 x 4 quads) from its 5 x 5 texels tx[y][x].  The 32
-// triangles' weights wait in wt (element t at wt[t * stride]) between the two
-// passes.  Returns false if the normal equations are singular.
+// Fit of a leaf block (4 x 4 quads) from its 5 x 5 texels tx[y][x]; the forms G and
+// F carry a factor 24 (fit_store takes it out of the residual), so a triangle's
+// weight is 1 / max(|cross|, 1e-6).  The 32 weights wait in wt (element t at wt[t *
+// stride]) between the two passes.  Returns false if the normal equations are
+// singular.
+//
+// The kernel is bound by FP64 issue, so the sums are arranged for few operations:
+// with S the sum of a triangle's normals n0, n1, n2 and (i, j) its quad, the right
+// hand sides of the hats s and t of either half are moments of w S, w n1 and w n2,
+//     sum w (sum_v s_v n_v + (sum_v s_v) S) = 1/4 sum w ((4 i + 1) S + n1)   lower
+//                                           = 1/4 sum w ((4 i + 3) S - n1)   upper triangle
+// (t alike with j and n2), and those of 1 are 4 sum w S; the second pass takes the
+// misfit at each texel once, not at each triangle's vertices.
 __host__ __device__ __forceinline__ bool leaf_fit_texels(const float2 (&tx)[kLeafQuads + 1][kLeafQuads + 1], QF &out,
                                                          double *wt, int stride)
 {
     constexpr int Q = kLeafQuads;
-    double G[10], R[4][2];
+    double G[10];
+    double A[2][2], X[2][2], Y[2][2];  // per cluster half and component: sums of w S and the moments above
 #pragma unroll
     for (int k = 0; k < 10; ++k) G[k] = 0.0;
 #pragma unroll
-    for (int a = 0; a < 4; ++a) R[a][0] = R[a][1] = 0.0;
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int c = 0; c < 2; ++c) A[h][c] = X[h][c] = Y[h][c] = 0.0;
     // pass 1: normal equations
 #pragma unroll
     for (int qj = 0; qj < Q; ++qj)
 #pragma unroll
-        for (int qi = 0; qi < Q; ++qi)
+        for (int qi = 0; qi < Q; ++qi) {
+            const double u[4][2] = {{tx[qj][qi].x, tx[qj][qi].y},
+                                    {tx[qj][qi + 1].x, tx[qj][qi + 1].y},
+                                    {tx[qj + 1][qi].x, tx[qj + 1][qi].y},
+                                    {tx[qj + 1][qi + 1].x, tx[qj + 1][qi + 1].y}};
+            const double mid[2] = {u[1][0] + u[2][0], u[1][1] + u[2][1]};
 #pragma unroll
             for (int tri = 0; tri < 2; ++tri) {
+                // tri 0: (u0, u1, u2), tri 1: (u3, u2, u1)
+                const double(&n0)[2] = u[tri ? 3 : 0];
+                const double(&n1)[2] = u[tri ? 2 : 1];
+                const double(&n2)[2] = u[tri ? 1 : 2];
                 // cluster half by the centroid: lower iff qi + qj <= Q - 1 (tri 0), Q - 2 (tri 1)
-                const int base = qi + qj <= Q - 1 - tri ? 0 : 1;  // active hats base..base+2
-                double nx[3], ny[3], h[3][3];
-#pragma unroll
-                for (int v = 0; v < 3; ++v) {
-                    const int x = vx(qi, tri, v), y = vy(qj, tri, v);
-                    nx[v] = tx[y][x].x;
-                    ny[v] = tx[y][x].y;
-#pragma unroll
-                    for (int k = 0; k < 3; ++k) h[v][k] = hat(base + k, double(x) / Q, double(y) / Q);
-                }
-                const double cr = (nx[1] - nx[0]) * (ny[2] - ny[0]) - (ny[1] - ny[0]) * (nx[2] - nx[0]);
-                const double w = (1.0 / 24.0) * inv_pos(fmax(fabs(cr), kJacEps));
+                const int half = qi + qj <= Q - 1 - tri ? 0 : 1;
+                const double cr = (n1[0] - n0[0]) * (n2[1] - n0[1]) - (n1[1] - n0[1]) * (n2[0] - n0[0]);
+                const double w = inv_pos(fmax(fabs(cr), kJacEps));
                 wt[((qj * Q + qi) * 2 + tri) * stride] = w;
-                const double sx = nx[0] + nx[1] + nx[2], sy = ny[0] + ny[1] + ny[2];
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {
+                    const double wS = w * (mid[c] + n0[c]);
+                    A[half][c] += wS;
+                    X[half][c] += (4 * qi + (tri ? 3 : 1)) * wS;
+                    Y[half][c] += (4 * qj + (tri ? 3 : 1)) * wS;
+                    X[half][c] += tri ? -w * n1[c] : w * n1[c];
+                    Y[half][c] += tri ? -w * n2[c] : w * n2[c];
+                }
+                double h[3][3];
+#pragma unroll
+                for (int v = 0; v < 3; ++v)
+#pragma unroll
+                    for (int k = 0; k < 3; ++k)
+                        h[v][k] = hat(half + k, double(vx(qi, tri, v)) / Q, double(vy(qj, tri, v)) / Q);
 #pragma unroll
                 for (int k = 0; k < 3; ++k) {
                     const double hk = h[0][k] + h[1][k] + h[2][k];
-                    R[base + k][0] += w * (h[0][k] * nx[0] + h[1][k] * nx[1] + h[2][k] * nx[2] + hk * sx);
-                    R[base + k][1] += w * (h[0][k] * ny[0] + h[1][k] * ny[1] + h[2][k] * ny[2] + hk * sy);
 #pragma unroll
                     for (int k2 = k; k2 < 3; ++k2) {
                         const double hk2 = h[0][k2] + h[1][k2] + h[2][k2];
-                        G[sym(base + k, base + k2)] +=
+                        G[sym(half + k, half + k2)] +=
                             w * (h[0][k] * h[0][k2] + h[1][k] * h[1][k2] + h[2][k] * h[2][k2] + hk * hk2);
                     }
                 }
             }
+        }
+    double R[4][2];
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+        const double x0 = X[0][c] * (1.0 / Q), y0 = Y[0][c] * (1.0 / Q), x1 = X[1][c] * (1.0 / Q), y1 = Y[1][c] * (1.0 / Q);
+        const double a1 = 4.0 * A[1][c];
+        R[0][c] = 4.0 * A[0][c] - x0 - y0;  // hats 1 - s - t, s, t
+        R[1][c] = x0 + (a1 - y1);           // and 1 - t
+        R[2][c] = y0 + (a1 - x1);           // and 1 - s
+        R[3][c] = x1 + y1 - a1;             // s + t - 1
+    }
     if (!solve_spd(G, R, out.g)) return false;
-    // pass 2: F(c*) as a sum of non-negative terms
+    // pass 2: F(c*) as a sum of non-negative terms, from the misfit d and |d|^2
+    // of two rows of texels at a time
     double F = 0.0;
+    double d[2][Q + 1][2], e[2][Q + 1];
 #pragma unroll
-    for (int qj = 0; qj < Q; ++qj)
+    for (int y = 0; y <= Q; ++y) {
 #pragma unroll
-        for (int qi = 0; qi < Q; ++qi)
+        for (int x = 0; x <= Q; ++x) {
+            const bool low = x + y <= Q;
+            double f[2];
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                // lower plane about c00, upper about c11
+                const double o = out.g[low ? 0 : 3][c];
+                const double gx = low ? out.g[1][c] - o : o - out.g[2][c], gy = low ? out.g[2][c] - o : o - out.g[1][c];
+                const double px = low ? double(x) / Q : double(x - Q) / Q, py = low ? double(y) / Q : double(y - Q) / Q;
+                f[c] = (o + py * gy) + px * gx - double(c ? tx[y][x].y : tx[y][x].x);
+                d[y & 1][x][c] = f[c];
+            }
+            e[y & 1][x] = f[0] * f[0] + f[1] * f[1];
+        }
+        if (y == 0) continue;
+        const int r0 = (y - 1) & 1, r1 = y & 1;
+#pragma unroll
+        for (int qi = 0; qi < Q; ++qi) {
+            const double mx = d[r0][qi + 1][0] + d[r1][qi][0], my = d[r0][qi + 1][1] + d[r1][qi][1];
+            const double me = e[r0][qi + 1] + e[r1][qi];
 #pragma unroll
             for (int tri = 0; tri < 2; ++tri) {
-                const int base = qi + qj <= Q - 1 - tri ? 0 : 1;
-                double nx[3], ny[3], dx[3], dy[3];
-#pragma unroll
-                for (int v = 0; v < 3; ++v) {
-                    const int x = vx(qi, tri, v), y = vy(qj, tri, v);
-                    nx[v] = tx[y][x].x;
-                    ny[v] = tx[y][x].y;
-                    double ax = 0.0, ay = 0.0;
-#pragma unroll
-                    for (int k = 0; k < 3; ++k) {
-                        const double hv = hat(base + k, double(x) / Q, double(y) / Q);
-                        ax += hv * out.g[base + k][0];
-                        ay += hv * out.g[base + k][1];
-                    }
-                    dx[v] = ax - nx[v];
-                    dy[v] = ay - ny[v];
-                }
-                const double w = wt[((qj * Q + qi) * 2 + tri) * stride];
-                const double sx = dx[0] + dx[1] + dx[2], sy = dy[0] + dy[1] + dy[2];
-                F += w * (dx[0] * dx[0] + dx[1] * dx[1] + dx[2] * dx[2] + dy[0] * dy[0] + dy[1] * dy[1] +
-                          dy[2] * dy[2] + sx * sx + sy * sy);
+                const double sx = mx + (tri ? d[r1][qi + 1][0] : d[r0][qi][0]);
+                const double sy = my + (tri ? d[r1][qi + 1][1] : d[r0][qi][1]);
+                const double se = me + (tri ? e[r1][qi + 1] : e[r0][qi]);
+                F += wt[(((y - 1) * Q + qi) * 2 + tri) * stride] * (se + sx * sx + sy * sy);
             }
+        }
+    }
 #pragma unroll
     for (int k = 0; k < 10; ++k) out.G[k] = G[k];
     out.F = F;
@@ -398,7 +444,7 @@ __device__ void fit_store(const MapDesc &d, const ClusterDesc &cd, int l, uint32
         float d11x = float(c[3][0] - c[0][0]), d11y = float(c[3][1] - c[0][1]);
         rec[0] = make_float4(c0, c1, d10x, d10y);
         rec[1] = make_float4(d01x, d01y, d11x, d11y);
-        *ev = float(sqrt(fmax(qf.F, 0.0)));
+        *ev = float(sqrt(fmax(qf.F, 0.0) * (1.0 / 24.0)));
         widen_corner(b, c0, c1, 0.f, 0.f);
         widen_corner(b, c0, c1, d10x, d10y);
         widen_corner(b, c0, c1, d01x, d01y);
@@ -426,7 +472,7 @@ constexpr int kTileThreads = 1 << (2 * kTileLevels);  // 256 leaf blocks
 // at one (255 registers) for the 8192^2 cluster hierarchy; the FP64 pipe
 // needs the second CTA's warps to stay busy.
 template <int TFMT, int BFMT>
-__global__ void __launch_bounds__(kTileThreads, 2) cluster_tiles(MapDesc d, ClusterDesc cd, QF *__restrict__ out6)
+__global__ void __launch_bounds__(kTileThreads, PNDF_CL_CTAS) cluster_tiles(MapDesc d, ClusterDesc cd, QF *__restrict__ out6)
 {
     extern __shared__ double wt_s[];  // [32][kTileThreads]
     __shared__ QF part[16];
