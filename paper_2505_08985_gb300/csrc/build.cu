@@ -33,6 +33,9 @@ namespace {
 constexpr int kTileQuadsMax = 64;
 constexpr int kTileTexMax = kTileQuadsMax + 1;
 constexpr int kBuildThreads = 256;
+#ifndef PNDF_BUILD_CTAS
+#define PNDF_BUILD_CTAS 3  // 80 registers; at two (91) an 8192^2 build takes 0.25 ms longer
+#endif
 
 // Second moments of a set of normals about a reference point.
 struct Moments {
@@ -132,7 +135,7 @@ __device__ __forceinline__ float2 copy_texel(const void *src, void *dst, size_t 
 // VEC = texels per 16-byte load (2 for FP32, 4 for FP16), or 1 when rows are
 // not 16-byte aligned (n not a multiple of VEC).
 template <int TFMT, int BFMT, int VEC>
-__global__ void __launch_bounds__(kBuildThreads) build_tiles(const void *__restrict__ src, MapDesc d, int tileQ,
+__global__ void __launch_bounds__(kBuildThreads, PNDF_BUILD_CTAS) build_tiles(const void *__restrict__ src, MapDesc d, int tileQ,
                                                             int lq)
 {
     __shared__ float2 tex[kTileTexMax * kTileTexMax];
