@@ -1315,6 +1315,7 @@ struct SplitPlan {
     float *wt;                 // the target w_t (served steps: written by the plan for the step kernel)
     uint32_t cap;              // entries capacity
     int resident_warps;
+    bool one_cta;              // planned by split_small, which also clears the counters
 };
 
 template <class Q>
@@ -1403,6 +1404,44 @@ __global__ void split_plan(MapDesc d, const pndf_query *__restrict__ qs, int64_t
 {
     const float wt = split_target(p);
     for (int64_t k = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; k < nq; k += int64_t(gridDim.x) * blockDim.x) {
+        const auto q = make_query<KERN>(qs[k], jac_eps);
+        int level;
+        uint32_t tiles;
+        p.marker[k] = split_choice(q, d.L, wt, level, tiles) && split_reserve(p, uint32_t(k), 0, level, tiles);
+    }
+}
+
+// split_work and split_plan of a small batch in one CTA, which also sets the
+// work cursor and the counters to zero: one launch in place of a memset and two.
+constexpr int64_t kSplitSmall = 8192;
+
+template <int KERN>
+__global__ void __launch_bounds__(1024) split_small(MapDesc d, const pndf_query *__restrict__ qs, int nq, float jac_eps,
+                                                    SplitPlan p, unsigned long long *__restrict__ cursor)
+{
+    __shared__ double red[32];
+    __shared__ double total;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    double acc = 0.0;
+    for (int k = threadIdx.x; k < nq; k += 1024) acc += double(split_estimate(make_query<KERN>(qs[k], jac_eps)));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(kFull, acc, o);
+    if (lane == 0) red[warp] = acc;
+    __syncthreads();
+    if (warp == 0) {
+        acc = red[lane];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(kFull, acc, o);
+        if (lane == 0) {
+            total = acc;
+            *p.ctr = 0ull;
+            *cursor = 0ull;
+        }
+    }
+    __syncthreads();
+    p.work = &total;
+    const float wt = split_target(p);
+    for (int k = threadIdx.x; k < nq; k += 1024) {
         const auto q = make_query<KERN>(qs[k], jac_eps);
         int level;
         uint32_t tiles;
@@ -1740,9 +1779,14 @@ cudaError_t launch_traverse(const MapDesc &d, const ClusterDesc &cd, float tau, 
         sp.resident_warps = int(grid) * warps;
         int64_t blocks = (nq + 255) / 256;
         if (blocks > int64_t(sms) * 8) blocks = int64_t(sms) * 8;
-        split_work<KERN><<<unsigned(blocks), 256, 0, s>>>(q, nq, jac_eps, sp.work);
-        split_plan<KERN><<<unsigned(blocks), 256, 0, s>>>(d, q, nq, jac_eps, sp);
-        count_launches(2);
+        if (sp.one_cta) {
+            split_small<KERN><<<1, 1024, 0, s>>>(d, q, int(nq), jac_eps, sp, cursor);
+            count_launches(1);
+        } else {
+            split_work<KERN><<<unsigned(blocks), 256, 0, s>>>(q, nq, jac_eps, sp.work);
+            split_plan<KERN><<<unsigned(blocks), 256, 0, s>>>(d, q, nq, jac_eps, sp);
+            count_launches(2);
+        }
     } else if (grid > want) {
         grid = want;
     }
@@ -1804,11 +1848,17 @@ pndf_status launch_eval(const pndf_hierarchy *h, const pndf_query *q, int64_t nq
 {
     if (nq == 0) return PNDF_OK;
     const MapDesc &d = h->d;
-    const bool sort = cfg.sort != 0;
     const bool split = cfg.mode == PNDF_MODE_HIERARCHY && !(cfg.tau > 0.f) && cfg.split == 0;
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    // A batch of up to four queries per resident warp (24 per SM) gains nothing
+    // from the order when its large footprints are divided: no warp holds more
+    // than a few queries, and neighbours do not stay in flight together (4,096
+    // footprints on 16384^2 and 20,011 on 8192^2: 5.10 and 5.09 ms in arrival
+    // order, 5.12 and 5.14 ms sorted; 131,072: 24.6 and 19.8 ms).  The sort's
+    // four launches would then be most of a small call.
+    const bool sort = cfg.sort != 0 && !(split && nq <= int64_t(4) * 24 * sms);
     const uint32_t cap = uint32_t(2 * 64 * (sms > 0 ? sms : 1) + 64);  // >= 2 x resident warps
     // scratch: cursor, split counter and work sum (padded to 256), key
     // histogram, keys, order, split markers and entries
@@ -1832,9 +1882,10 @@ pndf_status launch_eval(const pndf_hierarchy *h, const pndf_query *q, int64_t nq
         sp.ctr = reinterpret_cast<unsigned long long *>(base + 8);
         sp.work = reinterpret_cast<double *>(base + 16);
         sp.cap = cap;
+        sp.one_cta = !sort && nq <= kSplitSmall;
     }
     uint32_t *order = nullptr;
-    cudaError_t e = cudaMemsetAsync(base, 0, sort ? off_keys : 256, s);
+    cudaError_t e = sp.one_cta ? cudaSuccess : cudaMemsetAsync(base, 0, sort ? off_keys : 256, s);
     if (e == cudaSuccess && sort) {
         order = reinterpret_cast<uint32_t *>(base + off_order);
         e = sort_launch(d, q, nq, cfg.sort, reinterpret_cast<uint32_t *>(base + off_hist),

@@ -224,25 +224,31 @@ __device__ __forceinline__ float deferred_value(const MapDesc &d, const Dir &w, 
     return wa.wt[r][slot] * v;
 }
 
+__device__ __forceinline__ uint32_t band_count(const pndf_query &r, int n)
+{
+    const Req q = make_req(r, n);
+    const int rows = q.j1 - q.j0 + 1;
+    return rows > 0 ? uint32_t((rows + kBand - 1) / kBand) : 0u;
+}
+
 __global__ void pa_bands(MapDesc d, const pndf_query *__restrict__ qs, int64_t k0, int cnt, uint32_t *__restrict__ nb)
 {
     int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= cnt) return;
-    Req q = make_req(qs[k0 + t], d.n);
-    int rows = q.j1 - q.j0 + 1;
-    nb[t] = rows > 0 ? uint32_t((rows + kBand - 1) / kBand) : 0u;
+    if (t < cnt) nb[t] = band_count(qs[k0 + t], d.n);
 }
 
-// exclusive scan of cnt (<= 65536) values in place, one CTA of 1024 threads;
-// total goes to nb[cnt]
-__device__ __forceinline__ void scan_bands(uint32_t *__restrict__ nb, int cnt)
+// Exclusive scan of cnt (<= 65536) values value(i) into nb, one CTA of 1024
+// threads; the total goes to nb[cnt] and the work cursor to zero.  (value may
+// read nb[i] itself.)
+template <class F>
+__device__ __forceinline__ void scan_bands(F value, uint32_t *__restrict__ nb, int cnt, unsigned int *__restrict__ cursor)
 {
     __shared__ uint32_t part[1024];
     const int per = (cnt + 1023) / 1024;
     const int b0 = threadIdx.x * per;
     uint32_t sum = 0;
     for (int i = 0; i < per; ++i)
-        if (b0 + i < cnt) sum += nb[b0 + i];
+        if (b0 + i < cnt) sum += value(b0 + i);
     part[threadIdx.x] = sum;
     __syncthreads();
     for (int off = 1; off < 1024; off <<= 1) {
@@ -254,15 +260,29 @@ __device__ __forceinline__ void scan_bands(uint32_t *__restrict__ nb, int cnt)
     uint32_t run = part[threadIdx.x] - sum;
     for (int i = 0; i < per; ++i) {
         if (b0 + i < cnt) {
-            uint32_t v = nb[b0 + i];
+            uint32_t v = value(b0 + i);
             nb[b0 + i] = run;
             run += v;
         }
     }
-    if (threadIdx.x == 1023) nb[cnt] = part[1023];
+    if (threadIdx.x == 1023) {
+        nb[cnt] = part[1023];
+        *cursor = 0u;
+    }
 }
 
-__global__ void __launch_bounds__(1024) pa_scan(uint32_t *__restrict__ nb, int cnt) { scan_bands(nb, cnt); }
+__global__ void __launch_bounds__(1024) pa_scan(uint32_t *nb, int cnt, unsigned int *cursor)
+{
+    scan_bands([&](int i) { return nb[i]; }, nb, cnt, cursor);
+}
+
+// pa_bands and pa_scan of up to kPrepSmall requests in one launch.
+constexpr int kPrepSmall = 4096;
+__global__ void __launch_bounds__(1024) pa_prep(MapDesc d, const pndf_query *__restrict__ qs, int64_t k0, int cnt,
+                                                uint32_t *nb, unsigned int *cursor)
+{
+    scan_bands([&](int i) { return band_count(qs[k0 + i], d.n); }, nb, cnt, cursor);
+}
 
 // Band `band` (kBand quad rows) of request (q, w) on map d, integrated by one
 // warp: the band's quads inside the ellipse in row order, one per lane, both
@@ -453,16 +473,18 @@ __global__ void area_step_bands(const MapDesc *__restrict__ maps, const uint32_t
                                 const AreaReq *__restrict__ areq, uint32_t *__restrict__ nb)
 {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= int(*count)) return;
-    const AreaReq a = areq[t];
-    const Req q = make_req(*a.q, maps[a.map].n);
-    const int rows = q.j1 - q.j0 + 1;
-    nb[t] = rows > 0 ? uint32_t((rows + kBand - 1) / kBand) : 0u;
+    if (t < int(*count)) nb[t] = band_count(*areq[t].q, maps[areq[t].map].n);
 }
 
-__global__ void __launch_bounds__(1024) area_step_scan(const uint32_t *__restrict__ count, uint32_t *__restrict__ nb)
+__global__ void __launch_bounds__(1024) area_step_scan(const uint32_t *__restrict__ count, uint32_t *nb, unsigned int *cursor)
 {
-    scan_bands(nb, int(*count));
+    scan_bands([&](int i) { return nb[i]; }, nb, int(*count), cursor);
+}
+
+__global__ void __launch_bounds__(1024) area_step_prep(const MapDesc *__restrict__ maps, const uint32_t *__restrict__ count,
+                                                       const AreaReq *__restrict__ areq, uint32_t *nb, unsigned int *cursor)
+{
+    scan_bands([&](int i) { return band_count(*areq[i].q, maps[areq[i].map].n); }, nb, int(*count), cursor);
 }
 
 template <int TFMT>
@@ -888,10 +910,12 @@ cudaError_t launch_area_step(int texel_fmt, const MapDesc *maps, int nmaps, cons
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaError_t e = cudaMemsetAsync(cursor, 0, sizeof(unsigned int), s);
-    if (e != cudaSuccess) return e;
-    area_step_bands<<<(cap + 255) / 256, 256, 0, s>>>(maps, count, areq, off);
-    area_step_scan<<<1, 1024, 0, s>>>(count, off);
+    if (cap <= kPrepSmall) {
+        area_step_prep<<<1, 1024, 0, s>>>(maps, count, areq, off, cursor);
+    } else {
+        area_step_bands<<<(cap + 255) / 256, 256, 0, s>>>(maps, count, areq, off);
+        area_step_scan<<<1, 1024, 0, s>>>(count, off, cursor);
+    }
     int occ = 0;
     if (texel_fmt == PNDF_TEXEL_F32X2) {
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, area_step_items<PNDF_TEXEL_F32X2>, 256, 0);
@@ -934,10 +958,13 @@ pndf_status launch_projarea(const pndf_hierarchy *h, const pndf_query *q, const 
     cudaError_t e = cudaSuccess;
     for (int64_t k0 = 0; k0 < nq && e == cudaSuccess; k0 += chunk) {
         int cnt = int(nq - k0 < chunk ? nq - k0 : chunk);
-        e = cudaMemsetAsync(cursor, 0, sizeof(unsigned int), s);
-        if (e != cudaSuccess) break;
-        pa_bands<<<(cnt + 255) / 256, 256, 0, s>>>(d, q, k0, cnt, off);
-        pa_scan<<<1, 1024, 0, s>>>(off, cnt);
+        if (cnt <= kPrepSmall) {
+            pa_prep<<<1, 1024, 0, s>>>(d, q, k0, cnt, off, cursor);
+        } else {
+            pa_bands<<<(cnt + 255) / 256, 256, 0, s>>>(d, q, k0, cnt, off);
+            pa_scan<<<1, 1024, 0, s>>>(off, cnt, cursor);
+            count_launches(1);
+        }
         int occ = 0;
         if (d.texel_fmt == PNDF_TEXEL_F32X2) {
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, pa_items<PNDF_TEXEL_F32X2>, 256, 0);
@@ -947,7 +974,7 @@ pndf_status launch_projarea(const pndf_hierarchy *h, const pndf_query *q, const 
             pa_items<PNDF_TEXEL_F16X2><<<sms * (occ > 0 ? occ : 1), 256, 0, s>>>(d, q, omega, k0, cnt, off, part, cursor);
         }
         pa_reduce<<<(cnt * 32 + 255) / 256, 256, 0, s>>>(q, k0, cnt, off, part, P, d.status);
-        count_launches(4);
+        count_launches(3);
         e = cudaGetLastError();
     }
     cudaError_t ef = cudaFreeAsync(scratch, s);
