@@ -192,11 +192,12 @@ def hbm_peak():
 
 
 def kernel_source_hash() -> str:
-    return sources_hash(("eval.cu", "common.cuh"))
+    return sources_hash(("eval.cu", "common.cuh", "tri.cuh"))
 
 
 CENSUS_FILE = os.path.join(ROOT, "profiles", "kernels_census_flake4096_mixed4096.txt")
-CENSUS_SOURCES = ("build.cu", "cluster.cu", "eval.cu", "projarea.cu", "sample.cu", "common.cuh", "ggx.cuh")
+CENSUS_SOURCES = ("build.cu", "cluster.cu", "eval.cu", "projarea.cu", "sample.cu", "common.cuh", "ggx.cuh",
+                  "tri.cuh", "meang.cuh", "pair.cuh", "visible.cuh")
 
 
 def code_text(src: str) -> str:
@@ -336,9 +337,9 @@ def traversal_roofline(dev, work_f16: dict, nq: int, kernel_ms: float, world: in
     warp instructions per query of the committed ncu capture of the same
     kernel source (152 SMs x 4 schedulers x the maximum SM clock).  `bound` is
     the ceiling with the larger fraction; the other is kept beside it, and so
-    is the builder's own byte model (every level-0 box tested, each tested
-    triangle's three texels, 40 B per query), which counts texels of a leaf
-    block once per triangle that reads them."""
+    is the builder's own byte model (every node, group record and texel that a
+    test reads, 40 B per query), which counts a texel once per test that reads
+    it."""
     pk, pk_kind = hbm_peak()
     sec = kernel_ms / 1e3
     s8d = work_f16["nodes"] * 8 + work_f16["leaf_blocks"] * 25 * 8 + 36 * nq
@@ -516,6 +517,15 @@ def pyramid_bytes(n: int, texel_bytes: int, box_bytes: int) -> int:
     from paper_2505_08985_gb300 import pndf
     quads = 4 ** pndf.top_level(n)
     return 2 * n * n * texel_bytes + (quads + tree_nodes(n)) * box_bytes + 8 * quads
+
+
+def build_bytes(n: int, texel_bytes: int, node_bytes: int) -> int:
+    """Algorithmic bytes of one pyramid build as it is laid out now: the map
+    read once, the hierarchy's copy written once, every node of levels 2..L
+    (box and slab) and one 16-byte record per 2 x 2 quads.  (pyramid_bytes is
+    the same count for a layout with a box and a capsule per quad.)"""
+    from paper_2505_08985_gb300 import pndf
+    return 2 * n * n * texel_bytes + tree_nodes(n) * node_bytes + 16 * 4 ** (pndf.top_level(n) - 1)
 
 
 def run_census(dev):
@@ -1068,12 +1078,14 @@ def run_gpu(args, world, rank, local):
         pndf.pndf_eval_batch(h, q, out=D, stats=stt)
         s = stt.to(torch.int64).sum(0).cpu().tolist()
         h.free()
-        node_b = 8 if tag == "f16" else 16
+        node_b = 16 if tag == "f16" else 24
         texel_b = 8
-        # per unit: a node or quad box (node_b), a tested triangle's three
-        # vertices (3 texels), and per query its record, order slot and result
+        # per unit: a node's box and slab (node_b), a leaf block's four group
+        # records (64 B), a tested group's nine texels, a decided triangle's
+        # three, and per query its record, order slot and result
         work[tag] = {"nodes": s[0], "quads": s[7], "leaf_blocks": s[1], "tri_tests": s[2], "hits": s[3],
-                     "bytes": (s[0] + s[7]) * node_b + s[2] * 3 * texel_b + nq * (32 + 4 + 4)}
+                     "bytes": s[0] * node_b + s[1] * 64 + (s[7] // 4) * 9 * texel_b + s[2] * 3 * texel_b +
+                     nq * (32 + 4 + 4)}
         del stt
     torch.cuda.synchronize()
 
@@ -1372,7 +1384,7 @@ def kernel_rooflines(dev, n, nq, stage_ms, traverse_ms, traverse_roof, cluster, 
            "census": "profiles/" + os.path.basename(CENSUS_FILE) if census else None}
     fams = {}
     fams["pyramid_build"] = family_roofline("pyramid_build", ["build_tiles", "build_up"], stage_ms["pyramid_build"],
-                                            n * n, "texel", pyramid_bytes(n, 8, 8) / (n * n), census, peaks, pk)
+                                            n * n, "texel", build_bytes(n, 8, 16) / (n * n), census, peaks, pk)
     fams["query_sort"] = family_roofline("query_sort", ["key_hist", "key_scan", "key_place"], stage_ms["query_sort"],
                                          nq, "query", 44, census, peaks, pk)
     tr = family_roofline("traverse", ["traverse_kernel"], traverse_ms, nq, "query",
@@ -1397,7 +1409,7 @@ def kernel_rooflines(dev, n, nq, stage_ms, traverse_ms, traverse_roof, cluster, 
     if mixed:
         m = mixed["map_n"]
         pa = mixed["projected_area"]
-        fams["projected_area"] = family_roofline("projected_area", ["pa_bands", "pa_scan", "pa_items", "pa_reduce"], pa["ms"],
+        fams["projected_area"] = family_roofline("projected_area", ["pa_prep", "pa_bands", "pa_scan", "pa_items", "pa_reduce"], pa["ms"],
                                                  pa["triangles"], "triangle", 8, census, peaks, pk)
         gf = mixed["ggx_fit"]
         fams["ggx_fit"] = family_roofline("ggx_fit", ["ggx_leaf", "ggx_up"], gf["build_ms"], leaf_blocks(m),

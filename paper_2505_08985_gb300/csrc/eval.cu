@@ -655,10 +655,11 @@ __device__ __forceinline__ void test_leaf(const MapDesc &d, const Q &q, uint32_t
 }
 
 // Leaf queue: up to 15 leaf blocks held over from the last step plus one
-// step's children; cut cluster nodes fill it from the back (entry k at
-// kLeafQ - 1 - k), and a step's new leaf blocks and cut nodes number at most
-// 4 kPop together, so the two ends never meet.
+// step's children.
 constexpr int kLeafQ = 16 + 4 * kPop;
+// Cut ring, with the cluster cut only: cut nodes (at most 31 held over plus one
+// step's children), tested 32 at a time.
+constexpr int kCutRing = 128;
 // Group ring: 2 x 2-quad groups whose box and slab hold m (at most 31 held over
 // plus one pass's 64): Morton index at level 1 (at most 26 bits), kMarked where
 // the group holds a near-singular triangle.
@@ -673,15 +674,16 @@ constexpr int kTriRing = 64;
 constexpr int kHitRing = 64;
 // Shared memory per warp: DFS stack, leaf queue, the rings.
 template <bool CLUSTER>
-constexpr int kWarpSmemWords = kStackCap + kLeafQ + kGroupRing + kTriRing + (CLUSTER ? 4 * kHitRing : 0);
+constexpr int kWarpSmemWords = kStackCap + kLeafQ + kGroupRing + kTriRing + (CLUSTER ? 4 * kHitRing + kCutRing : 0);
 static_assert((kStackCap + kLeafQ + kGroupRing + kTriRing) % 4 == 0, "hit ring alignment");
 
 // A warp's shared memory and the rings' heads and counts.
 struct LeafState {
     uint32_t *groups, *tris;
     float4 *hits;
-    uint32_t ghead, thead, hhead;
-    int ng, nt, nh;
+    uint32_t *cuts;
+    uint32_t ghead, thead, hhead, chead;
+    int ng, nt, nh, nc;
 };
 
 // tiny_triangle of triangle `tri` of quad (gi, gj) when its leaf block meets the
@@ -913,19 +915,19 @@ __device__ __forceinline__ void weigh_clusters(const MapDesc &d, const Q &q, con
     weigh<STATS>(q, int(I << l), int(J << l), l, tri, h.x, h.y, h.z, id, acc);
 }
 
-// All 32 lanes: lane k < cnt tests the two cluster triangles of the cut node
-// in last[-k] (index in the box array): lower (c00, c10, c01) at uv (O, O + (a,
+// All 32 lanes: lane k < cnt tests the two cluster triangles of cut node k of
+// the cut ring: lower (c00, c10, c01) at uv (O, O + (a,
 // 0), O + (0, a)), upper (c11, c01, c10) at (O + (a, a), O + (0, a), O + (a,
 // 0)), a = 2^l; hits join the hit ring.
 template <bool STATS, class Q>
 __device__ __forceinline__ void test_clusters(const MapDesc &d, const ClusterDesc &cd, const Q &q,
-                                              const uint32_t *last, int cnt, LeafState &ls, int lane, Acc &acc)
+                                              LeafState &ls, int cnt, int lane, Acc &acc)
 {
     const unsigned lt = (1u << lane) - 1u;
     bool h0 = false, h1 = false;
     float4 v0 = make_float4(0.f, 0.f, 0.f, 0.f), v1 = v0;
     if (lane < cnt) {
-        const uint32_t k = last[-lane];
+        const uint32_t k = ls.cuts[(ls.chead + uint32_t(lane)) & (kCutRing - 1)];
         const int l = node_level(k, d.L);
         const uint32_t m = k - node_index(d.L, l, 0);
         const float4 *rec = cd.cl + 2 * size_t(k);
@@ -1044,7 +1046,7 @@ __device__ __forceinline__ void eval_range(const MapDesc &d, const ClusterDesc &
                                            int a1, int c0, int c1, int lane, uint32_t *smem, Acc &acc)
 {
     uint32_t *stk = smem, *lq = smem + kStackCap;
-    int top = 0, nleaf = 0, ncl = 0;
+    int top = 0, nleaf = 0;
     const unsigned lt = (1u << lane) - 1u;
     const uint32_t leaf0 = node_index(d.L, kLeafLevel, 0);  // from here on a node is a leaf block
     // With the cut, a slab above the leaf level says nothing: it holds the
@@ -1060,6 +1062,9 @@ __device__ __forceinline__ void eval_range(const MapDesc &d, const ClusterDesc &
         const uint32_t m = k - node_index(d.L, l, 0);
         return node_meets(q, l, compact1by1(m), compact1by1(m >> 1), ins);
     };
+    uint32_t *rings = lq + kLeafQ;
+    float4 *hits = reinterpret_cast<float4 *>(rings + kGroupRing + kTriRing);
+    LeafState ls{rings, rings + kGroupRing, hits, reinterpret_cast<uint32_t *>(hits + kHitRing), 0u, 0u, 0u, 0u, 0, 0, 0, 0};
     // entry nodes: at most 4 x 4
     {
         int a = a0 + (lane & 3), c = c0 + (lane >> 2);
@@ -1078,17 +1083,15 @@ __device__ __forceinline__ void eval_range(const MapDesc &d, const ClusterDesc &
         unsigned mp = __ballot_sync(kFull, pass && !cut);
         unsigned mc = __ballot_sync(kFull, cut);
         if (pass && !cut) (e == kLeafLevel ? lq : stk)[__popc(mp & lt)] = k | (inside ? kInside : 0u);
-        if (CLUSTER && cut) lq[kLeafQ - 1 - __popc(mc & lt)] = k;
+        if (CLUSTER && cut) ls.cuts[__popc(mc & lt)] = k;
         if (e == kLeafLevel)
             nleaf = __popc(mp);
         else
             top = __popc(mp);
-        ncl = __popc(mc);
+        ls.nc = __popc(mc);
         __syncwarp();
     }
     bool overflow = false;
-    uint32_t *rings = lq + kLeafQ;
-    LeafState ls{rings, rings + kGroupRing, reinterpret_cast<float4 *>(rings + kGroupRing + kTriRing), 0u, 0u, 0u, 0, 0, 0};
     while (true) {
         // leaf blocks are filtered sixteen to a pass (four lanes each, twice):
         // while the stack still holds nodes only whole passes run, and the rest
@@ -1102,14 +1105,14 @@ __device__ __forceinline__ void eval_range(const MapDesc &d, const ClusterDesc &
             __syncwarp();
         }
         nleaf -= nrun;
-        if (CLUSTER) {
-            // cut nodes sit at the back of the leaf queue
-            for (int k0 = 0; k0 < ncl; k0 += 32) {
-                test_clusters<STATS>(d, cd, q, lq + kLeafQ - 1 - k0, min(32, ncl - k0), ls, lane, acc);
+        if (CLUSTER)
+            while (ls.nc >= (top == 0 ? 1 : 32)) {  // full warps of cut nodes, the rest at the end
+                const int cnt = min(ls.nc, 32);
+                test_clusters<STATS>(d, cd, q, ls, cnt, lane, acc);
+                ls.chead += uint32_t(cnt);
+                ls.nc -= cnt;
                 __syncwarp();
             }
-            ncl = 0;
-        }
         if (top == 0) break;
         // pop up to kPop nodes; lane k tests child (k & 3) of popped nodes
         // (k >> 2) + 8 r, so kPer loads per lane are in flight
@@ -1162,8 +1165,8 @@ __device__ __forceinline__ void eval_range(const MapDesc &d, const ClusterDesc &
             unsigned ms = __ballot_sync(kFull, to_stack);
             if (CLUSTER) {
                 unsigned mc = __ballot_sync(kFull, cut[r]);
-                if (cut[r]) lq[kLeafQ - 1 - ncl - __popc(mc & lt)] = ck[r];
-                ncl += __popc(mc);
+                if (cut[r]) ls.cuts[(ls.chead + uint32_t(ls.nc) + __popc(mc & lt)) & (kCutRing - 1)] = ck[r];
+                ls.nc += __popc(mc);
             }
             if (to_leaf) lq[nleaf + __popc(ml & lt)] = ck[r];
             if (to_stack) {

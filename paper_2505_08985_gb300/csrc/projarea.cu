@@ -46,7 +46,12 @@ constexpr unsigned kFull = 0xffffffffu;
 #ifndef PNDF_PA_CTAS
 #define PNDF_PA_CTAS 4
 #endif
-constexpr int kBand = 8;                 // quad rows per work item
+// A band is long enough to pay for its row setup and its rings' last, partly
+// filled evaluations, and short enough to spread a few footprints over the SMs:
+// 8 / 4 / 2 rows, 192 requests on 16384^2 14.6 / 13.0 / 12.4 ms, 64 on 4096^2 1.06 /
+// 0.63 / 0.47 ms, 1000 small ones 0.33 / 0.32 / 0.32 ms; the partial sums (and a
+// server's scratch) double with each halving.
+constexpr int kBand = 4;                 // quad rows per work item
 
 // V_T / |cross| in closed form (visible.cuh, FP64), for the largest triangles;
 // the segment form of Eq. 13 where the normals collapsed (|cross| < 1e-12).

@@ -52,6 +52,8 @@ struct pndf_server {
     MapDesc *maps_dev = nullptr;
     ClusterDesc *clusters_dev = nullptr;  // per map, read only with tau > 0
     cudaStream_t cap = nullptr;
+    cudaStream_t cap_area = nullptr;  // the captured step's second branch
+    cudaEvent_t fork = nullptr, join = nullptr;
     int area_cap = 0;     // projected-area requests per step
     int area_bands = 0;   // bands per request at most (largest map)
     static constexpr int kMaxSlots = 8;
@@ -76,6 +78,9 @@ void release(pndf_server *s)
     if (s->maps_dev) cudaFree(s->maps_dev);
     if (s->clusters_dev) cudaFree(s->clusters_dev);
     if (s->cap) cudaStreamDestroy(s->cap);
+    if (s->cap_area) cudaStreamDestroy(s->cap_area);
+    if (s->fork) cudaEventDestroy(s->fork);
+    if (s->join) cudaEventDestroy(s->join);
     delete s;
 }
 
@@ -104,9 +109,13 @@ cudaError_t capture_slot(pndf_server *s, Slot &sl)
     cudaMemsetAsync(cursor, 0, sizeof(unsigned long long), s->cap);
     const ServeVariant v{s->kernel, s->tau, s->jac_eps};
     char *split = dev + up256(tb) + 256;
-    launch_serve(s->texel_fmt, s->bounds_fmt, v, s->maps_dev, s->clusters_dev, s->nmaps, table, segs, cursor,
-                 s->warps, s->ctas, s->split_cap > 0 ? split : nullptr, s->split_cap, s->cap);
+    // The projected-area part is a branch of its own beside the P-NDF part: a
+    // step's few area requests are long chains on few warps, and one after the
+    // other the two took the sum of their times.  It is launched first, so that
+    // its blocks are placed before the P-NDF kernel fills the SMs.
     if (s->area_cap > 0) {
+        e = cudaEventRecord(s->fork, s->cap);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(s->cap_area, s->fork, 0);
         char *at = dev + pndf_table_bytes(s->max_segs);
         char *scratch = split + up256(serve_split_bytes(s->split_cap));
         auto *off = reinterpret_cast<uint32_t *>(scratch);
@@ -115,11 +124,19 @@ cudaError_t capture_slot(pndf_server *s, Slot &sl)
         scratch += up256(size_t(s->area_cap) * s->area_bands * sizeof(float2));
         launch_area_step(s->texel_fmt, s->maps_dev, s->nmaps, reinterpret_cast<const uint32_t *>(at),
                          reinterpret_cast<const AreaReq *>(at + 16), s->area_cap, off, part,
-                         reinterpret_cast<unsigned int *>(scratch), s->cap);
+                         reinterpret_cast<unsigned int *>(scratch), s->cap_area);
+        if (e == cudaSuccess) e = cudaEventRecord(s->join, s->cap_area);
     }
+    launch_serve(s->texel_fmt, s->bounds_fmt, v, s->maps_dev, s->clusters_dev, s->nmaps, table, segs, cursor,
+                 s->warps, s->ctas, s->split_cap > 0 ? split : nullptr, s->split_cap, s->cap);
+    if (s->area_cap > 0 && e == cudaSuccess) e = cudaStreamWaitEvent(s->cap, s->join, 0);
     cudaGraph_t g = nullptr;
     cudaError_t ec = cudaStreamEndCapture(s->cap, &g);
     if (ec != cudaSuccess) return ec;
+    if (e != cudaSuccess) {
+        cudaGraphDestroy(g);
+        return e;
+    }
     e = cudaGraphInstantiate(&sl.exec, g, 0);
     cudaGraphDestroy(g);
     return e;
@@ -197,6 +214,9 @@ pndf_status pndf_server_create(const pndf_hierarchy *const *maps, int32_t nmaps,
               cudaMemcpy(s->clusters_dev, host_clusters, sizeof(ClusterDesc) * nmaps, cudaMemcpyHostToDevice) ==
                   cudaSuccess &&
               cudaStreamCreateWithFlags(&s->cap, cudaStreamNonBlocking) == cudaSuccess &&
+              cudaStreamCreateWithFlags(&s->cap_area, cudaStreamNonBlocking) == cudaSuccess &&
+              cudaEventCreateWithFlags(&s->fork, cudaEventDisableTiming) == cudaSuccess &&
+              cudaEventCreateWithFlags(&s->join, cudaEventDisableTiming) == cudaSuccess &&
               prepare_serve(s->texel_fmt, s->bounds_fmt, ServeVariant{s->kernel, s->tau, s->jac_eps}, s->warps) ==
                   cudaSuccess;
     for (int k = 0; ok && k < s->nslots; ++k) {
