@@ -355,9 +355,10 @@ pndf_status pndf_eval_batch_host(const pndf_hierarchy *h, const pndf_query *q_ho
  * term).  w is used as the unit vector w / |w|.  k_r(T) is the kernel at T's
  * uv centroid (cut at q > 16).  A triangle whose normals collapsed onto a
  * segment (|cross| < 1e-12) contributes the segment form of Eq. 13: k_r(T)
- * times the uv-triangle integral of max(n~(u).w, 0) / n~_z(u).  Fully
- * visible triangles are integrated in FP32; partly visible ones, long
- * slivers and collapsed ones in FP64.  The aggregated diffuse BRDF is
+ * times the uv-triangle integral of max(n~(u).w, 0) / n~_z(u).  Triangles
+ * are integrated by quadrature of that integrand in FP32 (cut along the
+ * visibility boundary where it crosses them), very large ones in closed form
+ * in FP64.  The aggregated diffuse BRDF is
  * f_d = P / (pi w_z) (Eq. 13) and the shadow-masking Lambda = P / w_z - 1
  * (Sec. 4.3).
  *   q_dev:     device, nq pndf_query (x, y, sxx, sxy, syy used; ms, mt ignored).

@@ -41,7 +41,7 @@
 // 23 ms, so DRAM is not the limit).  Per query of the 8192^2 flake workload it
 // tests 10.5k nodes, 1.2k leaf blocks, 1.4k groups and 972 triangles for 964
 // hits, in 62k warp instructions; with a box and a capsule per quad in place of
-// the slabs and groups it took 187k, and 896 ms per 4M queries against 345 ms.
+// the slabs and groups it took 187k, and 897 ms per 4M queries against 329 ms.
 //
 // Hit test (tie rule): m inside the closed normal bounding box and all three
 // edge functions sign-consistent with the triangle orientation (>= 0 after
@@ -60,11 +60,13 @@ __device__ unsigned int g_status_eval;
 
 namespace {
 
-// Children a lane tests per step, all their loads in flight.  Per 1M queries of
-// the flake map 2: 94.8 ms, 3: 86.5 ms, 4: 93.0 ms; of the scratch map 13.7,
-// 14.3 and 14.9 ms.
-constexpr int kPer = 3;
-constexpr int kPop = 8 * kPer;     // nodes popped per step (four children each)
+// Children a lane tests per step, all their loads in flight: three with FP16
+// bounds, two with FP32 bounds, whose nodes take half as many registers again.
+// 512k flake queries on 8192^2 at 2 / 3: FP16 50.1 / 44.9 ms, FP32 50.5 / 52.6 ms;
+// 512k scratch queries, FP32, 6.9 / 7.2 ms (4 with FP16 was no better than 3).
+template <int BFMT>
+constexpr int kPer = BFMT == PNDF_BOUNDS_F32 ? 2 : 3;
+constexpr int kPop = 24;           // nodes popped per step at most (four children each)
 // DFS stack entries per warp.  A step leaves at most 3 kPop more than it found
 // on the way down a level: 3 kPop per level below the entry (at most 12), the
 // last step's 4 kPop and the 16 entry nodes.
@@ -1114,16 +1116,18 @@ __device__ __forceinline__ void eval_range(const MapDesc &d, const ClusterDesc &
                 __syncwarp();
             }
         if (top == 0) break;
-        // pop up to kPop nodes; lane k tests child (k & 3) of popped nodes
+        // pop up to 8 kPer nodes; lane k tests child (k & 3) of popped nodes
         // (k >> 2) + 8 r, so kPer loads per lane are in flight
-        int npop = min(top, kPop);
+        constexpr int per = kPer<BFMT>;
+        static_assert(8 * per <= kPop, "stack and queue capacities");
+        int npop = min(top, 8 * per);
         top -= npop;
-        bool pass[kPer], ins[kPer], cut[kPer];
-        uint32_t ck[kPer];
-        Node<BFMT> nd[kPer];
-        float ev[kPer];
+        bool pass[per], ins[per], cut[per];
+        uint32_t ck[per];
+        Node<BFMT> nd[per];
+        float ev[per];
 #pragma unroll
-        for (int r = 0; r < kPer; ++r) {
+        for (int r = 0; r < per; ++r) {
             int slot = (lane >> 2) + 8 * r;
             uint32_t ent = slot < npop ? stk[top + slot] : 0u;
             ck[r] = (ent << 2) | uint32_t(lane & 3);  // shifts "inside" out
@@ -1136,13 +1140,13 @@ __device__ __forceinline__ void eval_range(const MapDesc &d, const ClusterDesc &
         // the costly test, only for the few children that hold m (98 ms against
         // 105 ms with the uv box first, 1M flake queries).
 #pragma unroll
-        for (int r = 0; r < kPer; ++r)
+        for (int r = 0; r < per; ++r)
             if (pass[r]) {
                 nd[r] = load_node<BFMT>(d, ck[r]);
                 if (CLUSTER) ev[r] = __ldg(cd.ce + ck[r]);
             }
 #pragma unroll
-        for (int r = 0; r < kPer; ++r) {
+        for (int r = 0; r < per; ++r) {
             pass[r] = pass[r] && node_box_holds<BFMT, CLAMP>(nd[r], q);
             if (CLUSTER) {
                 pass[r] = pass[r] && in_footprint(ck[r], ins[r]);
@@ -1157,7 +1161,7 @@ __device__ __forceinline__ void eval_range(const MapDesc &d, const ClusterDesc &
         }
         __syncwarp();
 #pragma unroll
-        for (int r = 0; r < kPer; ++r) {
+        for (int r = 0; r < per; ++r) {
             const bool keep = pass[r] && !cut[r];
             bool to_leaf = keep && ck[r] >= leaf0;
             bool to_stack = keep && ck[r] < leaf0;

@@ -1,6 +1,7 @@
 // Visible part of one normal triangle for the projected area (Eq. 10-11,
-// Alg. 1, App. B), the general path: triangles that are only partly visible,
-// thin slivers and triangles whose normals collapsed onto a segment.
+// Alg. 1, App. B) in closed form: the triangles too large for the quadrature of
+// meang.cuh.  It holds for any triangle, partly visible, thin or collapsed onto a
+// segment.
 //
 // Notation.  m = (m_x, m_y) is a projected normal, z(m) = sqrt(1 - |m|^2) the
 // height of m~ on the hemisphere, w = (w_x, w_y, w_z) the unit direction
@@ -33,8 +34,7 @@
 // scaled frame (foot of the perpendicular and half chord), and the circle
 // angles from atan2 of the corner pair.  All of it runs in FP64: the visible
 // part of a clipped triangle can be many orders of magnitude smaller than
-// the triangle, and an FP32 evaluation of the same sums (tried, with a
-// rounding estimate) could not be trusted to 1e-5 there.
+// the triangle, and these sums of excesses partly cancel.
 //
 // Triangles whose normal-space area is (numerically) zero are the segment
 // form of Eq. 13, integrated in closed form (collapsed_visible).
