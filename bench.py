@@ -1051,7 +1051,7 @@ def run_clamp_sampling(args, world, st, q, gauss_kernel_ms, D_exact):
     U = torch.rand(nq, 2, device=dev, generator=g)
     ms = timed(lambda: pndf.pndf_sample_normals(h, q, U, jac_eps=eps))
     out["sampling"] = {"value": sum_over_ranks(world, float(nq)) / (ms / 1e3), "unit": "samples/s", "ms_per_step": ms,
-                       "note": "Gaussian footprints of the workload (sigma 1..512), FP64 position arithmetic"}
+                       "note": "Gaussian footprints of the workload (sigma 1..512), position in pairs of FP32 numbers"}
     h.free()
     return out
 
