@@ -144,54 +144,73 @@ __device__ __forceinline__ float ray_enter(const Dir &w, const Ray &r, float2 d)
     return __fdividef(qc, root - qb);
 }
 
-// Gauss-Legendre on [0, 1]: six points across, five along (times the abscissa).
-__constant__ float kGx6[6] = {0.033765242898424f, 0.169395306766868f, 0.380690406958402f,
-                              0.619309593041599f, 0.830604693233132f, 0.966234757101576f};
-__constant__ float kGw6[6] = {0.085662246189585f, 0.180380786524069f, 0.233956967286346f,
-                              0.233956967286346f, 0.180380786524069f, 0.085662246189585f};
+// Gauss-Legendre on [0, 1]: four points across the visible polygon and five along
+// it, five across a cap and two along its rays (weights 1/2).
+__constant__ float kGx4[4] = {0.069431844202974f, 0.330009478207572f, 0.669990521792428f, 0.930568155797026f};
+__constant__ float kGw4[4] = {0.173927422568727f, 0.326072577431273f, 0.326072577431273f, 0.173927422568727f};
 __constant__ float kGx5[5] = {0.046910077030668f, 0.230765344947158f, 0.5f, 0.769234655052842f, 0.953089922969332f};
 __constant__ float kGw5[5] = {0.118463442528095f, 0.239314335249683f, 0.284444444444444f, 0.239314335249683f,
                               0.118463442528095f};
+__constant__ float kGx2[2] = {0.211324865405187f, 0.788675134594813f};
 
 // Half the mean of g over a triangle of class kPartial; negative if it needs the
-// closed form after all (two edges that both dip into view between vertices
-// that do not).  Let A be the vertex whose visibility differs from the other
-// two, p and q the points where edges AB and AC meet the boundary.
-//   One vertex visible: the triangle (A, p, q) with the side pq bowed out to the
-//     boundary (but not past BC).
-//   Two: the straight triangle (p, B, C) and (C, p, q), pq again bowed out (C
-//     the one that sees more).
-//   None: the cap between an edge's visible part and the boundary.
-// Bowed triangles are integrated along rays from their apex, caps along rays
-// across the edge, each ray cut at the boundary, 6 x 5 points.  Root mean square
-// error against 64 bits, FP32 rounding included, 2e-9 (h up to 0.4) to 2e-8
-// (0.8).  Clipped in FP64, the same 2% of all triangles kept the kernel's FP64
-// pipe 53% busy and took most of its time.
+// closed form after all.  Let A be the vertex whose visibility differs from the
+// other two and p, q the points where edges AB and AC meet the boundary.  The
+// visible part is a polygon, on which g is smooth, and the cap between its chord
+// pq and the boundary, which bows out of it (the visible region is convex):
+//   one vertex visible: the triangle (A, p, q);
+//   two: the quadrilateral (B, C, q, p);
+//   none: no polygon, p and q both on the one edge that dips into view.
+// The polygon is integrated along the lines from its base (A, or BC) to the chord,
+// 4 x 5 points, the triangle as a quadrilateral whose base has no length; the cap
+// along rays across the chord, 5 x 2 points, each ray cut at the boundary.  The
+// boundary is a conic that meets the chord at its ends, so the cut follows without
+// cancellation, however close p and q are to A or to each other.  E, the rays'
+// direction, lies across the chord in the uv triangle; where it runs along it in
+// normal space (slivers), the boundary's slopes along E at the chord's two ends
+// differ, and the closed form takes the triangle once they differ by more than
+// twice (up to there the cap is good to 1e-6 of itself).  So it does where an edge
+// between vertices that are not visible cuts the cap off, or where two of them dip
+// into view: 1 to 4 in 10,000 partly visible triangles of flake, scratch, bump and
+// noise maps.
+//   Error against the closed form, FP32 rounding included: at most 1.2e-7, root
+// mean square 1e-9 to 6e-9, over 2.6 million such triangles of those maps, two
+// thirds of them with the direction turned until a vertex or an edge came within
+// 1e-8 .. 0.03 of the boundary.
+//   All lanes run the same 30 points, so that a mixed warp pays for one kind of
+// triangle: against a fan of rays from A alone, which missed what lies beside AC
+// where q is near A, 192 requests on the 16384^2 mixed map 15.75 -> 15.52 ms, 1000
+// small footprints on a scratch map 283 -> 270 us; with a fan for one vertex and two
+// triangles for two (66 points for a mixed warp) 14.13 -> 14.96 ms and 341 -> 374 us
+// in another run.
 __device__ __noinline__ float partial_mean(float2 a, float2 b, float2 c, const Dir &w)
 {
     float fa = phi_of(w, a, zof(a)), fb = phi_of(w, b, zof(b)), fc = phi_of(w, c, zof(c));
     const bool va = fa >= 0.f, vb = fb >= 0.f, vc = fc >= 0.f;
     const int seen = int(va) + int(vb) + int(vc);
     auto g = [&](float x, float y) { return fmaxf(w.wz + slope_at(w, x, y), 0.f); };
-    auto ray = [&](float2 m, float f, float z) { return Ray{fmaf(w.wx, m.x, w.wy * m.y), f, z, m}; };
-    // rays O + x dO, directions E + x dE, x in [0, 1], t up to 1 / (l + x dl)
-    float2 O, dO = make_float2(0.f, 0.f), E, dE = make_float2(0.f, 0.f);
-    float l, dl = 0.f, coef, rest = 0.f;
+    auto ray = [&](float2 m, float f) { return Ray{fmaf(w.wx, m.x, w.wy * m.y), f, zof(m), m}; };
+    // visible part [t0, t1] of the edge m -> m + e between vertices that are not visible
+    auto dips = [&](float2 m, float f, float2 e, float &t0, float &t1) {
+        float qa, qb, qc, root;
+        ray_terms(w, ray(m, f), e, qa, qb, qc, root);
+        t0 = fmaxf(__fdividef(-qb - root, qa), 0.f);
+        t1 = fminf(__fdividef(root - qb, qa), 1.f);
+        return root > 0.f && t0 < t1;
+    };
+    // the cap: chord O + x dO, rays along E; coef: |dO x E| in barycentric coordinates
+    float2 O = make_float2(0.f, 0.f), dO = O, E = O;
+    float coef = 0.f, poly = 0.f;
     if (seen == 0) {
         int edges = 0;
-        O = E = dO;
-        l = 1.f;
-        coef = 0.f;
 #pragma unroll 1
         for (int k = 0; k < 3; ++k) {
             const float2 e = sub(b, a);
-            float qa, qb, qc, root;
-            ray_terms(w, ray(a, fa, zof(a)), e, qa, qb, qc, root);
-            const float tn = __fdividef(-qb - root, qa), tf = __fdividef(root - qb, qa);
-            if (root > 0.f && tn > 0.f && tf < 1.f) {
+            float t0, t1;
+            if (dips(a, fa, e, t0, t1)) {
                 ++edges;
-                O = make_float2(fmaf(tn, e.x, a.x), fmaf(tn, e.y, a.y));
-                coef = tf - tn;
+                coef = t1 - t0;
+                O = make_float2(fmaf(t0, e.x, a.x), fmaf(t0, e.y, a.y));
                 dO = make_float2(coef * e.x, coef * e.y);
                 E = make_float2(c.x - 0.5f * (a.x + b.x), c.y - 0.5f * (a.y + b.y));
             }
@@ -202,50 +221,65 @@ __device__ __noinline__ float partial_mean(float2 a, float2 b, float2 c, const D
         if (edges > 1) return -1.f;
     } else {
         const bool one = seen == 1;
-        // the odd vertex to the front, and of the other two the higher last
-        if (vb != va && vb != vc) {
+        if (vb != va && vb != vc) {  // the odd vertex to the front
             const float2 t = a; a = b; b = t;
             const float f = fa; fa = fb; fb = f;
         } else if (vc != va && vc != vb) {
             const float2 t = a; a = c; c = t;
             const float f = fa; fa = fc; fc = f;
         }
-        if (fb > fc) {
-            const float2 t = b; b = c; c = t;
-            const float f = fb; fb = fc; fc = f;
-        }
+        float t0, t1;
+        if (one && dips(b, fb, sub(c, b), t0, t1)) return -1.f;
         const float2 ab = sub(b, a), ac = sub(c, a);
-        const Ray ra = ray(a, fa, zof(a));
+        const Ray ra = ray(a, fa);
         const float tb = fminf(fmaxf(one ? ray_exit(w, ra, ab) : ray_enter(w, ra, ab), 0.f), 1.f);
         const float tc = fminf(fmaxf(one ? ray_exit(w, ra, ac) : ray_enter(w, ra, ac), 0.f), 1.f);
-        const float2 p = make_float2(fmaf(tb, ab.x, a.x), fmaf(tb, ab.y, a.y));
-        const float2 q = make_float2(fmaf(tc, ac.x, a.x), fmaf(tc, ac.y, a.y));
-        O = one ? a : c;
-        E = sub(p, O);
-        dE = sub(q, p);
-        // areas against the triangle's: (A, p, q) tb tc, (C, p, q) tb (1 - tc), (p, B, C) 1 - tb
-        coef = one ? tb * tc : tb * (1.f - tc);
-        l = one ? tb : 0.25f;
-        dl = one ? tc - tb : 0.f;
-        if (!one) rest = 0.5f * (1.f - tb) * quad6(p, sub(b, p), sub(c, p), g);
-    }
-    const bool fan = seen != 0;
-    float sum = 0.f;
+        O = make_float2(fmaf(tb, ab.x, a.x), fmaf(tb, ab.y, a.y));
+        dO = make_float2(fmaf(tc, ac.x, a.x) - O.x, fmaf(tc, ac.y, a.y) - O.y);
+        // (tc, tb) in barycentric coordinates, across the chord (-tb, tc); away from A, or towards it
+        const float out = one ? 1.f : -1.f;
+        E = make_float2(out * fmaf(tc, ab.x, tb * ac.x), out * fmaf(tc, ab.y, tb * ac.y));
+        coef = fmaf(tb, tb, tc * tc);
+        const float base = one ? 0.f : 1.f;
+        const float2 u0 = one ? a : b, du = one ? make_float2(0.f, 0.f) : sub(c, b);
 #pragma unroll 1
-    for (int i = 0; i < 6; ++i) {
-        const float x = kGx6[i];
-        const float2 o = make_float2(fmaf(x, dO.x, O.x), fmaf(x, dO.y, O.y));
-        const float2 e = make_float2(fmaf(x, dE.x, E.x), fmaf(x, dE.y, E.y));
-        const float z = zof(o), f = fmaxf(phi_of(w, o, z), 0.f);
-        float t = ray_exit(w, ray(o, f, z), e);
-        t = t >= 0.f ? fminf(t, fminf(4.f, __fdividef(1.f, fmaf(x, dl, l)))) : 0.f;  // (0 / 0: a point ray)
+        for (int i = 0; i < 4; ++i) {
+            const float x = kGx4[i];
+            const float2 u = make_float2(fmaf(x, du.x, u0.x), fmaf(x, du.y, u0.y));
+            const float2 e = make_float2(fmaf(x, dO.x, O.x) - u.x, fmaf(x, dO.y, O.y) - u.y);
+            float s0 = 0.f, s1 = 0.f;
+#pragma unroll
+            for (int k = 0; k < 5; ++k) {
+                const float v = g(fmaf(kGx5[k], e.x, u.x), fmaf(kGx5[k], e.y, u.y));
+                s0 = fmaf(kGw5[k], v, s0);
+                s1 = fmaf(kGw5[k] * kGx5[k], v, s1);
+            }
+            // the map's Jacobian (barycentric) goes from j0 at the base to j1 at the chord
+            const float yb = (1.f - x) * (base - tb), yc = x * (base - tc);
+            const float j0 = base * (yb + yc), j1 = fmaf(tc, yb, tb * yc);
+            poly = fmaf(kGw4[i], fmaf(j1 - j0, s1, j0 * s0), poly);
+        }
+        poly = fabsf(poly);
+        if (coef < 1e-12f) return poly;  // (the cap is less than 1e-6 of the corner that A cuts off, which underflows)
+    }
+    // (w_z m~_z)^2 - (w_xy . m)^2 = ch x (1 - x) on the chord, ch x (1 - x) - 2 qb t - qa t^2 at t along its rays
+    const float wd = fmaf(w.wx, E.x, w.wy * E.y), wc = fmaf(w.wx, dO.x, w.wy * dO.y), wz2 = w.wz * w.wz;
+    const float qa = fmaf(wd, wd, wz2 * len2(E)), ch = fmaf(wc, wc, wz2 * len2(dO));
+    auto slope = [&](float2 m) { return fmaf(fmaf(w.wx, m.x, w.wy * m.y), wd, wz2 * fmaf(m.x, E.x, m.y * E.y)); };
+    const float q0 = slope(O), q1 = slope(make_float2(O.x + dO.x, O.y + dO.y));
+    if (!(fminf(q0, q1) >= 0.5f * fmaxf(q0, q1) && q0 > 0.f)) return -1.f;
+    float cap = 0.f;
+#pragma unroll 1
+    for (int i = 0; i < 5; ++i) {
+        const float x = kGx5[i], f = ch * (x * (1.f - x)), qb = fmaf(x, q1 - q0, q0);
+        const float t = __fdividef(f, qb + sqrtf(fmaf(qb, qb, qa * f)));
+        const float ox = fmaf(x, dO.x, O.x), oy = fmaf(x, dO.y, O.y);
         float in = 0.f;
 #pragma unroll
-        for (int k = 0; k < 5; ++k)
-            in = fmaf(kGw5[k] * (fan ? kGx5[k] : 1.f), g(fmaf(kGx5[k] * t, e.x, o.x), fmaf(kGx5[k] * t, e.y, o.y)), in);
-        sum = fmaf(kGw6[i] * (fan ? t * t : t), in, sum);
+        for (int k = 0; k < 2; ++k) in += g(fmaf(kGx2[k] * t, E.x, ox), fmaf(kGx2[k] * t, E.y, oy));
+        cap = fmaf(kGw5[i] * t, in, cap);
     }
-    return fmaf(coef, sum, rest);
+    return fmaf(0.5f * coef, cap, poly);
 }
 
 }  // namespace pndf
