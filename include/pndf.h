@@ -104,7 +104,11 @@ typedef enum pndf_eval_mode {
 
 typedef enum pndf_sort_mode {
     PNDF_SORT_NONE = 0,         /* caller order                                       */
-    PNDF_SORT_LEVEL_TILE = 1,   /* entry level (largest first), then centre tile (default) */
+    PNDF_SORT_LEVEL_TILE = 1,   /* entry level (largest first), then centre tile          */
+                                /* (default); caller order for batches of up to four     */
+                                /* queries per resident warp (96 per SM at the default   */
+                                /* launch shape) whose large footprints are divided, for */
+                                /* which the sort's launches cost more than it saves     */
     PNDF_SORT_LEVEL_NORMAL = 2, /* entry level, then query-normal bin                    */
     PNDF_SORT_LEVEL_TILE_NORMAL = 3, /* entry level, centre tile, then normal bin          */
     PNDF_SORT_LEVEL_NORMAL_TILE = 4  /* entry level, normal bin, then centre tile          */
@@ -126,7 +130,8 @@ typedef enum pndf_kernel {
 
 typedef struct pndf_eval_config {
     int32_t mode;           /* pndf_eval_mode                                         */
-    int32_t sort;           /* query order before traversal (pndf_sort_mode)          */
+    int32_t sort;           /* query order before traversal (pndf_sort_mode); never    */
+                            /* changes a result                                        */
     int32_t warps_per_cta;  /* 0 = library default                                   */
     int32_t ctas_per_sm;    /* 0 = as many as fit                                    */
     float tau;              /* cluster cut (Sec. 4.2): a node whose residual e <=      */

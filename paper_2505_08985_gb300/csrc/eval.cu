@@ -78,6 +78,7 @@ constexpr int kKeyBins = 1 << (4 + kMaxSubBits);  // largest histogram (2^18 bin
 // 5-10% longer on the flake map and 5 CTAs 24%
 #define PNDF_TRAVERSE_MIN_CTAS 3
 #endif
+constexpr int kTraverseWarps = 8 * PNDF_TRAVERSE_MIN_CTAS;  // resident per SM at the default launch shape
 constexpr unsigned kFull = 0xffffffffu;
 
 // MurmurHash3 32-bit finalizer (Appleby), fingerprints hit sets in stats mode.
@@ -1859,13 +1860,17 @@ pndf_status launch_eval(const pndf_hierarchy *h, const pndf_query *q, int64_t nq
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    // A batch of up to four queries per resident warp (24 per SM) gains nothing
-    // from the order when its large footprints are divided: no warp holds more
-    // than a few queries, and neighbours do not stay in flight together (4,096
-    // footprints on 16384^2 and 20,011 on 8192^2: 5.10 and 5.09 ms in arrival
-    // order, 5.12 and 5.14 ms sorted; 131,072: 24.6 and 19.8 ms).  The sort's
-    // four launches would then be most of a small call.
-    const bool sort = cfg.sort != 0 && !(split && nq <= int64_t(4) * 24 * sms);
+    // The default order is left out for a batch of up to four queries per resident
+    // warp whose large footprints are divided: it gains nothing there (no warp holds
+    // more than a few queries, and neighbours do not stay in flight together; 4,096
+    // footprints on 16384^2 and 20,011 on 8192^2: 5.10 and 5.09 ms in arrival order,
+    // 5.12 and 5.14 ms sorted; 131,072: 24.6 and 19.8 ms), and the sort's four
+    // launches would be most of a small call.  Another order was asked for: it is made.
+    const int warps = cfg.warps_per_cta > 0 ? cfg.warps_per_cta : 8;
+    const int resident = cfg.ctas_per_sm > 0 && warps * int64_t(cfg.ctas_per_sm) < kTraverseWarps
+                             ? warps * cfg.ctas_per_sm : kTraverseWarps;
+    const bool sort = cfg.sort != PNDF_SORT_NONE &&
+                      !(cfg.sort == PNDF_SORT_DEFAULT && split && nq <= int64_t(4) * resident * sms);
     const uint32_t cap = uint32_t(2 * 64 * (sms > 0 ? sms : 1) + 64);  // >= 2 x resident warps
     // scratch: cursor, split counter and work sum (padded to 256), key
     // histogram, keys, order, split markers and entries
