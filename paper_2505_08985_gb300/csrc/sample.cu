@@ -12,14 +12,17 @@
 //   Gaussian cut at q = 16: |v|^2 = -2 ln(1 - U1 (1 - e^-8)), angle 2 pi U2;
 //   disk (q <= 1.5^2): |v| = 1.5 sqrt(U1), angle 2 pi U2;
 //   box (|v|_inf <= 1.5): v = 1.5 (2 U1 - 1, 2 U2 - 1).
-// One thread per sample.  The position has to be good to about 1e-12 of the
-// footprint, so that the triangle chosen for u agrees with a 64-bit reference
-// except at ties; in FP64 that bound the kernel (86% of the FP64 pipe, 395 us per
-// million samples).  It runs in pairs of FP32 numbers (pair.cuh) instead, the
-// centre's integer part kept apart so that only the offset within the footprint
-// is rounded: 41 us per million samples, bound by FP32 issue (about 450
-// instructions) and the four texel loads.  Records outside the range where that is as good as FP64
-// (extreme covariances or centres) take the FP64 form (sample_fp64).
+// One thread per sample.  The position has to be as good as FP64 makes it, so that
+// the triangle chosen for u agrees with a 64-bit reference except at ties; in FP64
+// that bound the kernel (86% of the FP64 pipe, 395 us per million samples).  It runs
+// in pairs of FP32 numbers (pair.cuh) instead, the centre's integer part kept apart
+// so that only the offset within the footprint is rounded: 41 us, bound by FP32 issue and the four
+// texel loads.  Largest error of the offset in sigma, pairs and FP64: Gaussian
+// 3.7e-13 and 5.9e-13 (both where U1 is next to 0 and the logarithm's argument next
+// to 1), disk 2.5e-14 and 7e-16, box 3.5e-14 and 6e-16, where FP64 rounds the centre
+// too, to 1e-13 of a texel on a 2048^2 map and 1e-12 on a 16384^2 one.  Records
+// outside the range where the pairs serve (extreme covariances or centres) take the
+// FP64 form (sample_fp64).
 #include <math.h>
 
 #include "common.cuh"
@@ -114,7 +117,7 @@ __device__ __noinline__ Sampled sample_fp64(const MapDesc &d, const pndf_query &
     return o;
 }
 
-// 1 / (1 + i / 128 ...): log table over the mantissa's top 7 bits i.  c is near
+// Logarithm table over the mantissa's top 7 bits i.  c is near
 // the reciprocal of the interval's middle (halved from i = 53 on, so that the
 // reduced argument lies in [0.707, 1.414)) with 8 significant bits, so that m c -
 // 1 is exact; -log c as a pair.  c = 1 at both ends, next to the argument 1.
@@ -249,11 +252,14 @@ __device__ const float4 kLog[128] = {
     {1.0f, 0.0f, 0.0f, 0.f},
 };
 
-// Natural logarithm of a > 0 (a.h in [2^-20, 1]): a.h = 2^k m, log = k ln 2 - log c
-// + log1p(m c - 1), the last by its series (|m c - 1| <= 2^-7).
-__device__ __forceinline__ Pair log_pair(Pair a)
+// Natural logarithm of a + e + l, a in [2^-20, 1], |e| <= 2^-25 and 0 below a = 1/2,
+// |l| <= 2^-23 a: a = 2^k m, log = k ln 2 - log c + log1p(m c - 1), the last by its
+// series (|m c - 1| <= 2^-7), as in the table-driven logarithm of Tang, "Table-driven
+// implementation of the logarithm function in IEEE floating-point arithmetic", 1990.
+// e is added exactly: next to 1 the logarithm is no larger than it.
+__device__ __forceinline__ Pair log_sum(float a, float e, float l)
 {
-    const uint32_t bits = __float_as_uint(a.h), i = (bits >> 16) & 127u;
+    const uint32_t bits = __float_as_uint(a), i = (bits >> 16) & 127u;
     int k = int(bits >> 23) - 127;
     float m = __uint_as_float((bits & 0x7fffffu) | 0x3f800000u);
     if (i >= 53u) {
@@ -265,20 +271,22 @@ __device__ __forceinline__ Pair log_pair(Pair a)
     const Pair r2 = two_prod(r, r);
     const float q = r2.h * r * fmaf(r, fmaf(r, fmaf(r, fmaf(r, 1.0f / 7.0f, -1.0f / 6.0f), 0.2f), -0.25f), 1.0f / 3.0f);
     const Pair p = two_prod(float(k), 0.693147182f);
-    const Pair s0 = two_sum(p.h, t.y), s1 = two_sum(s0.h, r), s2 = two_sum(s1.h, -0.5f * r2.h);
+    const Pair s0 = two_sum(p.h, t.y), s1 = two_sum(s0.h, r), s2 = two_sum(s1.h, -0.5f * r2.h), s3 = two_sum(s2.h, e);
     float lo = fmaf(float(k), -1.90465421e-09f, p.l) + t.z;
-    lo += s0.l + s1.l + s2.l - 0.5f * r2.l + q + a.l / a.h;
-    return quick_sum(s2.h, lo);
+    lo += s0.l + s1.l + s2.l + s3.l - 0.5f * r2.l + q + fmaf(-0.5f * e, e, fmaf(e, 1.0f - a, l) / a);
+    return quick_sum(s3.h, lo);
 }
 
 // sin and cos of 2 pi u for u in [0, 1]: an exact reduction to |f| <= 1/4 of the
-// half turn, Taylor series with the leading coefficients as pairs.
+// half turn, Taylor series with the leading coefficients as pairs (the sine's up to
+// z^4, z = f^2: it is multiplied by f alone).
 __device__ __forceinline__ void sincos_turn(float u, Pair &sn, Pair &cs)
 {
     const float t = 2.0f * u, q = rintf(2.0f * t), f = __fmaf_rn(-0.5f, q, t);
     const Pair z = two_prod(f, f);
-    Pair s = Pair{-0.599264503f, -2.67954618e-08f} +
-             z.h * fmaf(z.h, fmaf(z.h, 0.000466302806f, -0.00737043095f), 0.0821458866f);
+    const float t9 = z.h * fmaf(z.h, fmaf(z.h, -2.19153535e-05f, 0.000466302805f), -0.00737043098f);
+    const Pair s9 = quick_sum(0.0821458846f, t9 + 1.97806404e-09f);
+    Pair s = Pair{-0.599264503f, -2.67954618e-08f} + z * s9;
     s = Pair{2.55016398f, 5.55786386e-08f} + z * s;
     s = Pair{-5.16771269f, -9.16039227e-08f} + z * s;
     s = (Pair{3.14159274f, -8.74227766e-08f} + z * s) * f;
@@ -321,16 +329,17 @@ __device__ __forceinline__ float third_of_sum(float a, float b, float c, float a
 }
 
 // The sample in pairs; false where the record is outside their range: centres
-// past 2^20, variances outside [1e-8, 1e10], correlation so strong that S_yy -
-// l21^2 keeps less than 1e-3 of S_yy.  (Zero, negative and infinite inputs are
-// among those.)
+// past 2^20, variances outside [1e-8, 2^24] (sigma 4096, where the pairs' error comes
+// to 1.4e-10 of a texel with the disk and box kernels), correlation so strong that
+// S_yy - l21^2 keeps less than 1e-3 of S_yy.  (Zero, negative and infinite inputs
+// are among those.)
 template <int TFMT>
 __device__ __forceinline__ bool sample_pair(const MapDesc &d, const pndf_query &r, float u1, float u2, int kernel,
                                             float jac_eps, float rho, Sampled &o)
 {
     const float cc = r.sxx * r.syy;
-    if (!(fabsf(r.x) < 1048576.f && fabsf(r.y) < 1048576.f && r.sxx > 1e-8f && r.sxx < 1e10f && r.syy > 1e-8f &&
-          r.syy < 1e10f && fmaf(-r.sxy, r.sxy, cc) > 1e-3f * cc && u1 >= 0.f && u1 <= 1.f && u2 >= 0.f && u2 <= 1.f))
+    if (!(fabsf(r.x) < 1048576.f && fabsf(r.y) < 1048576.f && r.sxx > 1e-8f && r.sxx <= 0x1p24f && r.syy > 1e-8f &&
+          r.syy <= 0x1p24f && fmaf(-r.sxy, r.sxy, cc) > 1e-3f * cc && u1 >= 0.f && u1 <= 1.f && u2 >= 0.f && u2 <= 1.f))
         return false;
     Pair v1, v2;
     if (kernel == PNDF_KERNEL_BOX) {
@@ -341,8 +350,9 @@ __device__ __forceinline__ bool sample_pair(const MapDesc &d, const pndf_query &
         if (kernel == PNDF_KERNEL_DISK) {
             rad = root(Pair{u1, 0.f}) * 1.5f;
         } else {  // sqrt(-2 log(1 - u1 (1 - e^-8)))
-            const Pair a = -(Pair{0.999664545f, -7.68710695e-09f} * u1) + 1.0f;
-            const Pair g = log_pair(a);
+            // as (1 - u1) + u1 e^-8, which keeps its digits for u1 next to 0 and to 1
+            const Pair s = two_sum(1.0f, -u1), e8 = two_prod(u1, 3.3546262e-04f), a = two_sum(s.h, e8.h);
+            const Pair g = log_sum(a.h, s.l, a.l + fmaf(u1, 3.695373e-12f, e8.l));
             rad = root(Pair{-2.0f * g.h, -2.0f * g.l});
         }
         Pair sn, cs;
