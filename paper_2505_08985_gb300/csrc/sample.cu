@@ -331,8 +331,8 @@ __device__ __forceinline__ float third_of_sum(float a, float b, float c, float a
 // The sample in pairs; false where the record is outside their range: centres
 // past 2^20, variances outside [1e-8, 2^24] (sigma 4096, where the pairs' error comes
 // to 1.4e-10 of a texel with the disk and box kernels), correlation so strong that
-// S_yy - l21^2 keeps less than 1e-3 of S_yy.  (Zero, negative and infinite inputs
-// are among those.)
+// S_yy - l21^2 keeps less than 1e-3 of S_yy (zero, negative and infinite inputs are
+// among those), normals that are not finite.
 template <int TFMT>
 __device__ __forceinline__ bool sample_pair(const MapDesc &d, const pndf_query &r, float u1, float u2, int kernel,
                                             float jac_eps, float rho, Sampled &o)
@@ -398,7 +398,8 @@ __device__ __forceinline__ bool sample_pair(const MapDesc &d, const pndf_query &
         o.my = blend(l0, lb, lc, na.y, nb.y, nc.y);
     }
     o.tri = 2u * (uint32_t(j) * uint32_t(d.n - 1) + uint32_t(i)) + uint32_t(tri);
-    return true;
+    // (texels that are not finite or whose products are not: a pair's low part is lost with them)
+    return isfinite(o.mx) && isfinite(o.my);
 }
 
 template <int TFMT>
