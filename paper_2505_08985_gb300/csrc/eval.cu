@@ -510,7 +510,7 @@ __device__ __forceinline__ bool capsule_holds(float2 n0, float2 n1, float2 n2, f
 // (0: none) and what became of it.
 struct Tiny {
     float w;
-    int state;  // 0: no area, 1: evaluated, 2: out of reach (support or capsule)
+    int state;  // 0: no area, 1: evaluated, 2: out of reach (support or capsule), 3: evaluated in FP32
 };
 template <class Q>
 __device__ __forceinline__ Tiny tiny_triangle(const Q &q, float2 na, float2 nb, float2 nc, int ai, int aj, float dir)
@@ -535,12 +535,12 @@ __device__ __forceinline__ Tiny tiny_triangle(const Q &q, float2 na, float2 nb, 
 template <bool STATS>
 __device__ __forceinline__ void add_tiny(const Tiny &t, uint32_t id, Acc &acc)
 {
-    if (t.state != 1) {
+    if (t.state == 0 || t.state == 2) {
         if (STATS && t.state == 0) acc.degen++;
         return;
     }
-    if (STATS) acc.fp64++;
-    acc.flags |= PNDF_QF_FP64;
+    if (STATS) acc.fp64 += t.state == 1 ? 1u : 0u;
+    acc.flags |= t.state == 1 ? PNDF_QF_FP64 : 0u;
     if (t.w == 0.f) return;
     acc_add(acc, t.w);
     if (STATS) {
@@ -574,20 +574,36 @@ __device__ __forceinline__ bool edges_hold(const Q &q, float2 na, float2 nb, flo
     return cr > 0.f ? (e0 >= 0.f && e1 >= 0.f && e2 >= 0.f) : (e0 <= 0.f && e1 <= 0.f && e2 <= 0.f);
 }
 
-// Add the contribution of an FP32 hit: cross cr and edge functions e1, e2 (so
-// l1 = e1 / cr, l2 = e2 / cr) of triangle `tri` of the quad, or of the level-l
-// cluster, at (gi, gj); its uv legs are a = 2^l and the Jacobian cr / a^2.
-template <bool STATS, class Q>
-__device__ __forceinline__ void weigh(const Q &q, int gi, int gj, int l, int tri, float cr, float e1, float e2,
-                                      uint32_t id, Acc &acc)
+// Does an FP32 hit (cross cr, edge functions e1, e2) lie in its triangle?  Where the
+// cross is rounding noise (normals on a line) so is the hit's place in uv, and it
+// may lie in the support although the hit's node does not meet it, which node_meets
+// lets by.  Such a hit counts only if the node meets the support by the exact test.
+__device__ __forceinline__ bool in_place(float cr, float e1, float e2)
+{
+    return fabsf(e1 + e2) <= fabsf(cr) * (1.0f + 1e-6f);
+}
+
+// Kernel weight of an FP32 hit: cross cr and edge functions e1, e2 (so l1 = e1 / cr,
+// l2 = e2 / cr) of triangle `tri` of the quad, or of the level-l cluster, at (gi,
+// gj), whose uv legs are a = 2^l.
+template <class Q>
+__device__ __forceinline__ float kernel_at(const Q &q, int gi, int gj, int l, int tri, float cr, float e1, float e2)
 {
     const float a = float(1 << l);
     const float inv = 1.0f / cr;
     const float dir = tri ? -a : a;
     const float dx = (float(gi + (tri << l)) - q.x) + dir * (e1 * inv);
     const float dy = (float(gj + (tri << l)) - q.y) + dir * (e2 * inv);
-    const float qq = qform(q, dx, dy);
-    const float w = kweight(q, dx, qq);
+    return kweight(q, dx, qform(q, dx, dy));
+}
+
+// Add the contribution of such a hit; the Jacobian is cr / a^2.
+template <bool STATS, class Q>
+__device__ __forceinline__ void weigh(const Q &q, int gi, int gj, int l, int tri, float cr, float e1, float e2,
+                                      uint32_t id, Acc &acc)
+{
+    const float a = float(1 << l);
+    const float w = kernel_at(q, gi, gj, l, tri, cr, e1, e2);
     if (w == 0.f) return;
     acc_add(acc, w * (a * a) / fabsf(cr));
     if (STATS) {
@@ -689,16 +705,47 @@ struct LeafState {
     int ng, nt, nh, nc;
 };
 
-// tiny_triangle of triangle `tri` of quad (gi, gj) when its leaf block meets the
-// support (exactly: node_meets lets some by) and m is in the quad's capsule; out of line, so that the rare path costs the common one neither
-// registers nor instruction fetches.
+// Edge functions at m of the replacement of Eq. 6 for triangle (a, b, c): the
+// equilateral one (vertex k at 90 + 120 k degrees around the centroid g, radius
+// rho), in vertex-relative form p = m - E0.  True if it holds m.
+template <class Q>
+__device__ __forceinline__ bool replacement_holds(const Q &q, float2 na, float2 nb, float2 nc, float &ecr, float &e1,
+                                                  float &e2)
+{
+    const float gx = (na.x + nb.x + nc.x) * (1.0f / 3.0f), gy = (na.y + nb.y + nc.y) * (1.0f / 3.0f);
+    const float h = 0.8660254f * q.rho;  // E1 - E0 = rho (-sqrt3/2, -3/2), E2 - E0 = rho (sqrt3/2, -3/2)
+    const float2 b = make_float2(-h, -1.5f * q.rho), c = make_float2(h, -1.5f * q.rho);
+    const float2 p = make_float2(q.mx - gx, (q.my - gy) - q.rho);
+    ecr = diff_prod(b.x, c.y, b.y, c.x);  // > 0: counter-clockwise
+    const float e0 = diff_prod(c.x - b.x, p.y - b.y, c.y - b.y, p.x - b.x);
+    e1 = diff_prod(p.x, c.y, p.y, c.x);
+    e2 = diff_prod(b.x, p.y, b.y, p.x);
+    return e0 >= 0.f && e1 >= 0.f && e2 >= 0.f;
+}
+
+// Triangle `tri` of quad (gi, gj) when it is near-singular or its hit is out of
+// place: nothing unless its leaf block meets the support by the exact test, and,
+// near-singular, m is in the quad's capsule.  Out of line and called from one place,
+// so that the rare path costs the common one neither registers nor instruction
+// fetches (with a call of its own for the hits out of place the flake workload took
+// 8% longer, like this 0.1%).
 template <int BFMT, int TFMT, bool CLAMP, class Q>
-__device__ __noinline__ Tiny tiny_in_capsule(const MapDesc &d, const Q &q, int gi, int gj, int tri)
+__device__ __noinline__ Tiny rare_triangle(const MapDesc &d, const Q &q, int gi, int gj, int tri)
 {
     if (!node_in_footprint(q, kLeafLevel, uint32_t(gi) >> kLeafLevel, uint32_t(gj) >> kLeafLevel)) return Tiny{0.f, 2};
     const float2 n0 = texel<TFMT>(d, gi, gj), n1 = texel<TFMT>(d, gi + 1, gj);
     const float2 n2 = texel<TFMT>(d, gi, gj + 1), n3 = texel<TFMT>(d, gi + 1, gj + 1);
+    const float2 na = tri ? n3 : n0, nb = tri ? n2 : n1, nc = tri ? n1 : n2;
+    float cr = orient(na.x, na.y, nb.x, nb.y, nc.x, nc.y), e1, e2;
+    const bool clamp = CLAMP && fabsf(cr) < q.jac;
+    if (clamp || fabsf(cr) >= kTinyCross) {
+        const bool hit = clamp ? replacement_holds(q, na, nb, nc, cr, e1, e2) : edges_hold(q, na, nb, nc, cr, e1, e2);
+        const float w = hit ? kernel_at(q, gi, gj, 0, tri, cr, e1, e2) : 0.f;
+        return Tiny{w == 0.f ? 0.f : w / fabsf(cr), 3};
+    }
     if (!capsule_holds<BFMT>(n0, n1, n2, n3, q.mx, q.my, CLAMP ? q.rho : 0.f)) return Tiny{0.f, 2};
+    // (two copies: with one, the register allocator's choices in the caller took the
+    // flake workload 6% longer)
     return tri ? tiny_triangle(q, n3, n2, n1, gi + 1, gj + 1, -1.f) : tiny_triangle(q, n0, n1, n2, gi, gj, 1.f);
 }
 
@@ -718,25 +765,21 @@ __device__ __forceinline__ void test_tris(const MapDesc &d, const Q &q, const Le
     if (!tri_box_holds<CLAMP>(q, na, nb, nc)) return;
     const float cr = orient(na.x, na.y, nb.x, nb.y, nc.x, nc.y);
     if (CLAMP && fabsf(cr) < q.jac) {
-        // Eq. 6: the equilateral replacement (vertex k at 90 + 120 k degrees
-        // around the centroid g, radius rho), in vertex-relative form p = m - E0
-        const float gx = (na.x + nb.x + nc.x) * (1.0f / 3.0f), gy = (na.y + nb.y + nc.y) * (1.0f / 3.0f);
-        const float h = 0.8660254f * q.rho;  // E1 - E0 = rho (-sqrt3/2, -3/2), E2 - E0 = rho (sqrt3/2, -3/2)
-        const float2 b = make_float2(-h, -1.5f * q.rho), c = make_float2(h, -1.5f * q.rho);
-        const float2 p = make_float2(q.mx - gx, (q.my - gy) - q.rho);
-        const float ecr = diff_prod(b.x, c.y, b.y, c.x);  // > 0: counter-clockwise
-        const float e0 = diff_prod(c.x - b.x, p.y - b.y, c.y - b.y, p.x - b.x);
-        const float e1 = diff_prod(p.x, c.y, p.y, c.x);
-        const float e2 = diff_prod(b.x, p.y, b.y, p.x);
-        if (e0 >= 0.f && e1 >= 0.f && e2 >= 0.f) weigh<STATS>(q, gi, gj, 0, tri, ecr, e1, e2, id, acc);
-        return;
-    }
-    if (fabsf(cr) >= kTinyCross) {
+        float ecr, e1, e2;
+        if (!replacement_holds(q, na, nb, nc, ecr, e1, e2)) return;
+        if (in_place(ecr, e1, e2)) {
+            weigh<STATS>(q, gi, gj, 0, tri, ecr, e1, e2, id, acc);
+            return;
+        }
+    } else if (fabsf(cr) >= kTinyCross) {
         float e1, e2;
-        if (edges_hold(q, na, nb, nc, cr, e1, e2)) weigh<STATS>(q, gi, gj, 0, tri, cr, e1, e2, id, acc);
-        return;
+        if (!edges_hold(q, na, nb, nc, cr, e1, e2)) return;
+        if (in_place(cr, e1, e2)) {
+            weigh<STATS>(q, gi, gj, 0, tri, cr, e1, e2, id, acc);
+            return;
+        }
     }
-    add_tiny<STATS>(tiny_in_capsule<BFMT, TFMT, CLAMP>(d, q, gi, gj, tri), id, acc);
+    add_tiny<STATS>(rare_triangle<BFMT, TFMT, CLAMP>(d, q, gi, gj, tri), id, acc);
 }
 
 // The 3 x 3 texels of group (i, j) (i, j even), rows j..j + 2; past the map's
@@ -903,6 +946,13 @@ __device__ __forceinline__ bool cluster_edge_test(const Q &q, float2 p, float2 b
     return false;
 }
 
+// Node (l, a, c) meets the support by the exact test, out of line for a rare caller.
+template <class Q>
+__device__ __noinline__ bool meets_exactly(const Q &q, int l, uint32_t a, uint32_t c)
+{
+    return node_in_footprint(q, l, a, c);
+}
+
 // All 32 lanes: lane k < cnt weighs hit k of the hit ring.
 template <bool STATS, class Q>
 __device__ __forceinline__ void weigh_clusters(const MapDesc &d, const Q &q, const LeafState &ls, int cnt, int lane,
@@ -914,6 +964,7 @@ __device__ __forceinline__ void weigh_clusters(const MapDesc &d, const Q &q, con
     const int tri = int(__float_as_uint(h.w) & 1u), l = node_level(k, d.L);
     const uint32_t m = k - node_index(d.L, l, 0);
     const uint32_t I = compact1by1(m), J = compact1by1(m >> 1);
+    if (!in_place(h.x, h.y, h.z) && !meets_exactly(q, l, I, J)) return;
     const uint32_t id = kClusterTag | (uint32_t(l) << 27) | (((J << (d.L - l)) + I) << 1) | uint32_t(tri);
     weigh<STATS>(q, int(I << l), int(J << l), l, tri, h.x, h.y, h.z, id, acc);
 }
