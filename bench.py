@@ -1224,7 +1224,52 @@ def run_gpu(args, world, rank, local):
         line["cpu_baseline"] = {"value": rate, "unit": UNIT, "cores": oracle.default_threads(), "kind": "oracle",
                                 "sample": f"{n_done} random queries of the same workload, {secs:.1f} s wall"}
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        print(json.dumps({"details": line}), file=sys.stderr, flush=True)
+        print(json.dumps(summary_line(line)), flush=True)
+
+
+LINE_LIMIT = 6000  # characters; whoever reads the last lines of a log gets the whole line
+
+
+def rounded(v):
+    """Floats to six significant digits."""
+    if isinstance(v, float):
+        return float(f"{v:.6g}")
+    if isinstance(v, dict):
+        return {k: rounded(x) for k, x in v.items()}
+    return [rounded(x) for x in v] if isinstance(v, list) else v
+
+
+def summary_line(line: dict) -> dict:
+    """The line on stdout: every key of the measurement itself in full, and of the
+    other workloads' reports (which go to stderr whole) the headline figures."""
+    out = {k: v for k, v in line.items() if k not in ("accuracy_vs_fp64_oracle", "cluster_cut", "footprint_kernels",
+                                                      "jacobian_clamp_and_sampling", "glint_diffuse_16384", "serving",
+                                                      "kernel_rooflines", "traversal_flops", "work_per_launch")}
+    if "accuracy_vs_fp64_oracle" in line:
+        out["rel_err_max_vs_fp64_oracle"] = {
+            k: max(r["rel_err_max"] for r in v["results"].values()) if "results" in v else v.get("rel_err_max")
+            for k, v in line["accuracy_vs_fp64_oracle"].items()}
+    if "serving" in line:
+        out["serving"] = {
+            k: {"capacity_queries_per_s": v["capacity_queries_per_s"],
+                "loads": [{"load": x["load"], **{arm: {"p50_ms": r["p50_ms"], "p99_ms": r["p99_ms"]}
+                                                 for arm, r in x.items() if isinstance(r, dict)}} for x in v["loads"]]}
+            for k, v in line["serving"].items() if isinstance(v, dict)}
+    if "glint_diffuse_16384" in line:
+        out["glint_diffuse_16384"] = {k: {x: y for x, y in v.items() if not isinstance(y, (dict, list, str))}
+                                      for k, v in line["glint_diffuse_16384"].items()
+                                      if k in ("projected_area", "pndf", "served_stream")}
+    if "kernel_rooflines" in line:
+        out["kernel_rooflines"] = {k: {"ms": v["ms"], "bound": v["bound"], "frac": v["frac"]}
+                                   for k, v in line["kernel_rooflines"]["families"].items()}
+    out = rounded(out)
+    for k in ("value", "ms_per_step", "e2e"):
+        out[k] = line[k]
+    for drop in ("glint_diffuse_16384", "serving", "kernel_rooflines"):  # (not with the default workloads)
+        if len(json.dumps(out)) > LINE_LIMIT:
+            out.pop(drop, None)
+    return out
 
 
 # ---------------------------------------------------------------------------
