@@ -336,7 +336,8 @@ def traversal_roofline(dev, work_f16: dict, nq: int, kernel_ms: float, world: in
     FP32) + the query's 32 B record and 4 B result.  Instruction issue, on the
     warp instructions per query of the committed ncu capture of the same
     kernel source (152 SMs x 4 schedulers x the maximum SM clock).  `bound` is
-    the ceiling with the larger fraction; the other is kept beside it, and so
+    the ceiling with the larger fraction (HBM's by the capture's DRAM bytes, where
+    there is one of this source); the other is kept beside it, and so
     is the builder's own byte model (every node, group record and texel that a
     test reads, 40 B per query), which counts a texel once per test that reads
     it."""
@@ -353,10 +354,15 @@ def traversal_roofline(dev, work_f16: dict, nq: int, kernel_ms: float, world: in
         ach = wipq * nq / sec / 1e9
         issue = {"achieved": ach, "peak": peaks["issue"], "unit": "G warp-instructions/s", "frac": ach / peaks["issue"],
                  "warp_instructions_per_query": wipq, "peak_source": f"{peaks['sms']} SMs x 4 x {peaks['sm_mhz']:.0f} MHz"}
-    bound = "alu" if issue and issue["frac"] > hbm["frac"] else "hbm"
+    # where the DRAM traffic of this source was measured, that decides, not the model,
+    # which counts bytes that the slabs and group records keep the kernel from reading
+    traffic = committed_traffic("f16")
+    if traffic is not None:
+        hbm["measured_frac"] = traffic * (nq / synth.FLAKE_8192["queries"]) / sec / 1e9 / pk
+    bound = "alu" if issue and issue["frac"] > hbm.get("measured_frac", hbm["frac"]) else "hbm"
     top = issue if bound == "alu" else hbm
     out = {"bound": bound, "achieved": top["achieved"], "peak": top["peak"], "unit": top["unit"], "frac": top["frac"],
-           "traffic": committed_traffic("f16"), "hbm": hbm, "issue": issue,
+           "traffic": traffic, "hbm": hbm, "issue": issue,
            "ncu_pct_of_peak": committed_ncu_pct("f16"),
            "builder_byte_model": {"bytes_per_launch": work_f16["bytes"],
                                   "achieved_gbs": work_f16["bytes"] / sec / 1e9,

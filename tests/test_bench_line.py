@@ -1,5 +1,6 @@
 """bench.py's line on stdout (CPU only): the measurement's own keys whole, the other
-workloads' headline figures, and short enough to be read back from a log's end."""
+workloads' headline figures, and short enough to be read back from a log's end;
+the traversal's bound by the DRAM bytes measured on its source."""
 import json
 import os
 import sys
@@ -61,3 +62,17 @@ def test_line_is_short_and_keeps_the_measurement(bench, extra):
 def test_a_line_of_the_measurement_alone(bench):
     line = {k: v for k, v in full_line(bench).items() if k in ("metric", "value", "ms_per_step", "e2e", "config")}
     assert bench.summary_line(line) == line
+
+
+def test_measured_traffic_decides_the_bound(bench, monkeypatch):
+    monkeypatch.setattr(bench, "compute_peaks", lambda dev: {"issue": 1258.56, "fp32": 80.0, "fp64": 1.25, "sms": 152, "sm_mhz": 2070.0})
+    monkeypatch.setattr(bench, "hbm_peak", lambda: (6000.0, "measured"))
+    monkeypatch.setattr(bench, "committed_ncu_pct", lambda tag: None)
+    monkeypatch.setattr(bench, "committed_profile_value", lambda key: 6e4)
+    nq = bench.synth.FLAKE_8192["queries"]
+    w = {"nodes": 10000 * nq, "leaf_blocks": 1200 * nq, "bytes": 1, "quads": 1, "tri_tests": 1, "hits": 1}
+    monkeypatch.setattr(bench, "committed_traffic", lambda tag: 1.0e12)
+    r = bench.traversal_roofline(None, w, nq=nq, kernel_ms=330.0, world=1)
+    assert r["hbm"]["frac"] > r["issue"]["frac"] > r["hbm"]["measured_frac"]
+    assert r["bound"] == "alu" and r["frac"] == r["issue"]["frac"]
+    assert abs(r["hbm"]["measured_frac"] - 1.0e12 / 0.33 / 1e9 / 6000.0) < 1e-12
