@@ -58,8 +58,9 @@ typedef enum pndf_texel_fmt {
 } pndf_texel_fmt;
 
 typedef enum pndf_bounds_fmt {
-    PNDF_BOUNDS_F32 = 0,           /* exact float32 min/max per node (16 B)         */
-    PNDF_BOUNDS_F16_OUTWARD = 1    /* binary16 min rounded down, max rounded up (8 B) */
+    PNDF_BOUNDS_F32 = 0,           /* exact float32 min/max per node (24 B with its slab) */
+    PNDF_BOUNDS_F16_OUTWARD = 1    /* binary16 min rounded down, max rounded up (16 B     */
+                                   /* with its slab)                                      */
 } pndf_bounds_fmt;
 
 typedef struct pndf_build_params {
@@ -86,7 +87,8 @@ typedef struct pndf_query_stats {
     uint32_t hits;         /* contributing hits (m inside, q <= 16)                  */
     uint32_t hit_hash;     /* sum mod 2^32 of MurmurHash3-fmix32(triangle id) over hits */
     uint32_t fp64_tris;    /* triangles evaluated in FP64 (normal area < 1e-10)      */
-    uint32_t degenerate;   /* zero-area normal triangles met inside their bbox       */
+    uint32_t degenerate;   /* zero-area normal triangles, m in their bbox, among those */
+                           /* tested one by one (most are pruned before)               */
     uint32_t quads;        /* quads whose edge functions were tested, in 2 x 2 groups */
     uint32_t cluster_checks; /* nodes whose cluster residual was compared with the cut */
     uint32_t clusters;     /* cluster nodes whose two triangles were tested          */
@@ -285,7 +287,10 @@ pndf_status pndf_cluster_level(const pndf_hierarchy *h, int32_t level, float *re
  * bounding box); zero-area normal triangles are skipped (a delta, not a
  * density); triangles of normal-space area below 1e-10 are tested and
  * weighted in FP64, all others in FP32.  The pyramid only prunes, so the set
- * of contributing triangles equals that of the flat mode.  Each query's sum
+ * of contributing triangles equals that of the flat mode, but for triangles so
+ * thin that their FP32 cross is rounding noise (normals along a line): their
+ * hits' places in uv are noise too, and may lie in the support although their
+ * leaf block does not meet it; the flat mode counts those.  Each query's sum
  * is exact: every contribution is rounded once to a multiple of 2^-64 and
  * added in 128-bit fixed point, and the total is rounded to FP32 once, so D
  * does not depend on the order of the hits, on the batch, the launch shape or
@@ -484,8 +489,8 @@ typedef struct pndf_server_config {
  * requests (segment kind PNDF_SEGMENT_PROJECTED_AREA), evaluated in the same
  * step graph by the kernels of pndf_diffuse_projected_area (so P is the same
  * bit for bit as that call gives); each table slot reserves their band
- * scratch, 4 (max + 1) + 8 max B bytes with B = (N_max + 6) / 8 + 1 bands for
- * the largest map side N_max.
+ * scratch, 4 (max + 1) + 8 max B bytes with B = (N_max + 2) / 4 + 1 bands (of
+ * four quad rows) for the largest map side N_max.
  * Errors: INVALID_ARG (formats differ, bad counts, kernel / tau / jac_eps out
  * of range), UNSUPPORTED (tau with a map built without clusters, or with the
  * disk / box kernel or the clamp; the clamp with the disk / box kernel), OOM,

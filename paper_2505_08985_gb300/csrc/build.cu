@@ -5,7 +5,8 @@
 // so each normal triangle below it lies inside the box.  Levels
 // kLeafLevel..L are stored; level l is a (2^(L-l))^2 array in Morton order,
 // so the four children of node k at level l are nodes 4k..4k+3 at level l-1
-// (one 64-byte line in FP32, one 32-byte sector in FP16).
+// (64 contiguous bytes in either bound format: with FP16 bounds a node's box and
+// slab are one 16-byte record, with FP32 bounds the slabs are a second array).
 //
 // Beside the boxes, the nodes of levels 2..kSlabTop carry a slab (see
 // common.cuh), and level 1 holds one 16-byte record per 2 x 2 quads, a
@@ -16,8 +17,9 @@
 // texels are staged in shared memory with 16-byte vector loads (float4 = two
 // FP32 texels, uint4 = four FP16 texels) and stored unchanged into the
 // hierarchy's own copy of the map (each texel by exactly one tile, so the map
-// is read once per build); each thread builds one leaf node's 16 quad boxes
-// and their union, and levels up to 6 are reduced in shared memory.  A tile
+// is read once per build); each thread builds one leaf node from its 5 x 5
+// texels, its four groups' records and their union, warps build the slabs up to
+// kSlabTop by shuffles, and levels up to 6 are reduced in shared memory.  A tile
 // is a Morton-aligned square at every level, so its nodes form one contiguous
 // run and the writes are fully coalesced.
 // Kernel 2 (build_up): one launch per level above the tile, four contiguous
@@ -33,9 +35,7 @@ namespace {
 constexpr int kTileQuadsMax = 64;
 constexpr int kTileTexMax = kTileQuadsMax + 1;
 constexpr int kBuildThreads = 256;
-#ifndef PNDF_BUILD_CTAS
-#define PNDF_BUILD_CTAS 3  // 80 registers; at two (91) an 8192^2 build takes 0.25 ms longer
-#endif
+constexpr int kBuildCtas = 3;  // per SM, 80 registers; at two (91) an 8192^2 build takes 0.25 ms longer
 
 // Second moments of a set of normals about a reference point.
 struct Moments {
@@ -135,7 +135,7 @@ __device__ __forceinline__ float2 copy_texel(const void *src, void *dst, size_t 
 // VEC = texels per 16-byte load (2 for FP32, 4 for FP16), or 1 when rows are
 // not 16-byte aligned (n not a multiple of VEC).
 template <int TFMT, int BFMT, int VEC>
-__global__ void __launch_bounds__(kBuildThreads, PNDF_BUILD_CTAS) build_tiles(const void *__restrict__ src, MapDesc d, int tileQ,
+__global__ void __launch_bounds__(kBuildThreads, kBuildCtas) build_tiles(const void *__restrict__ src, MapDesc d, int tileQ,
                                                             int lq)
 {
     __shared__ float2 tex[kTileTexMax * kTileTexMax];

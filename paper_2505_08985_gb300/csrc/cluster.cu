@@ -41,9 +41,6 @@ namespace pndf {
 namespace {
 
 constexpr double kJacEps = 1e-6;
-#ifndef PNDF_CL_CTAS
-#define PNDF_CL_CTAS 2
-#endif
 
 // A node's quadratic form at its optimum: Gram matrix G (symmetric, upper
 // triangle packed: 00 01 02 03 11 12 13 22 23 33), optimal corners g
@@ -65,8 +62,10 @@ __host__ __device__ constexpr double hat(int a, double s, double t)
                         : (a == 0 ? 0.0 : a == 1 ? 1.0 - t : a == 2 ? 1.0 - s : s + t - 1.0);
 }
 
-// 1 / x for x > 0: the FP32 reciprocal (relative error below 2^-22) and one
-// cubic step, three FP64 operations where a division takes about twelve.
+// 1 / x for x > 0: the FP32 reciprocal (relative error e below 2^-22) and one
+// third-order Newton step, r (1 + e + e^2): what is left is e^3 < 2^-66 and the
+// rounding of the last operations, an ulp.  Three FP64 operations, where a division
+// takes about twelve.
 __host__ __device__ __forceinline__ double inv_pos(double x)
 {
 #ifdef __CUDA_ARCH__
@@ -468,11 +467,11 @@ __device__ __forceinline__ bool node_inside_map(const MapDesc &d, int l, uint32_
 constexpr int kTileLevels = 4;                        // levels 3..6 above the leaf level in one CTA
 constexpr int kTileThreads = 1 << (2 * kTileLevels);  // 256 leaf blocks
 
-// Two CTAs per SM (128 registers, the rest spilled): 32.1 ms against 38.3 ms
-// at one (255 registers) for the 8192^2 cluster hierarchy; the FP64 pipe
-// needs the second CTA's warps to stay busy.
+// Two CTAs per SM (128 registers): 5.9 ms against 7.1 ms at one for the 4096^2
+// cluster hierarchy; the FP64 pipe needs the second CTA's warps to stay busy.
+constexpr int kTileCtas = 2;
 template <int TFMT, int BFMT>
-__global__ void __launch_bounds__(kTileThreads, PNDF_CL_CTAS) cluster_tiles(MapDesc d, ClusterDesc cd, QF *__restrict__ out6)
+__global__ void __launch_bounds__(kTileThreads, kTileCtas) cluster_tiles(MapDesc d, ClusterDesc cd, QF *__restrict__ out6)
 {
     extern __shared__ double wt_s[];  // [32][kTileThreads]
     __shared__ QF part[16];

@@ -73,12 +73,10 @@ constexpr int kPop = 24;           // nodes popped per step at most (four childr
 constexpr int kStackCap = 36 * kPop + 4 * kPop + 16 + 16;
 constexpr int kMaxSubBits = 14;                   // sub-key bits below the 4 entry-level bits
 constexpr int kKeyBins = 1 << (4 + kMaxSubBits);  // largest histogram (2^18 bins)
-#ifndef PNDF_TRAVERSE_MIN_CTAS
 // 3 x 256 threads per SM at 80 registers: 4 CTAs (64 registers, spills) took
 // 5-10% longer on the flake map and 5 CTAs 24%
-#define PNDF_TRAVERSE_MIN_CTAS 3
-#endif
-constexpr int kTraverseWarps = 8 * PNDF_TRAVERSE_MIN_CTAS;  // resident per SM at the default launch shape
+constexpr int kTraverseCtas = 3;
+constexpr int kTraverseWarps = 8 * kTraverseCtas;  // resident per SM at the default launch shape
 constexpr unsigned kFull = 0xffffffffu;
 
 // MurmurHash3 32-bit finalizer (Appleby), fingerprints hit sets in stats mode.
@@ -1574,7 +1572,7 @@ __device__ __forceinline__ void tile_finish(const MapDesc &d, SplitEntry &E, con
 }
 
 template <int BFMT, int TFMT, bool STATS, bool FLAT, bool CLUSTER, int KERN>
-__global__ void __launch_bounds__(256, PNDF_TRAVERSE_MIN_CTAS)
+__global__ void __launch_bounds__(256, kTraverseCtas)
     traverse_kernel(MapDesc d, ClusterDesc cd, float tau, float jac_eps, const pndf_query *__restrict__ qs,
                     const uint32_t *__restrict__ order, int64_t nq, float *__restrict__ D,
                     uint32_t *__restrict__ flags, pndf_query_stats *__restrict__ stats,
@@ -2073,7 +2071,7 @@ __global__ void serve_split_plan(const MapDesc *__restrict__ maps, const uint32_
 }
 
 template <int BFMT, int TFMT, bool CLUSTER, int KERN>
-__global__ void __launch_bounds__(256, PNDF_TRAVERSE_MIN_CTAS)
+__global__ void __launch_bounds__(256, kTraverseCtas)
     serve_kernel(const MapDesc *__restrict__ maps, const ClusterDesc *__restrict__ clusters, int nmaps,
                  const uint32_t *__restrict__ table, const pndf_segment *__restrict__ segs,
                  unsigned long long *__restrict__ cursor, float tau, float jac_eps, SplitPlan sp)

@@ -40,17 +40,13 @@ __device__ unsigned int g_status_projarea;
 namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
-#ifndef PNDF_GGX_CTAS
-#define PNDF_GGX_CTAS 4  // of 3, 4, 5, 6 and 8 within 8% of each other
-#endif
-#ifndef PNDF_PA_CTAS
-#define PNDF_PA_CTAS 4
-#endif
+constexpr int kGgxCtas = 4;   // per SM, of 3, 4, 5, 6 and 8 within 8% of each other
+constexpr int kAreaCtas = 4;  // see pa_items
 // A band is long enough to pay for its row setup and its rings' last, partly
-// filled evaluations, and short enough to spread a few footprints over the SMs:
-// 8 / 4 / 2 rows, 192 requests on 16384^2 14.6 / 13.0 / 12.4 ms, 64 on 4096^2 1.06 /
-// 0.63 / 0.47 ms, 1000 small ones 0.33 / 0.32 / 0.32 ms; the partial sums (and a
-// server's scratch) double with each halving.
+// filled evaluations, and short enough to spread a few footprints over the SMs: 8
+// / 4 / 2 rows, the same 192 requests on 16384^2 14.3 / 13.0 / 12.2 ms, 64 on 4096^2
+// 0.99 / 0.64 / 0.49 ms, 1000 small ones 0.31 ms each.  Two rows are faster or
+// equal, but the partial sums (and a server's scratch) double with each halving.
 constexpr int kBand = 4;                 // quad rows per work item
 
 // V_T / |cross| in closed form (visible.cuh, FP64), for the largest triangles;
@@ -397,7 +393,7 @@ __device__ __forceinline__ float2 integrate_band(const MapDesc &d, const Req &q,
 // larger triangles instead of taking them in FP64: 1000 small footprints on a
 // scratch map, whose grooves have many, 0.49 -> 0.34 ms.
 template <int TFMT>
-__global__ void __launch_bounds__(256, PNDF_PA_CTAS) pa_items(MapDesc d, const pndf_query *__restrict__ qs,
+__global__ void __launch_bounds__(256, kAreaCtas) pa_items(MapDesc d, const pndf_query *__restrict__ qs,
                                                const float *__restrict__ omega, int64_t k0, int cnt,
                                                const uint32_t *__restrict__ off, float2 *__restrict__ part,
                                                unsigned int *__restrict__ cursor)
@@ -493,7 +489,7 @@ __global__ void __launch_bounds__(1024) area_step_prep(const MapDesc *__restrict
 }
 
 template <int TFMT>
-__global__ void __launch_bounds__(256, PNDF_PA_CTAS) area_step_items(const MapDesc *__restrict__ maps, int nmaps,
+__global__ void __launch_bounds__(256, kAreaCtas) area_step_items(const MapDesc *__restrict__ maps, int nmaps,
                                                       const uint32_t *__restrict__ count,
                                                       const AreaReq *__restrict__ areq,
                                                       const uint32_t *__restrict__ off, float2 *__restrict__ part,
@@ -615,7 +611,7 @@ constexpr int kGgxLeafWarps = 8;
 static_assert(kGgxDirs == 16, "two lanes per direction in the sums, four bits in a listed pair");
 
 template <int TFMT>
-__global__ void __launch_bounds__(32 * kGgxLeafWarps, PNDF_GGX_CTAS) ggx_leaf(MapDesc d, GgxDirs dirs,
+__global__ void __launch_bounds__(32 * kGgxLeafWarps, kGgxCtas) ggx_leaf(MapDesc d, GgxDirs dirs,
                                                                float *__restrict__ P, float4 *__restrict__ omega,
                                                                uint32_t nleaf)
 {
@@ -940,7 +936,7 @@ pndf_status launch_projarea(const pndf_hierarchy *h, const pndf_query *q, const 
 {
     if (nq == 0) return PNDF_OK;
     const MapDesc &d = h->d;
-    const int maxbands = (d.n - 1 + kBand - 1) / kBand + 1;
+    const int maxbands = area_max_bands(d.n);
     // requests per chunk: bounded by the scan (65536) and by 256 MiB of band partials
     int64_t chunk = (int64_t(1) << 28) / (int64_t(sizeof(float2)) * maxbands);
     if (chunk > 65536) chunk = 65536;
