@@ -36,11 +36,11 @@
 //               the support's bounding box.
 //
 // What bounds it: the descent is instruction issue and L2 latency in about equal
-// parts (half of all issue slots used, 6 of 12 cycles between a warp's issues
+// parts (55% of the issue slots used, 4.7 of 11 cycles between a warp's issues
 // spent on loads; the same footprints on maps from 2048^2 to 16384^2 take 18 to
 // 23 ms, so DRAM is not the limit).  Per query of the 8192^2 flake workload it
-// tests 10.5k nodes, 1.2k leaf blocks, 1.4k groups and 972 triangles for 964
-// hits, in 62k warp instructions; with a box and a capsule per quad in place of
+// tests 10.7k nodes, 1.2k leaf blocks, 1.4k groups and 998 triangles for 990
+// hits, in 59.7k warp instructions; with a box and a capsule per quad in place of
 // the slabs and groups it took 187k, and 897 ms per 4M queries against 329 ms.
 //
 // Hit test (tie rule): m inside the closed normal bounding box and all three

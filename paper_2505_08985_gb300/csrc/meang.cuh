@@ -11,8 +11,9 @@
 // 12 points (degree 6) 5e-9 at 0.5, 8e-8 at 0.8.  Rules: Dunavant, "High degree
 // efficient symmetrical Gaussian quadrature rules for the triangle", 1985.
 //
-// A triangle the boundary w . m~ = 0 crosses is cut along it into straight and
-// curved pieces, each again a positive smooth integral (partial_mean).  Larger
+// A triangle the boundary w . m~ = 0 crosses is cut along it into a polygon and the
+// cap that bows out of it, each again a positive smooth integral (partial_mean);
+// the few whose cap is cut off or too oblique take the closed form.  Larger
 // triangles are split in four at their edges' midpoints; what is still too
 // large goes to the closed form in FP64 (visible.cuh).
 #pragma once

@@ -14,7 +14,7 @@
 //    points for small triangles, 12 for those that straddle normal regions;
 //  * no vertex sees w and none of the triangle can: exactly 0 (Alg. 1 drops
 //    every edge);
-//  * otherwise cut along the visibility boundary into smooth pieces
+//  * otherwise the polygon and the cap that the visibility boundary cuts off it
 //    (partial_mean);
 //  * larger triangles are split in four, each part classified again; a part that
 //    is still too large takes the closed form of visible.cuh in FP64 (the clip
@@ -385,10 +385,11 @@ __device__ __forceinline__ float2 integrate_band(const MapDesc &d, const Req &q,
     return make_float2(s, c);
 }
 
-// What bounds it: FP32 issue (about 250 instructions per triangle: the six
-// quadrature points 80, classification and weights 80, row walk and sums 50, the
-// deferred classes 40).  Four CTAs per SM (64 registers): 192 requests on the
-// 16384^2 mixed map 13.5 ms, at three 14.3, at five and six 13.7, at eight 15.8;
+// What bounds it: FP32 issue (86% of the slots; about 340 instructions a triangle,
+// a quarter of them the six quadrature points, the rest classification, weights,
+// row walk, sums and the deferred classes).  Four CTAs per SM (64 registers): the same 192
+// requests on the 16384^2 mixed map 13.5 ms, at three 14.3, at five and six 13.7, at
+// eight 15.8;
 // with the FP64 path for every partly visible triangle it was 79 ms.  Splitting the
 // larger triangles instead of taking them in FP64: 1000 small footprints on a
 // scratch map, whose grooves have many, 0.49 -> 0.34 ms.
@@ -604,7 +605,7 @@ __device__ __forceinline__ void leaf_triangle(const MapDesc &d, int i0, int j0, 
 // from that; the (triangle, direction) pairs that the visibility boundary
 // crosses are listed and spread over the warp 32 at a time, and so are the few
 // to be split.  The sums over the triangles run in a fixed order.  The
-// whole fit of a 2048^2 mixed map takes 1.1 ms (17.2 ms with a closed-form integral
+// whole fit of a 2048^2 mixed map takes 1.0 ms (17.2 ms with a closed-form integral
 // per direction, FP64 for every partly visible pair and the 3 x 3 solve in FP64 by
 // one lane), and Omega's error against 64 bits fell from 6e-6 to 6e-7.
 constexpr int kGgxLeafWarps = 8;
